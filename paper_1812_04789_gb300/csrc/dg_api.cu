@@ -121,8 +121,7 @@ cudaError_t MG<T>::smooth(int l, const T* b, T* x, int nu, cudaStream_t st) {
     if (l >= 1 && L.coop.ok && !ilu && (L.Dinv16 || (L.inv_t && L.co_t))) {
       if (nu == 0) return cudaSuccess;
       return launch_coop_smoother(L.coop, L.Dinv, L.Dop, L.O, L.Dinv16, L.Dop16, L.O16, mesh->face_nbr(),
-                                  mesh->nfaces(), b, x, nu, K, L.cpart, L.cbar, mesh->status, coop_extra, L.nb,
-                                  mesh->E, st);
+                                  mesh->nfaces(), b, x, nu, K, L.cbuf, mesh->status, coop_extra, L.nb, mesh->E, st);
     }
   }
   CKE(op(l, x, L.r, st));
@@ -265,9 +264,12 @@ static dg_status alloc_mg(dg_pmg h, MG<T>& mg) {
       CK(plan_coop_smoother(bf16 ? 1 : 0, L.nb, M.nfaces(), M.E, nmax, &L.coop));
       if (L.coop.ok) {
         L.coop.nu_max = nmax;
-        CK(dalloc(mg.allocs, (void**)&L.cpart, sizeof(double) * (size_t)(L.coop.grid + 1) * (2 * (nmax + 1) + 1),
-                  &h->vector_bytes));
-        CK(dalloc(mg.allocs, (void**)&L.cbar, sizeof(unsigned) * COOP_BAR_WORDS, &h->vector_bytes));
+        CK(dalloc(mg.allocs, &L.cbuf.part, L.coop.part_bytes, &h->vector_bytes));
+        CK(dalloc(mg.allocs, &L.cbuf.z, L.coop.z_bytes, &h->vector_bytes));
+        CK(dalloc(mg.allocs, (void**)&L.cbuf.epoch, sizeof(unsigned), &h->vector_bytes));
+        CK(cudaMemset(L.cbuf.part, 0, L.coop.part_bytes));
+        CK(cudaMemset(L.cbuf.z, 0, L.coop.z_bytes));
+        CK(cudaMemset(L.cbuf.epoch, 0, sizeof(unsigned)));
       }
     }
   }

@@ -282,25 +282,32 @@ struct Krylov {
 // ----------------------------------------------------------------- pMG
 // Launch plan of the persistent coarse-level smoother (csrc/dg_smoother.cu):
 // grid CTAs (all co-resident, cooperative launch), chunk elements per CTA,
-// epc elements per pass of the block-sparse product, tpe threads per block,
-// dynamic shared memory for up to nu_max iterations.  ok = 0: not available.
+// epc elements per pass of the block-sparse product, tpe threads per block, ns
+// threads over an element's blocks, pre: blocks prefetched into L2, res: the CTA's blocks in shared memory,
+// dynamic shared memory for up to nu_max iterations, bytes of the exchange
+// buffers.  ok = 0: not available.
 struct CoopPlan {
-  int ok = 0, grid = 0, chunk = 0, epc = 0, tpe = 0, nu_max = 0;
-  size_t smem = 0;
+  int ok = 0, grid = 0, chunk = 0, epc = 0, tpe = 0, ns = 1, pre = 0, res = 0, nu_max = 0;
+  size_t smem = 0, part_bytes = 0, z_bytes = 0;
 };
 cudaError_t plan_coop_smoother(int bf16, int nb, int nf, int E, int nu, CoopPlan* plan);
-constexpr int COOP_BAR_WORDS = 64;   // barrier words per level (arrivals at 0, release at 32)
-// One SMOOTH call (nu GMRES(BJ) iterations from x on A x = b, Algorithm 2) in
-// one cooperative launch: FP32 vectors, blocks column-major in FP32 (inv_ld)
-// or, when Dinv16 is given, BF16 (ld_bf16).  part: grid * (2 (nu_max + 1) + 1)
-// doubles; bar: COOP_BAR_WORDS words (zeroed by the call, on the stream); a bounded
-// grid barrier that runs out sets ST_TIMEOUT in *status.  expect_extra > 0
-// makes every barrier wait for CTAs that do not exist (the wait then runs out).
+// Exchange buffers of a level (zero when allocated): the CTAs' partial sums,
+// the published directions and the epoch word.  Launches that share them are
+// ordered on one stream.
+struct CoopBuffers {
+  void* part = nullptr;
+  void* z = nullptr;
+  unsigned* epoch = nullptr;
+};
+// One SMOOTH call (nu >= 1 GMRES(BJ) iterations from x on A x = b, Algorithm 2)
+// in one cooperative launch: FP32 vectors, blocks column-major in FP32 (inv_ld)
+// or, when Dinv16 is given, BF16 (ld_bf16).  A bounded wait that runs out sets
+// ST_TIMEOUT in *status.  extra > 0 makes every exchange wait for a CTA that
+// does not exist (the wait then runs out).
 cudaError_t launch_coop_smoother(const CoopPlan& pl, const float* Dinv, const float* Dop, const float* O,
                                  const unsigned short* Dinv16, const unsigned short* Dop16, const unsigned short* O16,
                                  const int* nbr, int nf, const float* b, float* x, int nu, Krylov<float>& K,
-                                 double* part, unsigned* bar, int* status, int expect_extra, int nb, int E,
-                                 cudaStream_t st);
+                                 const CoopBuffers& buf, int* status, int extra, int nb, int E, cudaStream_t st);
 
 template <class T>
 struct Level {
@@ -322,8 +329,7 @@ struct Level {
   unsigned short* Dop16 = nullptr;
   unsigned short* O16 = nullptr;
   CoopPlan coop;             // persistent smoother (FP32 coarse levels), when available
-  double* cpart = nullptr;   //   its reduction partials [grid][2 (nu + 1) + 1], then the totals
-  unsigned* cbar = nullptr;  //   and barrier counter
+  CoopBuffers cbuf;          //   and its exchange buffers
 };
 
 template <class T>

@@ -7,39 +7,51 @@
 // One CTA per SM owns a contiguous range of elements for the whole call and
 // keeps its rows of the Krylov basis V, of the preconditioned directions Z and
 // of the work vector w in shared memory (the coarse levels are small: a level
-// whose rows do not fit keeps the launch-per-operation smoother).  Only z_j
-// goes to device memory, where the neighbours' products read it.  Per
-// iteration j:
-//   A  v_j = w / ||w||; z_j = D^{-1} v_j (own elements)                 | grid barrier
-//   B  w = A z_j (own elements, neighbours' z_j read); partial V^T w    | grid barrier
-//   C  h1 = sum of partials; w -= V h1; partial V^T w and ||w||^2       | grid barrier
-//   D  h2 = sum of partials; w -= V h2; ||w - V h2||^2 = ||w||^2 - ||h2||^2
-// (CGS2, as the launch-per-operation Arnoldi; the norm after the second pass
-// by Pythagoras, as in the low-synchronisation Gram-Schmidt variants of
-// Swirydowicz et al. 2021, which saves a barrier: h2 is at rounding level
-// against w, so the difference loses nothing.  Where it would cancel, more
-// than 99 % of ||w||^2, the norm is summed explicitly behind a fourth
-// barrier; every CTA takes the same branch.)  A barrier that ends a
-// reduction also sums it: the last CTA to arrive adds the CTAs' partials in a
-// fixed order (FP64) and publishes the sums before it releases the others,
-// which then read only the sums.  Every CTA keeps its own copy of the
-// Hessenberg matrix, the Givens rotations and g, so all CTAs hold identical
-// scalars and the final x += Z y needs no further barrier.  The arithmetic
-// inside a CTA is FP32 (products and their sums over the CTA's rows, w -= V h
-// with h rounded to FP32, the Givens rotations and the small least-squares
-// solve, x += Z y): GB300 runs FP64 and FP32<->FP64 conversions at a small
-// fraction of its FP32 rate, with long latencies, and FP64 there made the
-// smoother FP64-bound; only the sums across CTAs are FP64.
+// whose rows do not fit keeps the launch-per-operation smoother), and, where
+// they fit as well (p = 0), its blocks.
 //
-// The grid barrier counts arrivals in one word and releases the waiting CTAs
-// through another (its own 128-byte line, so the polls do not contend with
-// the arrivals); both are zeroed before the launch.  Every wait is bounded
-// (2 s of the global timer): on expiry the CTA sets ST_TIMEOUT in the mesh
-// status word and returns, and the other CTAs see the flag while they wait
-// and return too; a launch that finds ST_TIMEOUT already set returns at once.
-// A handle whose status shows ST_TIMEOUT has an unfinished smoother result:
-// the application is untrusted until the status is cleared (dg_status_sync)
-// and the preconditioner refreshed.
+// The coarse levels are bound by the exchanges between the CTAs, not by
+// arithmetic: with three grid barriers per iteration (an arrival counter, the
+// last CTA summing the partials, a release word) an iteration took 23 us at
+// p = 0 on 16^3 elements, of which the barriers were 14.  Two things bring
+// that down.
+//  * One reduction per iteration instead of two: Gram-Schmidt twice with the
+//    second pass delayed (the low-synchronisation CGS2 of Swirydowicz et al.
+//    2021 and Bielich et al. 2022).  Exchange j carries, beside V^T w for the
+//    new column, V^T v_j for the second pass over v_j itself, v_j.v_j and w.w:
+//      s = V^T v_j, beta^2 = v_j.v_j - s.s, v_j <- (v_j - V s) / beta,
+//      h_i = V_i.w (i < j), h_j = (v_j.w - s.V^T w) / beta,
+//      v_{j+1} = rho^{-1} (w - V h),  rho^2 = w.w - h.h (an estimate; a scale only)
+//    and column j - 1 of the Hessenberg matrix, whose last vector was still
+//    v_j's first pass, is completed: H_{i,j-1} += rho s_i, H_{j,j-1} = rho beta.
+//    The directions z_j = D^{-1} v_j are those of the first pass: the outer
+//    form is flexible (A Z = V H holds for any Z), so they need no second pass.
+//  * No barriers: every value that another CTA needs travels with its epoch in
+//    the same 8 (z_j) or 2 x 8 bytes (the partial sums), and the reader polls
+//    the value itself.  The partial sums take two such hops (to the CTA that
+//    owns the sum and back), the directions one, in place of arrival, sum,
+//    release and read.  Epochs only grow (a word in device memory holds the next one), so
+//    nothing is cleared between calls.  z_j's buffer is reused every
+//    iteration (exchange j ends only after every CTA has consumed z_j), the
+//    partials' buffer every second one.
+// Per iteration j:
+//   w = A z_j (own rows; the neighbours' z_j polled), partials        | exchange
+//   second pass for v_j, v_{j+1}, z_{j+1} = D^{-1} v_{j+1} published
+// The sums over the CTAs are in two-float arithmetic (the exact error of every
+// addition carried along, 48 bits) and in a fixed order, rounded to FP32 at the
+// end; all CTAs hold identical scalars and the final x += Z y needs no
+// exchange.  FP64 sums cost more than a hop (GB300 has two FP64 lanes per SM).  The arithmetic inside a CTA is FP32.  A warp of its own
+// keeps the Hessenberg matrix, the Givens rotations and the small
+// least-squares solve off the critical path.
+// 16^3 elements, p_fine = 4 (us per call): p = 2, nu = 10: 880 -> 765;
+// p = 1, nu = 10: 400 -> 188; p = 0, nu = 30: 690 -> 290.
+//
+// Every wait is bounded (2 s of the global timer): on expiry the CTA sets
+// ST_TIMEOUT in the mesh status word and returns, and the other CTAs see the
+// flag while they wait and return too; a launch that finds ST_TIMEOUT already
+// set returns at once.  A handle whose status shows ST_TIMEOUT has an
+// unfinished smoother result: the application is untrusted until the status
+// is cleared (dg_status_sync) and the preconditioner refreshed.
 #include <math.h>
 
 #include <algorithm>
@@ -48,22 +60,45 @@
 
 namespace dgk {
 
-// R consecutive rows of one column of a column-major block from 16 bytes.
+// R consecutive rows of one column of a column-major block from 16 bytes, from
+// device memory (streamed) or, RES, from shared memory.
 template <class S>
 struct Col16;
 template <>
 struct Col16<float> {
   static constexpr int R = 4;
+  template <bool RES>
   __device__ __forceinline__ static void load(const float* p, float* v) {
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
-                 : "l"(p));
+    if constexpr (RES) {
+      const float4 t = *reinterpret_cast<const float4*>(p);
+      v[0] = t.x;
+      v[1] = t.y;
+      v[2] = t.z;
+      v[3] = t.w;
+    } else {
+      asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+                   : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                   : "l"(p));
+    }
   }
 };
 template <>
 struct Col16<unsigned short> {
   static constexpr int R = 8;
-  __device__ __forceinline__ static void load(const unsigned short* p, float* v) { ld_bf16x8(p, v); }
+  template <bool RES>
+  __device__ __forceinline__ static void load(const unsigned short* p, float* v) {
+    if constexpr (RES) {
+      const uint4 t = *reinterpret_cast<const uint4*>(p);
+      const unsigned w[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[2 * k] = __uint_as_float(w[k] << 16);
+        v[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+      }
+    } else {
+      ld_bf16x8(p, v);
+    }
+  }
 };
 
 template <class S>
@@ -74,439 +109,517 @@ struct CoopArgs {
   const int* nbr;       // [E][nf]
   const float* b;
   float* x;
-  float* Z;             // nu x N: the directions z_j, read by the neighbours' products
-  double* part;         // [grid][2 (nu + 1) + 1] partials, then one row of sums
-  unsigned* bar;        // [0]: arrivals, [32]: released barrier number; zero at launch
+  unsigned long long* zx;   // [N] (value, epoch) of the direction z_j
+  uint4* px;            // [2][ni][grid + 1] (s, epoch, t, epoch): the CTAs' partial sums
+  uint4* sums;          // [2][ni] their sums over the CTAs
+  unsigned* epoch;      // first free epoch - 1
   int* status;          // mesh status word (ST_TIMEOUT)
   int* kflag;           // Krylov status bits (ST_NONFINITE)
-  long N;
-  int nu, nb, ld, nf, E, chunk, epc, tpe, expect;
+  int nu, nb, ld, E, chunk, epc, tpe, ns, ni, extra;
+  int pre;              // ask for the blocks ahead of their use (a level that L2 holds)
 };
 
-constexpr int COOP_THREADS = 512;
+constexpr int COOP_WORK = 512;                  // threads that compute
+constexpr int COOP_THREADS = COOP_WORK + 32;    // and the scalar warp
 
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-
-// Grid-wide barrier number k (k * expect arrivals); false when a wait ran out
-// here or elsewhere (ST_TIMEOUT), and then the caller returns.
-__device__ bool grid_barrier(unsigned* bar, unsigned k, unsigned expect, int* status, int* sflag) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    __threadfence();
-    const unsigned old = atomicAdd(bar, 1u);
-    if (old + 1u == k * expect) {
-      __threadfence();
-      atomicExch(bar + 32, k);            // the last arrival releases barrier k
-    } else {
-      const unsigned long long t0 = global_ns();
-      while (*(volatile unsigned*)(bar + 32) < k) {
-        if (*(volatile int*)status & ST_TIMEOUT) {
-          ok = 0;
-          break;
-        }
-        if (global_ns() - t0 > 2000000000ull) {
-          atomicOr(status, ST_TIMEOUT);
-          ok = 0;
-          break;
-        }
-        __nanosleep(20);
-      }
-    }
-    __threadfence();
-    *sflag = ok;
-  }
-  __syncthreads();
-  return *sflag != 0;
+__device__ __forceinline__ unsigned long long ld_val(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_val(unsigned long long* p, float f, unsigned ep) {
+  const unsigned long long v = ((unsigned long long)ep << 32) | __float_as_uint(f);
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ uint4 ld_pair(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_pair(uint4* p, float s, float t, unsigned ep) {
+  asm volatile("st.volatile.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(__float_as_uint(s)), "r"(ep),
+               "r"(__float_as_uint(t)), "r"(ep)
+               : "memory");
 }
 
-// Grid barrier number k that also sums the CTAs' partials: the last CTA to
-// arrive adds part[c * stride + off + i] over c = 0..G-1 for i < nv (16 lanes
-// per value, each lane its c = lane, lane + 16, .. loaded at once and summed as
-// a tree, then a butterfly: the same order whichever CTA is last) into tot[i], then releases the
-// others; every CTA copies tot[0, nv) into dst (shared memory).  One CTA reads
-// the G x nv partials instead of every CTA.  False when a wait ran out here or
-// elsewhere (ST_TIMEOUT), and then the caller returns.
-__device__ bool grid_barrier_sum(unsigned* bar, unsigned k, unsigned expect, int* status, int* sflag,
-                                 const double* part, int stride, int off, int nv, int G, double* tot,
-                                 double* dst) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned old = atomicAdd(bar, 1u);
-    __threadfence();
-    sflag[2] = old + 1u == k * expect ? 1 : 0;
+// A bounded wait: expired() is called once per failed poll and looks at the
+// clock and the status word every 64th time.
+struct Wait {
+  unsigned n = 0;
+  unsigned long long t0 = 0;
+  __device__ __forceinline__ bool expired(int* status) {
+    if ((++n & 63u) != 0) return false;
+    if (*(volatile int*)status & ST_TIMEOUT) return true;
+    const unsigned long long t = global_ns();
+    if (t0 == 0) t0 = t;
+    if (t - t0 > 2000000000ull) {
+      atomicOr(status, ST_TIMEOUT);
+      return true;
+    }
+    return false;
   }
-  __syncthreads();
-  if (sflag[2]) {
-    const int grp = threadIdx.x >> 4, l16 = threadIdx.x & 15, ngrp = blockDim.x >> 4;
-    for (int i0 = 0; i0 < nv; i0 += ngrp) {
-      const int i = i0 + grp;   // uniform per 16-lane group
-      // every load of a lane issued at once (12 per lane: G <= 192 in one
-      // round trip), summed as a tree
-      double t[12];
-#pragma unroll
-      for (int u = 0; u < 12; ++u) {
-        const int c = l16 + 16 * u;
-        t[u] = (i < nv && c < G) ? __ldcg(part + (size_t)c * stride + off + i) : 0.0;
-      }
-      double s = (((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]))) +
-                 ((t[8] + t[9]) + (t[10] + t[11]));
-      for (int c = l16 + 192; i < nv && c < G; c += 16) s += __ldcg(part + (size_t)c * stride + off + i);
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (i < nv && l16 == 0) tot[i] = s;
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      atomicExch(bar + 32, k);            // release barrier k
-      sflag[0] = 1;
-    }
-  } else if (threadIdx.x == 0) {
-    int ok = 1;
-    const unsigned long long t0 = global_ns();
-    while (*(volatile unsigned*)(bar + 32) < k) {
-      if (*(volatile int*)status & ST_TIMEOUT) {
-        ok = 0;
-        break;
-      }
-      if (global_ns() - t0 > 2000000000ull) {
-        atomicOr(status, ST_TIMEOUT);
-        ok = 0;
-        break;
-      }
-      __nanosleep(20);
-    }
-    __threadfence();
-    sflag[0] = ok;
-  }
-  __syncthreads();
-  if (!sflag[0]) return false;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) dst[i] = __ldcg(tot + i);
-  __syncthreads();
-  return true;
+};
+
+// Start bringing `bytes` (a multiple of 16, 16-byte aligned) into L2.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// FP32 sum over the CTA's threads of f (warp butterflies, then warp 0 over
-// the warp sums), valid in every thread; redf: 33 floats, [32] the result
-__device__ float block_sum_f(float f, float* redf) {
+// (h, l) += x with the rounding error of the addition kept in l
+__device__ __forceinline__ void two_add(float& h, float& l, float x) {
+  const float s = h + x, b = s - h;
+  l += (h - (s - b)) + (x - b);
+  h = s;
+}
+
+// The CTA's partial sums of exchange j, a warp per item: (V_i.v_j, V_i.w) for
+// i <= j and (w.w, 0), in FP32 (a lane's rows, then the warp's butterfly),
+// published as they are ready; w = null (the closing exchange): zeros for w.
+__device__ void publish_dots(int j, const float* Vs, int ldv, const float* w, int rows, uint4* out, int stride,
+                             unsigned ep) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp >= COOP_WORK / 32) return;
+  const float* vj = Vs + (size_t)j * ldv;
+  for (int i = warp; i < j + 2; i += COOP_WORK / 32) {
+    const float* v = i <= j ? Vs + (size_t)i * ldv : w;
+    float fs = 0.f, ft = 0.f;
+    if (v) {
+      for (int r = lane; r < rows; r += 32) {
+        const float x = v[r];
+        if (i <= j) {
+          fs = fmaf(x, vj[r], fs);
+          if (w) ft = fmaf(x, w[r], ft);
+        } else {
+          fs = fmaf(x, x, fs);
+        }
+      }
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();   // earlier readers of redf are done
-  if (lane == 0) redf[warp] = f;
-  __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+      fs += __shfl_xor_sync(0xffffffffu, fs, o);
+      ft += __shfl_xor_sync(0xffffffffu, ft, o);
+    }
+    if (lane == 0) st_pair(out + (size_t)i * stride, fs, ft, ep);
+  }
+}
+
+// st[i] = the sums over all CTAs of the items i < ni of an exchange: CTA i mod G
+// owns item i, a warp of it polls the G partials in[i stride + c] (5 loads of a
+// lane at once), adds them in two-float arithmetic, a lane's CTAs and then the
+// lanes by a butterfly, and publishes the sum, and one warp of every CTA
+// polls the ni sums.  Two hops of little traffic: one hop, with every CTA
+// reading all G x ni partials, saturated the L2 with polls and took 8 us.
+// False where a wait ran out.
+__device__ bool gather_dots(const uint4* in, int stride, int ni, int G, uint4* sums, unsigned ep, int* status,
+                            float2* st) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, C = gridDim.x;
+  bool ok = true;
+  if (warp >= COOP_WORK / 32) return ok;
+  Wait wt;
+  // (the owned items i = blockIdx.x + k C, shared out over the warps; warp 0 collects)
+  for (int i = blockIdx.x + (warp - 1) * C; warp > 0 && i < ni; i += (COOP_WORK / 32 - 1) * C) {
+    float hs = 0.f, ls = 0.f, ht = 0.f, lt = 0.f;
+    for (int c0 = lane; c0 < G; c0 += 160) {
+      uint4 q[5];
+#pragma unroll
+      for (int u = 0; u < 5; ++u) q[u] = ld_pair(in + (size_t)i * stride + min(c0 + 32 * u, G - 1));
+#pragma unroll
+      for (int u = 0; u < 5; ++u) {
+        if (c0 + 32 * u >= G) continue;
+        while (ok && (q[u].y != ep || q[u].w != ep)) {
+          if (wt.expired(status)) ok = false;
+          q[u] = ld_pair(in + (size_t)i * stride + c0 + 32 * u);
+        }
+        two_add(hs, ls, __uint_as_float(q[u].x));
+        two_add(ht, lt, __uint_as_float(q[u].z));
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float a = __shfl_xor_sync(0xffffffffu, hs, o), b = __shfl_xor_sync(0xffffffffu, ls, o);
+      const float c = __shfl_xor_sync(0xffffffffu, ht, o), d = __shfl_xor_sync(0xffffffffu, lt, o);
+      two_add(hs, ls, a);
+      ls += b;
+      two_add(ht, lt, c);
+      lt += d;
+    }
+    if (__all_sync(0xffffffffu, ok) && lane == 0) st_pair(sums + i, hs + ls, ht + lt, ep);
+  }
   if (warp == 0) {
-    float t = lane < nw ? redf[lane] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) redf[32] = t;
-  }
-  __syncthreads();
-  return redf[32];
-}
-
-// out[i] = sum over the CTA's rows of V_i . w (shared memory), i < nv, warp per
-// i, in FP32 (a lane's rows, then the warp's butterfly); the CTA partials are
-// then summed across CTAs in FP64
-__device__ void own_dots(int nv, const float* Vs, int ldv, const float* ws, int rows, double* out) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int i = warp; i < nv; i += nw) {
-    const float* v = Vs + (size_t)i * ldv;
-    float f0 = 0.f, f1 = 0.f;
-    int r = lane;
-    for (; r + 32 < rows; r += 64) {
-      f0 = fmaf(v[r], ws[r], f0);
-      f1 = fmaf(v[r + 32], ws[r + 32], f1);
+    for (int i = lane; i < ni; i += 32) {
+      uint4 q = ld_pair(sums + i);
+      while (ok && (q.y != ep || q.w != ep)) {
+        if (wt.expired(status)) ok = false;
+        q = ld_pair(sums + i);
+      }
+      st[i] = make_float2(__uint_as_float(q.x), __uint_as_float(q.z));
     }
-    if (r < rows) f0 = fmaf(v[r], ws[r], f0);
-    float f = f0 + f1;
+  }
+  return ok;
+}
+
+// The inputs of the block-sparse product for the CTA's elements p0 .. p0 + nl:
+// xs[el][who][nb], who = 0 the element itself, 1 + s its neighbour on face s.
+// own = null: from the vector in (no epochs); else own rows from `own`
+// (shared memory) and the others' from zx, polled for epoch ep.
+__device__ bool stage_inputs(const int* src, int nsrc, int p0, int nl, int nb, float inv_nb, int e_beg, int ne,
+                             const float* in, const float* own, const unsigned long long* zx, unsigned ep,
+                             int* status, float* xs) {
+  bool ok = true;
+  if (threadIdx.x >= COOP_WORK) return ok;
+  Wait wt;
+  const int n = nl * nsrc * nb;
+  for (int t0 = threadIdx.x; t0 < n; t0 += 4 * COOP_WORK) {
+    unsigned long long v[4];
+    const unsigned long long* ad[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if (lane == 0) out[i] = (double)f;
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + u * COOP_WORK;
+      ad[u] = nullptr;
+      if (t >= n) continue;
+      const int pair = (int)(((float)t + 0.5f) * inv_nb), j = t - pair * nb;   // exact: t < 2^20
+      const int e = src[p0 * nsrc + pair];
+      if (!own) {
+        xs[t] = __ldcg(in + (size_t)e * nb + j);
+      } else if ((unsigned)(e - e_beg) < (unsigned)ne) {
+        xs[t] = own[(e - e_beg) * nb + j];
+      } else {
+        ad[u] = zx + (size_t)e * nb + j;
+        v[u] = ld_val(ad[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (!ad[u]) continue;
+      while (ok && (unsigned)(v[u] >> 32) != ep) {
+        if (wt.expired(status)) ok = false;
+        v[u] = ld_val(ad[u]);
+      }
+      xs[t0 + u * COOP_WORK] = __uint_as_float((unsigned)v[u]);
+    }
+  }
+  return ok;
+}
+
+// acc[R] += rows of one column-major block times x, a run of columns' loads in
+// flight together.  The last, shorter run reads the last column again (times
+// zero): with a test around each load, or a loop over the remaining columns,
+// every load waits for the one before it.
+template <class S, bool RES>
+__device__ __forceinline__ void col_run(const S* B, int nb, int ld, const float* x, float* acc) {
+  constexpr int R = Col16<S>::R, U = 48 / R;
+  for (int c0 = 0; c0 < nb; c0 += U) {
+    float v[U][R], xv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int c = min(c0 + u, nb - 1);
+      Col16<S>::template load<RES>(B + (size_t)c * ld, v[u]);
+      xv[u] = c0 + u < nb ? x[c] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[j] = fmaf(v[u][j], xv[u], acc[j]);
   }
 }
 
-// ws[own rows of e] = [b_e -] (D_e in_e + sum_s O_{e,s} in_nbr(e,s)) for the
-// CTA's ne elements from e_beg: a thread per (element, R rows) sums all the
-// element's blocks, column by column with the 1 + NF blocks' loads of a column
-// in flight together (the coarse levels are latency-bound); the inputs are
-// staged in shared memory, epc elements a pass.
-template <class S, int NF>
-__device__ void bsr_own(const CoopArgs<S>& a, const float* in, const float* bsub, float* ws, int e_beg, int ne,
-                        float* xs) {
+// acc[R] = rows R tt .. of (D_e x_e + sum_s O_{e,s} x_nbr) over the blocks
+// [b0, b1) of one element: all blocks of a column in flight together where
+// one thread takes them all, else block by block with a run of columns in
+// flight.  rev: columns from the last to the first (the next product finds
+// the last ones of this one in L2).
+template <class S, int NF, bool RES>
+__device__ __forceinline__ void bsr_rows(const S* D, const S* O, int nb, int ld, size_t bs, int b0, int b1, bool rev,
+                                         const float* xe, float* acc) {
   constexpr int R = Col16<S>::R, NSRC = 1 + NF;
-  const int nb = a.nb, ld = a.ld, tpe = a.tpe, epc = a.epc;
-  const size_t bs = (size_t)nb * ld;
-  const int sub = threadIdx.x / tpe, tt = threadIdx.x - sub * tpe;
-  for (int p0 = 0; p0 < ne; p0 += epc) {
-    const int nl = min(epc, ne - p0);
-    for (int t = threadIdx.x; t < nl * NSRC * nb; t += blockDim.x) {
-      const int el = t / (NSRC * nb), q = t - el * NSRC * nb, who = q / nb, j = q - who * nb;
-      const int e = e_beg + p0 + el;
-      const int src = who == 0 ? e : a.nbr[(size_t)e * NF + who - 1];
-      xs[t] = __ldcg(in + (size_t)src * nb + j);
-    }
-    __syncthreads();
-    if (sub < nl) {
-      const int e = e_beg + p0 + sub;
-      const S* base[NSRC];
-      base[0] = a.Dop + (size_t)e * bs + R * tt;
 #pragma unroll
-      for (int b = 1; b < NSRC; ++b) base[b] = a.O + ((size_t)e * NF + b - 1) * bs + R * tt;
-      const float* xe = xs + (size_t)sub * NSRC * nb;
-      float acc[R];
+  for (int j = 0; j < R; ++j) acc[j] = 0.f;
+  if (b0 == 0 && b1 == NSRC) {
+    const S* base[NSRC];
+    base[0] = D;
 #pragma unroll
-      for (int j = 0; j < R; ++j) acc[j] = 0.f;
+    for (int b = 1; b < NSRC; ++b) base[b] = O + (size_t)(b - 1) * bs;
 #pragma unroll 2
-      for (int c = 0; c < nb; ++c) {
-        float v[NSRC][R];
+    for (int c_ = 0; c_ < nb; ++c_) {
+      const int c = rev ? nb - 1 - c_ : c_;
+      float v[NSRC][R];
 #pragma unroll
-        for (int b = 0; b < NSRC; ++b) Col16<S>::load(base[b] + (size_t)c * ld, v[b]);
+      for (int b = 0; b < NSRC; ++b) Col16<S>::template load<RES>(base[b] + (size_t)c * ld, v[b]);
 #pragma unroll
-        for (int b = 0; b < NSRC; ++b) {
-          const float xv = xe[(size_t)b * nb + c];
+      for (int b = 0; b < NSRC; ++b) {
+        const float xv = xe[b * nb + c];
 #pragma unroll
-          for (int j = 0; j < R; ++j) acc[j] += v[b][j] * xv;
-        }
+        for (int j = 0; j < R; ++j) acc[j] = fmaf(v[b][j], xv, acc[j]);
       }
-      const int r0 = (p0 + sub) * nb + R * tt;
-      const size_t n0 = (size_t)e_beg * nb;
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (R * tt + j < nb) ws[r0 + j] = bsub ? __ldcg(bsub + n0 + r0 + j) - acc[j] : acc[j];
     }
-    __syncthreads();
+  } else {
+    for (int b = b0; b < b1; ++b)
+      col_run<S, RES>(b == 0 ? D : O + (size_t)(b - 1) * bs, nb, ld, xe + b * nb, acc);
   }
 }
 
-// z_e = D_e^{-1} v_e for the CTA's elements: v from shared memory, z to shared
-// memory (own rows) and device memory (the neighbours' products read it)
-template <class S>
-__device__ void bj_own(const CoopArgs<S>& a, const float* vs, float* zs, float* zg, int e_beg, int ne) {
-  constexpr int R = Col16<S>::R;
-  const int nb = a.nb, ld = a.ld, tpe = a.tpe, epc = blockDim.x / tpe;
-  const size_t bs = (size_t)nb * ld;
-  const int sub = threadIdx.x / tpe, tt = threadIdx.x - sub * tpe;
-  for (int p0 = 0; p0 < ne; p0 += epc) {
-    const int nl = min(epc, ne - p0);
-    if (sub < nl) {
-      const S* base = a.Dinv + (size_t)(e_beg + p0 + sub) * bs + R * tt;
-      const float* xe = vs + (size_t)(p0 + sub) * nb;
-      float acc[R];
-#pragma unroll
-      for (int j = 0; j < R; ++j) acc[j] = 0.f;
-#pragma unroll 16
-      for (int c = 0; c < nb; ++c) {
-        float m[R];
-        Col16<S>::load(base + (size_t)c * ld, m);
-        const float xv = xe[c];
-#pragma unroll
-        for (int j = 0; j < R; ++j) acc[j] += m[j] * xv;
-      }
-      const int r0 = (p0 + sub) * nb + R * tt;
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (R * tt + j < nb) {
-          zs[r0 + j] = acc[j];
-          zg[(size_t)e_beg * nb + r0 + j] = acc[j];
-        }
-    }
-  }
-}
-
-template <class S, int NF>
+template <class S, int NF, bool RES>
 __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S> a) {
+  constexpr int R = Col16<S>::R, NSRC = 1 + NF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int nu = a.nu, ldh = nu + 1, nb = a.nb;
-  double* h1 = reinterpret_cast<double*>(smem_raw);   // nu + 1: first-pass coefficients (FP64 sums)
-  double* h2 = h1 + ldh;                              // nu + 2: second pass, then ||w||^2
-  double* hx = h2 + ldh + 1;                          // 2: broadcast scalars
-  int* sflag = reinterpret_cast<int*>(hx + 2);        // 4 ints
-  float* H = reinterpret_cast<float*>(sflag + 4);     // (nu + 1) x nu, column-major
-  float* cs = H + (size_t)ldh * nu;
-  float* sn = cs + nu;
-  float* g = sn + nu;                                 // nu + 1
-  float* hf = g + ldh;                                // nu + 1: coefficients rounded to FP32, then y
-  float* redf = hf + ldh;                             // 33
+  const int nu = a.nu, ldh = nu + 1, nb = a.nb, ld = a.ld, tpe = a.tpe, ns = a.ns;
+  const size_t bs = (size_t)nb * ld;
   const int rmax = a.chunk * nb;
-  float* Vs = redf + ((33 + 3) & ~3);                 // [nu + 1][rmax]
+  S* Rs = reinterpret_cast<S*>(smem_raw);             // RES: [chunk][Dop, O.., Dinv]
+  float* Vs = reinterpret_cast<float*>(Rs + (RES ? (size_t)a.chunk * (NSRC + 1) * bs : 0));   // [nu + 1][rmax]
   float* Zs = Vs + (size_t)ldh * rmax;                // [nu][rmax]
   float* ws = Zs + (size_t)nu * rmax;                 // [rmax]
-  float* xs = ws + rmax;                              // [epc][1 + nf][nb]
+  float* ps = ws + rmax;                              // ns > 1: [ns][rmax] partial products
+  float* xs = ps + (ns > 1 ? (size_t)ns * rmax : 0);  // [epc][NSRC][nb]
+  float* H = xs + (size_t)a.epc * NSRC * nb;          // (nu + 1) x nu, column-major
+  float* cs = H + (size_t)ldh * nu;
+  float* sn = cs + nu;
+  float* g = sn + nu;                                 // nu + 1, then y
+  int* src = reinterpret_cast<int*>(g + ldh);         // [chunk][NSRC] element ids
+  float2* st = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(src + (size_t)a.chunk * NSRC) + 7) & ~(uintptr_t)7);   // [nu + 2]
+  __shared__ int timed_out;
 
-  const int G = gridDim.x, stride = 2 * ldh + 1;
-  double* mypart = a.part + (size_t)blockIdx.x * stride;   // [0, ldh): pass 1, [ldh, 2 ldh): pass 2, last: norm
-  double* tot = a.part + (size_t)G * stride;               // the sums, written by the last CTA of a barrier
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, G = gridDim.x;
+  const bool scalar_warp = warp == COOP_WORK / 32;
   const int e_beg = min(a.E, (int)blockIdx.x * a.chunk), ne = min(a.E, e_beg + a.chunk) - e_beg;
   const int rows = ne * nb;
-  const long N = a.N;
-  const unsigned expect = (unsigned)a.expect;
-  unsigned nbar = 0;
-
-  if (threadIdx.x == 0) sflag[1] = (*(volatile int*)a.status & ST_TIMEOUT) ? 1 : 0;
+  const float inv_nb = 1.0f / (float)nb;
+  if (tid == 0) timed_out = (*(volatile int*)a.status & ST_TIMEOUT) ? 1 : 0;
+  const unsigned base = *(volatile unsigned*)a.epoch;   // advanced at the end, after every CTA has read it
+  for (int t = tid; t < ne * NSRC; t += COOP_THREADS) {
+    const int el = t / NSRC, who = t - el * NSRC, e = e_beg + el;
+    src[t] = who == 0 ? e : a.nbr[(size_t)e * NF + who - 1];
+  }
+  if constexpr (RES) {
+    constexpr int V16 = 16 / sizeof(S);
+    const int per = (int)(bs / V16);                  // 16-byte words per block
+    uint4* dst = reinterpret_cast<uint4*>(Rs);
+    for (int t = tid; t < ne * (NSRC + 1) * per; t += COOP_THREADS) {
+      const int blk = t / per, q = t - blk * per, el = blk / (NSRC + 1), b = blk - el * (NSRC + 1);
+      const size_t e = e_beg + el;
+      const S* p = b == 0 ? a.Dop + e * bs : (b <= NF ? a.O + (e * NF + b - 1) * bs : a.Dinv + e * bs);
+      dst[t] = __ldg(reinterpret_cast<const uint4*>(p) + q);
+    }
+  }
   __syncthreads();
-  if (sflag[1]) return;   // an earlier wait ran out: leave x as it is
+  if (timed_out) return;   // an earlier wait ran out: leave x as it is
+#define COOP_LEAVE_IF(fail)                                                       \
+  if (__syncthreads_or((fail) ? 1 : 0)) {                                         \
+    if (tid == 0) atomicMax(a.epoch, base + (unsigned)nu + 8u);                   \
+    return;                                                                       \
+  }
 
-  // r = b - A x into w, ||r||^2
-  bsr_own<S, NF>(a, a.x, a.b, ws, e_beg, ne, xs);
+  // out = A in, or b - A in, on own rows
+  const int span = a.epc * tpe, sp = tid / span, sub = (tid - sp * span) / tpe, tt = tid - sp * span - sub * tpe;
+  const int bb0 = sp * NSRC / ns, bb1 = (sp + 1) * NSRC / ns;
+#define COOP_PRODUCT(own, ep, bsub, out, rev)                                                             \
+  for (int p0 = 0; p0 < ne; p0 += a.epc) {                                                                \
+    const int nl = min(a.epc, ne - p0);                                                                   \
+    const bool got = stage_inputs(src, NSRC, p0, nl, nb, inv_nb, e_beg, ne, a.x, own, a.zx, ep, a.status, xs); \
+    COOP_LEAVE_IF(!got)                                                                                   \
+    if (sp < ns && sub < nl) {                                                                     \
+      const int el = p0 + sub;                                                                            \
+      const size_t e = e_beg + el;                                                                        \
+      const S* D = (RES ? Rs + (size_t)el * (NSRC + 1) * bs : a.Dop + e * bs) + R * tt;                   \
+      const S* O = (RES ? Rs + ((size_t)el * (NSRC + 1) + 1) * bs : a.O + e * NF * bs) + R * tt;          \
+      float acc[R];                                                                                       \
+      bsr_rows<S, NF, RES>(D, O, nb, ld, bs, bb0, bb1, rev, xs + (size_t)sub * NSRC * nb, acc);           \
+      const int r0 = el * nb + R * tt;                                                                    \
+      _Pragma("unroll") for (int k = 0; k < R; ++k) if (R * tt + k < nb) {                                \
+        if (ns > 1)                                                                                       \
+          ps[(size_t)sp * rmax + r0 + k] = acc[k];                                                        \
+        else                                                                                              \
+          out[r0 + k] = bsub ? __ldcg(bsub + (size_t)e_beg * nb + r0 + k) - acc[k] : acc[k];              \
+      }                                                                                                   \
+    }                                                                                                     \
+    __syncthreads();                                                                                      \
+  }                                                                                                       \
+  if (ns > 1) {                                                                                           \
+    for (int r = tid; r < rows; r += COOP_THREADS) {                                                      \
+      float t = ps[r];                                                                                    \
+      for (int k = 1; k < ns; ++k) t += ps[(size_t)k * rmax + r];                                         \
+      out[r] = bsub ? __ldcg(bsub + (size_t)e_beg * nb + r) - t : t;                                      \
+    }                                                                                                     \
+    __syncthreads();                                                                                      \
+  }
+
+  // v_0 = r = b - A x, not normalised (exchange 0 brings its norm)
   {
-    float f = 0.f;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) f = fmaf(ws[r], ws[r], f);
-    const float s = block_sum_f(f, redf);
-    if (threadIdx.x == 0) mypart[2 * ldh] = (double)s;
+    const float* none = nullptr;
+    COOP_PRODUCT(none, 0u, a.b, Vs, false)
   }
-  if (!grid_barrier_sum(a.bar, ++nbar, expect, a.status, sflag, a.part, stride, 2 * ldh, 1, G, tot, h2)) return;
-  const double beta = sqrt(h2[0]);
-  if (!(beta > 0.0) || !isfinite(beta)) {
-    if (threadIdx.x == 0 && blockIdx.x == 0 && !isfinite(beta)) atomicOr(a.kflag, ST_NONFINITE);
-    return;   // b - A x = 0 (or not finite): nothing to smooth
-  }
-  for (int i = threadIdx.x; i < ldh; i += blockDim.x) g[i] = i == 0 ? (float)beta : 0.f;
-  float finv = (float)(1.0 / beta);
+  float rho = 1.f;          // |w - V h| as estimated: v_{j+1} = (w - V h) / rho
   int kdone = 0;
-  for (int j = 0; j < nu; ++j) {
-    // A: v_j = w / ||w||, z_j = D^{-1} v_j
+  for (int j = 0;; ++j) {
+    const unsigned ep = base + 1u + (unsigned)j;
     float* vj = Vs + (size_t)j * rmax;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) vj[r] = finv * ws[r];
-    __syncthreads();
-    float* zg = a.Z + (size_t)j * N;
-    bj_own<S>(a, vj, Zs + (size_t)j * rmax, zg, e_beg, ne);
-    if (!grid_barrier(a.bar, ++nbar, expect, a.status, sflag)) return;
-    // B: w = A z_j, first pass of inner products
-    bsr_own<S, NF>(a, zg, nullptr, ws, e_beg, ne, xs);
-    own_dots(j + 1, Vs, rmax, ws, rows, mypart);
-    if (!grid_barrier_sum(a.bar, ++nbar, expect, a.status, sflag, a.part, stride, 0, j + 1, G, tot, h1)) return;
-    // C: w -= V h1; second pass of inner products and ||w||^2 (at mypart[ldh + j + 1])
-    if (threadIdx.x <= j) hf[threadIdx.x] = (float)h1[threadIdx.x];
-    __syncthreads();
-    {
-      float f = 0.f;
-      for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-        float acc = ws[r];
-        for (int i = 0; i <= j; ++i) acc = fmaf(-hf[i], Vs[(size_t)i * rmax + r], acc);
-        ws[r] = acc;
-        f = fmaf(acc, acc, f);
+    if (j < nu) {
+      // the blocks of the coming product, meanwhile (see CoopArgs::pre)
+      const bool rev = (j & 1) == 0;
+      if constexpr (!RES) {
+        if (a.pre)
+          for (int t = tid; t < ne * NSRC; t += COOP_THREADS) {
+            const int el = t / NSRC, k = t - el * NSRC;
+            const size_t e = e_beg + el;
+            prefetch_l2(k == 0 ? a.Dop + e * bs : a.O + (e * NF + k - 1) * bs, (unsigned)(bs * sizeof(S)));
+          }
       }
-      const float s = block_sum_f(f, redf);
-      own_dots(j + 1, Vs, rmax, ws, rows, mypart + ldh);
-      if (threadIdx.x == 0) mypart[ldh + j + 1] = (double)s;
-    }
-    if (!grid_barrier_sum(a.bar, ++nbar, expect, a.status, sflag, a.part, stride, ldh, j + 2, G, tot, h2))
-      return;   // h2[j + 1] = ||w||^2
-    // D: w -= V h2, ||w - V h2|| from ||w||^2 - ||h2||^2; Hessenberg column j
-    // (h1 + h2, formed in parallel) in FP32
-    if (threadIdx.x <= j) {
-      hf[threadIdx.x] = (float)h2[threadIdx.x];
-      H[(size_t)j * ldh + threadIdx.x] = (float)(h1[threadIdx.x] + h2[threadIdx.x]);
-    }
-    if (threadIdx.x < 32) {   // ||h2||^2 (FP32: h2 is at rounding level against ||w||)
-      float q = 0.f;
-      for (int i = threadIdx.x; i <= j; i += 32) {
-        const float t = (float)h2[i];
-        q = fmaf(t, t, q);
-      }
+      // z_j = D^{-1} v_j: own rows to shared memory, published for the neighbours
+      float* zs = Zs + (size_t)j * rmax;
+      const int bsub_ = tid / tpe, btt = tid - bsub_ * tpe, bep = COOP_WORK / tpe;
+      if (bsub_ < bep) {
+        for (int el = bsub_; el < ne; el += bep) {
+          const size_t e = e_beg + el;
+          const S* M = (RES ? Rs + ((size_t)el * (NSRC + 1) + NSRC) * bs : a.Dinv + e * bs) + R * btt;
+          const float* xe = vj + (size_t)el * nb;
+          float acc[R];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      if (threadIdx.x == 0) hx[0] = h2[j + 1] - (double)q;
-    }
-    __syncthreads();
-    const double nw2 = h2[j + 1], hn2 = hx[0];
-    const bool explicit_norm = !(hn2 >= 0.01 * nw2);   // cancellation (or not finite): sum it
-    {
-      float f = 0.f;
-      for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-        float acc = ws[r];
-        for (int i = 0; i <= j; ++i) acc = fmaf(-hf[i], Vs[(size_t)i * rmax + r], acc);
-        ws[r] = acc;
-        f = fmaf(acc, acc, f);
+          for (int k = 0; k < R; ++k) acc[k] = 0.f;
+          col_run<S, RES>(M, nb, ld, xe, acc);
+          const int r0 = el * nb + R * btt;
+#pragma unroll
+          for (int k = 0; k < R; ++k)
+            if (R * btt + k < nb) {
+              zs[r0 + k] = acc[k];
+              st_val(a.zx + (size_t)e_beg * nb + r0 + k, acc[k], ep);
+            }
+        }
       }
-      if (explicit_norm) {
-        const float s = block_sum_f(f, redf);
-        if (threadIdx.x == 0) mypart[2 * ldh] = (double)s;
-      }
+      __syncthreads();
+      // w = A z_j
+      const float* none = nullptr;
+      COOP_PRODUCT(zs, ep, none, ws, rev)
     }
-    double hn;
-    if (explicit_norm) {
-      if (!grid_barrier_sum(a.bar, ++nbar, expect, a.status, sflag, a.part, stride, 2 * ldh, 1, G, tot, hx + 1))
-        return;
-      hn = sqrt(hx[1]);
-    } else {
-      hn = sqrt(hn2);
+    // exchange j
+    if constexpr (!RES) {
+      if (j < nu && a.pre)
+        for (int el = tid; el < ne; el += COOP_THREADS)
+          prefetch_l2(a.Dinv + (size_t)(e_beg + el) * bs, (unsigned)(bs * sizeof(S)));
     }
-    // earlier rotations, new rotation, g (every CTA alike, FP32)
-    if (threadIdx.x == 0) {
-      float* h = H + (size_t)j * ldh;
-      h[j + 1] = (float)hn;
-      for (int i = 0; i < j; ++i) {
-        const float p = h[i], q = h[i + 1];
-        h[i] = cs[i] * p + sn[i] * q;
-        h[i + 1] = -sn[i] * p + cs[i] * q;
-      }
-      const float p = h[j], q = h[j + 1];
-      const float rr = hypotf(p, q);
-      float c = 1.f, sv = 0.f;
-      if (rr != 0.f) {
-        c = p / rr;
-        sv = q / rr;
-      }
-      cs[j] = c;
-      sn[j] = sv;
-      h[j] = c * p + sv * q;
-      h[j + 1] = 0.f;
-      g[j + 1] = -sv * g[j];
-      g[j] = c * g[j];
+    uint4* px = a.px + (size_t)(j & 1) * (G + 1) * a.ni;
+    publish_dots(j, Vs, rmax, j < nu ? ws : nullptr, rows, px + blockIdx.x, G + 1, ep);
+    const bool got = gather_dots(px, G + 1, j + 2, G + a.extra, a.sums + (j & 1) * a.ni, ep, a.status, st);
+    COOP_LEAVE_IF(!got)
+    float ss = 0.f, sc = 0.f, tq = 0.f;
+    for (int i = 0; i < j; ++i) {
+      const float2 q = st[i];
+      ss = fmaf(q.x, q.x, ss);
+      sc = fmaf(q.x, q.y, sc);
+      tq = fmaf(q.y, q.y, tq);
     }
-    __syncthreads();
-    kdone = j + 1;
-    if (!(hn > 0.0) || !isfinite(hn)) {   // breakdown: the Krylov space is exhausted
-      if (threadIdx.x == 0 && blockIdx.x == 0 && !isfinite(hn)) atomicOr(a.kflag, ST_NONFINITE);
+    const float be2 = st[j].x - ss;
+    const bool fine = be2 > 0.f && isfinite(be2);
+    const float beta = fine ? sqrtf(be2) : 0.f, ib = fine ? 1.f / beta : 0.f;
+    const float hj = (st[j].y - sc) * ib, ww = st[j + 1].x;
+    if (scalar_warp) {
+      // column j - 1 completed and rotated, column j begun (this warp alone)
+      if (j == 0) {
+        for (int i = lane; i < ldh; i += 32) g[i] = i == 0 ? beta : 0.f;
+      } else {
+        float* h = H + (size_t)(j - 1) * ldh;
+        for (int i = lane; i < j; i += 32) h[i] = fmaf(rho, st[i].x, h[i]);
+        __syncwarp();
+        if (lane == 0) {
+          float p = h[0];
+          for (int i = 0; i + 1 < j; ++i) {
+            const float q = h[i + 1];
+            h[i] = cs[i] * p + sn[i] * q;
+            p = -sn[i] * p + cs[i] * q;
+          }
+          const float q = rho * beta, rr = hypotf(p, q);
+          float c = 1.f, sv = 0.f;
+          if (rr != 0.f) {
+            c = p / rr;
+            sv = q / rr;
+          }
+          cs[j - 1] = c;
+          sn[j - 1] = sv;
+          h[j - 1] = c * p + sv * q;
+          g[j] = -sv * g[j - 1];
+          g[j - 1] = c * g[j - 1];
+        }
+      }
+      if (j < nu && fine) {
+        float* h = H + (size_t)j * ldh;
+        for (int i = lane; i <= j; i += 32) h[i] = i < j ? st[i].y : hj;
+      }
+      __syncwarp();
+    }
+    kdone = j;
+    if (!fine || j == nu) {   // the Krylov space is exhausted (or not finite), or complete
+      if (!fine && !isfinite(be2) && tid == 0 && blockIdx.x == 0) atomicOr(a.kflag, ST_NONFINITE);
       break;
     }
-    finv = (float)(1.0 / hn);
+    const float est = fmaxf(ww - tq - hj * hj, 1e-6f * ww);
+    rho = est > 0.f ? sqrtf(est) : 1.f;
+    const float ir = 1.f / rho;
+    if (tid < COOP_WORK) {
+      float* vn = vj + rmax;
+      for (int r = tid; r < rows; r += COOP_WORK) {
+        float v = vj[r], w = ws[r];
+        const float* q = Vs + r;
+#pragma unroll 8
+        for (int i = 0; i < j; ++i) {
+          const float2 c = st[i];
+          const float vi = q[(size_t)i * rmax];
+          v = fmaf(-c.x, vi, v);
+          w = fmaf(-c.y, vi, w);
+        }
+        v *= ib;
+        vj[r] = v;
+        vn[r] = fmaf(-hj, v, w) * ir;
+      }
+    }
+    __syncthreads();
   }
-  // y = H[:k,:k]^{-1} g[:k] (back substitution, FP32, into hf), x += Z y on own rows
-  if (threadIdx.x == 0) {
+  if (blockIdx.x == 0 && tid == 0) *(volatile unsigned*)a.epoch = base + (unsigned)nu + 8u;
+  if (kdone == 0) return;   // b - A x = 0 (or not finite): nothing to smooth
+  // y = H[:k,:k]^{-1} g[:k] (into g; the scalar warp, which rotated it), x += Z y on own rows
+  if (scalar_warp) {
     for (int i = kdone - 1; i >= 0; --i) {
-      float s = g[i];
-      for (int c = i + 1; c < kdone; ++c) s -= H[(size_t)c * ldh + i] * hf[c];
-      const float d = H[(size_t)i * ldh + i];
-      hf[i] = d != 0.f ? s / d : 0.f;
+      const float d = H[(size_t)i * ldh + i], y = d != 0.f ? g[i] / d : 0.f;
+      __syncwarp();
+      for (int c = lane; c < i; c += 32) g[c] = fmaf(-H[(size_t)i * ldh + c], y, g[c]);
+      if (lane == 0) g[i] = y;
+      __syncwarp();
     }
   }
   __syncthreads();
   float* xo = a.x + (size_t)e_beg * nb;
-  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+  for (int r = tid; r < rows; r += COOP_THREADS) {
     float acc = xo[r];
-    for (int i = 0; i < kdone; ++i) acc = fmaf(hf[i], Zs[(size_t)i * rmax + r], acc);
+    for (int i = 0; i < kdone; ++i) acc = fmaf(g[i], Zs[(size_t)i * rmax + r], acc);
     xo[r] = acc;
   }
+#undef COOP_PRODUCT
+#undef COOP_LEAVE_IF
 }
 
-static size_t coop_smem(int nu, int nb, int nf, int chunk, int epc) {
-  const size_t ldh = nu + 1;
-  const size_t dbl = 2 * ldh + 1 + 2;
-  const size_t fsc = ldh * nu + 2 * (size_t)nu + 2 * ldh + 36;   // H, cs, sn, g, hf, redf (padded)
-  const size_t rmax = (size_t)chunk * nb;
-  const size_t flt = (2 * (size_t)nu + 2) * rmax + (size_t)epc * (1 + nf) * nb;
-  return dbl * sizeof(double) + 4 * sizeof(int) + (fsc + flt) * sizeof(float) + 16;
+// dynamic shared memory in bytes; res: with the CTA's blocks
+template <class S>
+static size_t coop_smem(int nu, int nb, int ld, int nf, int chunk, int epc, int ns, bool res) {
+  const size_t ldh = nu + 1, rmax = (size_t)chunk * nb;
+  const size_t fl = ldh * rmax + nu * rmax + rmax + (ns > 1 ? ns * rmax : 0) + (size_t)epc * (1 + nf) * nb +
+                    ldh * nu + 2 * (size_t)nu + ldh + (size_t)chunk * (1 + nf);
+  return fl * sizeof(float) + 8 + sizeof(float2) * (nu + 2) +
+         (res ? (size_t)chunk * (2 + nf) * nb * ld * sizeof(S) : 0);
 }
 
 template <class S, int NF>
-static cudaError_t plan_coop(int nb, int ld, int nf, int E, int nu, CoopPlan* plan) {
+static cudaError_t plan_coop(int nb, int ld, int E, int nu, CoopPlan* plan) {
   constexpr int R = Col16<S>::R;
   plan->ok = 0;
   if (ld % R || E < 1) return cudaSuccess;
   const int tpe = ld / R;
-  if (tpe > COOP_THREADS) return cudaSuccess;
-  auto kern = coop_smooth_kernel<S, NF>;
-  cudaError_t e = allow_max_smem(kern);
-  if (e != cudaSuccess) return e;
+  if (tpe > COOP_WORK) return cudaSuccess;
   int dev = 0, nsm = 0, smax = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -515,41 +628,65 @@ static cudaError_t plan_coop(int nb, int ld, int nf, int E, int nu, CoopPlan* pl
   int grid = std::min(E, nsm);
   const int chunk = (E + grid - 1) / grid;
   grid = (E + chunk - 1) / chunk;   // no CTA without elements
-  const int epc = std::max(1, std::min(chunk, COOP_THREADS / tpe));
-  const size_t smem = coop_smem(nu, nb, nf, chunk, epc);
-  cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, kern);
-  if (e != cudaSuccess) return e;
-  if (smem + fa.sharedSizeBytes > (size_t)smax) return cudaSuccess;   // the rows do not fit: per-operation smoother
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, COOP_THREADS, smem);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) return cudaSuccess;
-  plan->ok = 1;
-  plan->nu_max = nu;
-  plan->grid = grid;
-  plan->chunk = chunk;
-  plan->epc = epc;
-  plan->tpe = tpe;
-  plan->smem = smem;
+  const int epc = std::max(1, std::min(chunk, COOP_WORK / tpe));
+  // where one thread per (element, rows) leaves most of the CTA idle, an
+  // element's 1 + nf blocks are shared out over ns threads (p = 1, p = 0:
+  // chains of dependent loads, not bandwidth)
+  const int ns = epc < chunk ? 1 : std::max(1, std::min(1 + NF, COOP_WORK / (epc * tpe)));
+  // a level whose blocks stay in L2 from one product to the next has them asked
+  // for during the phases before (p = 1 on 16^3: 223 -> 190 us a call; 100 x 75
+  // quads, p = 2: 290 -> 243); the blocks of a larger level come from DRAM
+  // every time, and asking for them all at once only evicts what comes first
+  // (p = 2 on 16^3, 328 MB: 745 -> 985 us)
+  int l2 = 0;
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+  const int pre = (double)E * (2 + NF) * nb * ld * sizeof(S) <= 0.85 * l2 ? 1 : 0;
+  if ((long)epc * (1 + NF) * nb >= (1 << 20)) return cudaSuccess;   // stage_inputs' exact index range
+  for (int res = 1; res >= 0; --res) {
+    const size_t smem = coop_smem<S>(nu, nb, ld, NF, chunk, epc, ns, res);
+    auto kern = res ? coop_smooth_kernel<S, NF, true> : coop_smooth_kernel<S, NF, false>;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return e;
+    if (smem + fa.sharedSizeBytes > (size_t)smax) continue;   // rows only; then the per-operation smoother
+    e = allow_max_smem(kern);
+    if (e != cudaSuccess) return e;
+    int occ = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, COOP_THREADS, smem);
+    if (e != cudaSuccess) return e;
+    if (occ < 1) continue;
+    plan->ok = 1;
+    plan->nu_max = nu;
+    plan->grid = grid;
+    plan->chunk = chunk;
+    plan->epc = epc;
+    plan->tpe = tpe;
+    plan->ns = ns;
+    plan->pre = pre;
+    plan->res = res;
+    plan->smem = smem;
+    plan->part_bytes = sizeof(uint4) * 2 * (size_t)(grid + 2) * (nu + 2);
+    plan->z_bytes = sizeof(unsigned long long) * (size_t)E * nb;
+    return cudaSuccess;
+  }
   return cudaSuccess;
 }
 
 cudaError_t plan_coop_smoother(int bf16, int nb, int nf, int E, int nu, CoopPlan* plan) {
   plan->ok = 0;
   if (nf == 6)
-    return bf16 ? plan_coop<unsigned short, 6>(nb, ld_bf16(nb), nf, E, nu, plan)
-                : plan_coop<float, 6>(nb, inv_ld<float>(nb), nf, E, nu, plan);
+    return bf16 ? plan_coop<unsigned short, 6>(nb, ld_bf16(nb), E, nu, plan)
+                : plan_coop<float, 6>(nb, inv_ld<float>(nb), E, nu, plan);
   if (nf == 4)
-    return bf16 ? plan_coop<unsigned short, 4>(nb, ld_bf16(nb), nf, E, nu, plan)
-                : plan_coop<float, 4>(nb, inv_ld<float>(nb), nf, E, nu, plan);
+    return bf16 ? plan_coop<unsigned short, 4>(nb, ld_bf16(nb), E, nu, plan)
+                : plan_coop<float, 4>(nb, inv_ld<float>(nb), E, nu, plan);
   return cudaSuccess;   // other face counts keep the launch-per-operation smoother
 }
 
-template <class S>
+template <class S, int NF>
 static cudaError_t launch_coop(const CoopPlan& pl, const S* Dinv, const S* Dop, const S* O, int ld, const int* nbr,
-                               int nf, const float* b, float* x, int nu, Krylov<float>& K, double* part,
-                               unsigned* bar, int* status, int expect_extra, int nb, int E, cudaStream_t st) {
+                               const float* b, float* x, int nu, Krylov<float>& K, const CoopBuffers& buf,
+                               int* status, int extra, int nb, int E, cudaStream_t st) {
   CoopArgs<S> a;
   a.Dinv = Dinv;
   a.Dop = Dop;
@@ -557,23 +694,23 @@ static cudaError_t launch_coop(const CoopPlan& pl, const S* Dinv, const S* Dop, 
   a.nbr = nbr;
   a.b = b;
   a.x = x;
-  a.Z = K.Z;
-  a.part = part;
-  a.bar = bar;
+  a.zx = (unsigned long long*)buf.z;
+  a.px = (uint4*)buf.part;
+  a.sums = a.px + 2 * (size_t)(pl.grid + 1) * (pl.nu_max + 2);
+  a.epoch = buf.epoch;
   a.status = status;
   a.kflag = K.kdim + 1;
-  a.N = K.N;
   a.nu = nu;
   a.nb = nb;
   a.ld = ld;
-  a.nf = nf;
   a.E = E;
   a.chunk = pl.chunk;
   a.epc = pl.epc;
   a.tpe = pl.tpe;
-  a.expect = pl.grid + expect_extra;
-  cudaError_t e = cudaMemsetAsync(bar, 0, COOP_BAR_WORDS * sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
+  a.ns = pl.ns;
+  a.ni = pl.nu_max + 2;
+  a.extra = extra > 0 ? 1 : 0;
+  a.pre = pl.pre;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.grid);
   cfg.blockDim = dim3(COOP_THREADS);
@@ -585,21 +722,24 @@ static cudaError_t launch_coop(const CoopPlan& pl, const S* Dinv, const S* Dop, 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   note_launch();
-  if (nf == 6) return cudaLaunchKernelEx(&cfg, coop_smooth_kernel<S, 6>, a);
-  return cudaLaunchKernelEx(&cfg, coop_smooth_kernel<S, 4>, a);
+  if (pl.res) return cudaLaunchKernelEx(&cfg, coop_smooth_kernel<S, NF, true>, a);
+  return cudaLaunchKernelEx(&cfg, coop_smooth_kernel<S, NF, false>, a);
 }
 
 cudaError_t launch_coop_smoother(const CoopPlan& pl, const float* Dinv, const float* Dop, const float* O,
                                  const unsigned short* Dinv16, const unsigned short* Dop16, const unsigned short* O16,
                                  const int* nbr, int nf, const float* b, float* x, int nu, Krylov<float>& K,
-                                 double* part, unsigned* bar, int* status, int expect_extra, int nb, int E,
-                                 cudaStream_t st) {
-  if (!pl.ok || nu > pl.nu_max || nu > K.nmax) return cudaErrorInvalidValue;
-  if (Dinv16)
-    return launch_coop<unsigned short>(pl, Dinv16, Dop16, O16, ld_bf16(nb), nbr, nf, b, x, nu, K, part, bar, status,
-                                       expect_extra, nb, E, st);
-  return launch_coop<float>(pl, Dinv, Dop, O, inv_ld<float>(nb), nbr, nf, b, x, nu, K, part, bar, status,
-                            expect_extra, nb, E, st);
+                                 const CoopBuffers& buf, int* status, int extra, int nb, int E, cudaStream_t st) {
+  if (!pl.ok || nu < 1 || nu > pl.nu_max || nu > K.nmax) return cudaErrorInvalidValue;
+#define GO(NF)                                                                                                     \
+  return Dinv16 ? launch_coop<unsigned short, NF>(pl, Dinv16, Dop16, O16, ld_bf16(nb), nbr, b, x, nu, K, buf, status, \
+                                                  extra, nb, E, st)                                                \
+                : launch_coop<float, NF>(pl, Dinv, Dop, O, inv_ld<float>(nb), nbr, b, x, nu, K, buf, status, extra,   \
+                                         nb, E, st)
+  if (nf == 6) GO(6);
+  if (nf == 4) GO(4);
+#undef GO
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace dgk

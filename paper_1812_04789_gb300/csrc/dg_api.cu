@@ -229,9 +229,10 @@ static dg_status alloc_mg(dg_pmg h, MG<T>& mg) {
       // coarse blocks column-major when the FP32 neighbour blocks come from
       // probe_nbr_kernel (decided here once: the captured graph relies on it)
       // (the column-major mat-vec runs one thread per block and 16 bytes of rows: at most 256 per element)
-      const int tpb1 = (1 + 2 * M.d) * (inv_ld<T>(mg.lv[1].nb) / (int)(16 / sizeof(T)));
-      L.co_t = M.kind == DG_MESH_STRUCTURED && std::is_same<T, float>::value && tpb1 <= 256 &&
-                       probe_nbr_colmajor_ok(M, mg.lv[1].nm) ? 1 : 0;
+      // or, on triangles, from the coloured probe (which writes either layout)
+      const int tpb1 = (1 + M.nfaces()) * (inv_ld<T>(mg.lv[1].nb) / (int)(16 / sizeof(T)));
+      L.co_t = std::is_same<T, float>::value && tpb1 <= 256 &&
+                       (M.kind == DG_MESH_TRI || probe_nbr_colmajor_ok(M, mg.lv[1].nm)) ? 1 : 0;
       L.cs = L.co_t ? L.bs : (size_t)L.nb * L.nb;
       (void)nbl;
       CK(dalloc(mg.allocs, (void**)&L.Dop, sizeof(T) * (size_t)M.E * L.cs, &h->block_bytes));
@@ -254,12 +255,11 @@ static dg_status alloc_mg(dg_pmg h, MG<T>& mg) {
       h->vector_bytes += L.kr.bytes();
     }
     // persistent smoother of an inherited FP32 level (column-major or BF16
-    // blocks, face-neighbour graph of the structured mesh); DG_PMG_NO_COOP=1
-    // keeps the launch-per-operation smoother
+    // blocks); DG_PMG_NO_COOP=1 keeps the launch-per-operation smoother
     const char* nco = getenv("DG_PMG_NO_COOP");
     const bool bf16 = o.block_storage == DG_STORE_BF16;
-    if (std::is_same<T, float>::value && l >= 1 && o.cycle != DG_CYCLE_BJ && M.kind == DG_MESH_STRUCTURED &&
-        (L.co_t || bf16) && !(nco && nco[0] == '1') &&
+    if (std::is_same<T, float>::value && l >= 1 && o.cycle != DG_CYCLE_BJ && (L.co_t || bf16) &&
+        !(nco && nco[0] == '1') &&
         !(o.coarse_precond == DG_COARSE_BILU && l == nl - 1)) {
       CK(plan_coop_smoother(bf16 ? 1 : 0, L.nb, M.nfaces(), M.E, nmax, &L.coop));
       if (L.coop.ok) {
@@ -333,6 +333,7 @@ static dg_status compute_mg(dg_pmg h, MG<T>& mg, const double* W64, cudaStream_t
   if (mg.Pv) CK(launch_primal_cache(M, (const float*)mg.W, (float*)mg.Pv, (float*)mg.Pf, st));
   if (M.kind == DG_MESH_TRI)   // coloured JVP probing, seeds and products in level 0's work vectors
     CK(launch_probe_blocks_tri<T>(M, mg.W, (T)h->sigma, mg.lv[0].Dinv, mg.lv[0].bs, nl > 1 ? mg.lv[1].O : nullptr,
+                                  nl > 1 ? mg.lv[1].cs : 0, nl > 1 && mg.lv[1].co_t ? inv_ld<T>(mg.lv[1].nb) : 0,
                                   nl > 1 ? mg.lv[1].nm : 0, mg.lv[0].r, mg.lv[0].t, st));
   else
     CK(launch_probe_blocks<T>(M, mg.W, (T)h->sigma, mg.lv[0].Dinv, mg.lv[0].bs, nl > 1 ? mg.lv[1].O : nullptr,
@@ -731,7 +732,7 @@ static dg_status export_level(const MG<T>& mg, const Mesh& M, T* W, double sigma
       CK(launch_unpack_inverse<T>(L.O, L.cs, L.co_t, out, nb, (long)nblk, st));
   } else if (which == DG_BLOCKS_DIAG) {
     if (level == 0 && M.kind == DG_MESH_TRI)   // the fine-level probe again, at the stored state and shift
-      CK(launch_probe_blocks_tri<T>(M, W, (T)sigma, out, (size_t)nb * nb, nullptr, 0, mg.lv[0].r, mg.lv[0].t, st));
+      CK(launch_probe_blocks_tri<T>(M, W, (T)sigma, out, (size_t)nb * nb, nullptr, 0, 0, 0, mg.lv[0].r, mg.lv[0].t, st));
     else if (level == 0)
       CK(launch_probe_blocks<T>(M, W, (T)sigma, out, (size_t)nb * nb, nullptr, 0, 0, mg.scratch, mg.scratch_elems,
                                 st));

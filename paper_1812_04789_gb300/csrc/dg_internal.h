@@ -115,11 +115,12 @@ cudaError_t launch_residual(const Mesh& M, const T* W, const T* V, const T* S, T
                             T* out, cudaStream_t st, const T* Pv = nullptr, const T* Pf = nullptr, int parts = 3);
 
 // Blocks of a triangle mesh by coloured JVP probing (csrc/dg_tri.cu): D (row-
-// major, dstride apart) = dR_e/dW_e + sigma |J_e| I; O (if given, row-major
-// nbc^2 apart, [E][3]) the neighbour blocks on the modes of the first nmc.
+// major, dstride apart) = dR_e/dW_e + sigma |J_e| I; O (if given, [E][3], ostride
+// apart, column-major with leading dimension old or, old = 0, row-major) the
+// neighbour blocks on the modes of the first nmc.
 template <class T>
-cudaError_t launch_probe_blocks_tri(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, int nmc,
-                                    T* seed, T* out, cudaStream_t st);
+cudaError_t launch_probe_blocks_tri(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, size_t ostride,
+                                    int old, int nmc, T* seed, T* out, cudaStream_t st);
 // Residual / exact JVP on a triangle mesh (csrc/dg_tri.cu), same contract.
 template <class T>
 cudaError_t launch_residual_tri(const Mesh& M, const T* W, const T* V, const T* S, T sigma, bool jvp, T* out,

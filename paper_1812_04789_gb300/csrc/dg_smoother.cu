@@ -680,6 +680,9 @@ cudaError_t plan_coop_smoother(int bf16, int nb, int nf, int E, int nu, CoopPlan
   if (nf == 4)
     return bf16 ? plan_coop<unsigned short, 4>(nb, ld_bf16(nb), E, nu, plan)
                 : plan_coop<float, 4>(nb, inv_ld<float>(nb), E, nu, plan);
+  if (nf == 3)
+    return bf16 ? plan_coop<unsigned short, 3>(nb, ld_bf16(nb), E, nu, plan)
+                : plan_coop<float, 3>(nb, inv_ld<float>(nb), E, nu, plan);
   return cudaSuccess;   // other face counts keep the launch-per-operation smoother
 }
 
@@ -738,6 +741,7 @@ cudaError_t launch_coop_smoother(const CoopPlan& pl, const float* Dinv, const fl
                                          nb, E, st)
   if (nf == 6) GO(6);
   if (nf == 4) GO(4);
+  if (nf == 3) GO(3);
 #undef GO
   return cudaErrorInvalidValue;
 }

@@ -455,7 +455,7 @@ __global__ void tri_seed_kernel(long N, int nb, const int* __restrict__ colour, 
 template <class T>
 __global__ void tri_gather_kernel(int E, int nb, int nm, const int* __restrict__ colour, const int* __restrict__ nbr,
                                   int c, int jj, const T* __restrict__ out, const T* __restrict__ slots, T* D,
-                                  size_t dstride, T* O, int nmc) {
+                                  size_t dstride, T* O, size_t ostride, int old, int nmc) {
   const int nbc = 4 * nmc;
   const long nD = (long)E * nb, nO = O ? (long)E * 3 * nbc : 0;
   const int jv = jj / nm, ji = jj - jv * nm;
@@ -471,7 +471,8 @@ __global__ void tri_gather_kernel(int E, int nb, int nm, const int* __restrict__
       const int k = nbr[ef];
       if (ji < nmc && k != e && colour[k] == c) {
         const int rv = rc / nmc, ri = rc - rv * nmc;
-        O[ef * nbc * nbc + (size_t)rc * nbc + jv * nmc + ji] = slots[ef * nb + rv * nm + ri];
+        const int col = jv * nmc + ji;
+        O[ef * ostride + (old ? (size_t)col * old + rc : (size_t)rc * nbc + col)] = slots[ef * nb + rv * nm + ri];
       }
     }
   }
@@ -480,8 +481,8 @@ __global__ void tri_gather_kernel(int E, int nb, int nm, const int* __restrict__
 }  // namespace
 
 template <class T>
-cudaError_t launch_probe_blocks_tri(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, int nmc,
-                                    T* seed, T* out, cudaStream_t st) {
+cudaError_t launch_probe_blocks_tri(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, size_t ostride,
+                                    int old, int nmc, T* seed, T* out, cudaStream_t st) {
   const long N = (long)M.E * M.nb;
   const T* slots = std::is_same<T, double>::value ? (const T*)M.t64.slots : (const T*)M.t32.slots;
   const int gs = (int)std::min<long>((N + 255) / 256, 4096);
@@ -495,15 +496,15 @@ cudaError_t launch_probe_blocks_tri(const Mesh& M, const T* W, T sigma, T* D, si
       if (e != cudaSuccess) return e;
       note_launch();
       tri_gather_kernel<T><<<gg, 256, 0, st>>>(M.E, M.nb, M.nm, M.tcolour, M.tnbr, c, jj, out, slots, D, dstride, O,
-                                               nmc);
+                                               ostride, old, nmc);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
   return cudaSuccess;
 }
-template cudaError_t launch_probe_blocks_tri<double>(const Mesh&, const double*, double, double*, size_t, double*, int,
-                                                     double*, double*, cudaStream_t);
-template cudaError_t launch_probe_blocks_tri<float>(const Mesh&, const float*, float, float*, size_t, float*, int,
-                                                    float*, float*, cudaStream_t);
+template cudaError_t launch_probe_blocks_tri<double>(const Mesh&, const double*, double, double*, size_t, double*,
+                                                     size_t, int, int, double*, double*, cudaStream_t);
+template cudaError_t launch_probe_blocks_tri<float>(const Mesh&, const float*, float, float*, size_t, float*,
+                                                    size_t, int, int, float*, float*, cudaStream_t);
 
 // ---------------------------------------------------------------- mesh build
 namespace {

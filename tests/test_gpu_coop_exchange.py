@@ -35,12 +35,19 @@ def _lib():
     ("vortex", 2, (64, 61), 2, (2, 0), 1, 1),           # one iteration, 26 elements per CTA
     ("tgv", 3, (1, 4, 5), 2, (2, 1, 0), 8, 12),         # an element that is its own neighbour
     ("tgv", 3, (7, 9, 8), 3, (3, 2, 1, 0), 10, 35),     # 504 elements: chunks of 4, streamed and resident blocks
+    ("tri", 2, (2, 2), 1, (1, 0), 4, 8),                # 8 triangles, three faces each
+    ("tri", 2, (13, 11), 4, (4, 2, 1, 0), 10, 30),      # 286 triangles: chunks of 2
 ])
 def test_exchange_matches_launch_per_operation(case, dim, n, p, levels, nu, nuc, monkeypatch):
-    cfg = wl.make_config(case, dim, n, p, M=0.5 if dim == 2 else 0.1, Re=1000.0, dt_conv=0.05)
-    W = torch.from_numpy(wl.perturbed_state(cfg, amp=0.02)).cuda()
+    if case == "tri":
+        cfg = wl.tri_config(n, p, dt_conv=0.05)
+        W = torch.from_numpy(wl.tri_perturbed_state(cfg, amp=0.02)).cuda()
+        m = B.Mesh.from_tri_workload(wl.tri_mesh(cfg), wl.tri_physics(cfg), p)
+    else:
+        cfg = wl.make_config(case, dim, n, p, M=0.5 if dim == 2 else 0.1, Re=1000.0, dt_conv=0.05)
+        W = torch.from_numpy(wl.perturbed_state(cfg, amp=0.02)).cuda()
+        m = B.Mesh.from_workload(wl.mesh_desc(cfg), wl.physics(cfg))
     r = torch.from_numpy(wl.random_vector(W.shape, 7)).cuda()
-    m = B.Mesh.from_workload(wl.mesh_desc(cfg), wl.physics(cfg))
     out = []
     for off in ("1", "0"):
         monkeypatch.setenv("DG_PMG_NO_COOP", off)

@@ -369,6 +369,11 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
     return launch_probe_nbr(M, (const float*)W, (float*)O, nmc, 1, st);
   }
   bool nbr_only = false;
+  if constexpr (std::is_same<T, double>::value) {
+    const char* e = getenv("DG_PROBE_SIMT");
+    if (!(e && e[0] == '1') && probe64_fits(M, O ? nmc : 0))
+      return launch_probe64(M, W, sigma, D, dstride, O, nmc, nbr_colmajor, st);
+  }
   if (std::is_same<T, float>::value && use_tc(M)) {
     cudaError_t e = launch_probe_tc(M, (const float*)W, (float)sigma, (float*)D, dstride, st);
     if (e != cudaSuccess) return e;

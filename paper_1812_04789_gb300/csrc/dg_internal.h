@@ -176,6 +176,14 @@ cudaError_t launch_probe_tc(const Mesh& M, const float* W, float sigma, float* D
                             cudaStream_t st);
 cudaError_t build_tc_tables(Mesh& M);
 
+// FP64 blocks (csrc/dg_probe64.cu): D as launch_probe_blocks, O (may be null)
+// column-major with leading dimension inv_ld(nbc), nbc * inv_ld(nbc) apart, or
+// row-major, nbc^2 apart.  probe64_fits: structured, no direction of one
+// element, blocks within the kernel's registers and shared memory.
+bool probe64_fits(const Mesh& M, int nmc);
+cudaError_t launch_probe64(const Mesh& M, const double* W, double sigma, double* D, size_t dstride, double* O,
+                           int nmc, int colmajor, cudaStream_t st);
+
 // FP32 neighbour blocks O[e][2k+side] (first nmc modes per variable, row-major
 // nbc x nbc) for meshes with the tensor-core probe tables and no direction of
 // one element; probe_nbr_fits says whether the kernel applies.

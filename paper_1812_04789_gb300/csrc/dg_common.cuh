@@ -79,11 +79,69 @@ __host__ __device__ __forceinline__ float tan_part(float a) { return a; }
 // |x| continued so that the derivative at x = 0 is +1 (x >= 0 is "positive")
 template <class S> __host__ __device__ __forceinline__ S sabs(S x) { return val(x) >= 0 ? x : -x; }
 
+// c + a b and c - a b (a, b, c numbers or duals), written so that every product
+// of a dual's tangent fuses with an addition: three multiply-adds, where the
+// separate product and sum take five operations
+__host__ __device__ __forceinline__ double madd(double a, double b, double c) { return a * b + c; }
+__host__ __device__ __forceinline__ float madd(float a, float b, float c) { return a * b + c; }
+__host__ __device__ __forceinline__ double msub(double a, double b, double c) { return c - a * b; }
+__host__ __device__ __forceinline__ float msub(float a, float b, float c) { return c - a * b; }
+template <class T> __host__ __device__ __forceinline__ Dual<T> madd(Dual<T> a, Dual<T> b, Dual<T> c) {
+  return Dual<T>(a.v * b.v + c.v, a.d * b.v + (a.v * b.d + c.d));
+}
+template <class T> __host__ __device__ __forceinline__ Dual<T> msub(Dual<T> a, Dual<T> b, Dual<T> c) {
+  return Dual<T>(c.v - a.v * b.v, (c.d - a.v * b.d) - a.d * b.v);
+}
+template <class T> __host__ __device__ __forceinline__ Dual<T> madd(T a, Dual<T> b, Dual<T> c) {
+  return Dual<T>(a * b.v + c.v, a * b.d + c.d);
+}
+template <class T> __host__ __device__ __forceinline__ Dual<T> msub(T a, Dual<T> b, Dual<T> c) {
+  return Dual<T>(c.v - a * b.v, c.d - a * b.d);
+}
+// sqrt(a) where ia = 1/a is at hand: the tangent a' / (2 sqrt(a)) = a' sqrt(a) ia / 2
+// needs no division
+template <class T> __host__ __device__ __forceinline__ Dual<T> dsqrt(Dual<T> a, Dual<T> ia) {
+  const T r = sqrt(a.v);
+  return Dual<T>(r, a.d * (T(0.5) * r * ia.v));
+}
+__host__ __device__ __forceinline__ double dsqrt(double a, double) { return sqrt(a); }
+__host__ __device__ __forceinline__ float dsqrt(float a, float) { return sqrtf(a); }
+
 // ----------------------------------------------------------------- physics
+// The FP64 kernels are bound by the number of FP64 operations (two lanes per
+// clock and SM), so the pointwise physics spends as few as it can: primitives
+// once per trace, four divisions and three square roots per face point, the
+// symmetric parts of the stress and of rho v v once, the viscosity multiplied
+// into the stress only, structural zeros never touched.  A face point of the
+// JVP takes about 700 FP64 operations (2,050 when every routine formed its
+// own primitives and full tensors), a volume point 250.
 template <class T>
 struct Phys {
   T gamma, gm1, Pr, mu, Rgas, eta, roe_delta, kappa;  // kappa = mu c_p / Pr
+  T kq = T(0);    // kappa (gamma - 1) / R; 0 = form it here
+  T hrd = T(0);   // 1 / (2 roe_delta); 0 = form it here
+  __host__ __device__ __forceinline__ T heat() const { return kq != T(0) ? kq : kappa * (gm1 / Rgas); }
+  __host__ __device__ __forceinline__ T half_inv_delta() const { return hrd != T(0) ? hrd : T(0.5) / roe_delta; }
 };
+
+// 1/rho, velocity, specific total energy, pressure, total enthalpy
+template <int D, class S>
+struct Prim {
+  S ir, vel[D], e0, p, h0;
+};
+template <int D, class S, class T>
+__host__ __device__ __forceinline__ void primitives(const S* u, const Phys<T>& ph, Prim<D, S>& P) {
+  constexpr int M = D + 2;
+  P.ir = T(1) / u[0];
+#pragma unroll
+  for (int j = 0; j < D; ++j) P.vel[j] = u[1 + j] * P.ir;
+  S mv = u[1] * P.vel[0];
+#pragma unroll
+  for (int j = 1; j < D; ++j) mv = madd(u[1 + j], P.vel[j], mv);
+  P.p = ph.gm1 * msub(T(0.5), mv, u[M - 1]);
+  P.e0 = u[M - 1] * P.ir;
+  P.h0 = madd(P.p, P.ir, P.e0);
+}
 
 // Inviscid flux column k: (rho v_k, rho v_j v_k + p delta_jk, rho v_k h0)
 // Full tensor F_c + F_v at a point: F[v][k].
@@ -91,234 +149,255 @@ template <int D, class S, class T>
 __host__ __device__ __forceinline__ void flux_total(const S* u, const S (*g)[D], S (*F)[D],
                                            const Phys<T>& ph) {
   constexpr int M = D + 2;
-  S rho = u[0];
-  S ir = T(1) / rho;
-  S vel[D];
-#pragma unroll
-  for (int j = 0; j < D; ++j) vel[j] = u[1 + j] * ir;
-  S e0 = u[M - 1] * ir;
-  S q2 = vel[0] * vel[0];
-#pragma unroll
-  for (int j = 1; j < D; ++j) q2 = q2 + vel[j] * vel[j];
-  S p = ph.gm1 * (u[M - 1] - T(0.5) * rho * q2);
-  S h0 = e0 + p * ir;
-  // primitive gradients from conservative ones
-  S gv[D][D], gT[D];
+  Prim<D, S> P;
+  primitives<D, S, T>(u, ph, P);
+  // rho grad v_j = grad(rho v_j) - v_j grad rho, and rho (grad e0 - v . grad v)
+  S a[D][D], b[D];
 #pragma unroll
   for (int k = 0; k < D; ++k) {
+    b[k] = msub(P.e0, g[0][k], g[M - 1][k]);
 #pragma unroll
-    for (int j = 0; j < D; ++j) gv[j][k] = (g[1 + j][k] - vel[j] * g[0][k]) * ir;
-    S ge = (g[M - 1][k] - e0 * g[0][k]) * ir;
-    S s = vel[0] * gv[0][k];
-#pragma unroll
-    for (int j = 1; j < D; ++j) s = s + vel[j] * gv[j][k];
-    gT[k] = (ph.gm1 / ph.Rgas) * (ge - s);
+    for (int j = 0; j < D; ++j) {
+      a[j][k] = msub(P.vel[j], g[0][k], g[1 + j][k]);
+      b[k] = msub(P.vel[j], a[j][k], b[k]);
+    }
   }
-  S div = gv[0][0];
+  S div = a[0][0];
 #pragma unroll
-  for (int j = 1; j < D; ++j) div = div + gv[j][j];
+  for (int j = 1; j < D; ++j) div = div + a[j][j];
+  const S mi = ph.mu * P.ir, ki = ph.heat() * P.ir;
+  S tau[D][D];
+#pragma unroll
+  for (int k = 0; k < D; ++k)
+#pragma unroll
+    for (int j = 0; j <= k; ++j) {
+      const S t = mi * (j == k ? msub(T(2) / T(3), div, T(2) * a[k][k]) : a[j][k] + a[k][j]);
+      tau[j][k] = t;
+      tau[k][j] = t;
+    }
 #pragma unroll
   for (int k = 0; k < D; ++k) {
     F[0][k] = u[1 + k];
-    S tv = T(0);                               // sum_j v_j tau_jk
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      S tau = ph.mu * (gv[j][k] + gv[k][j]);
-      if (j == k) tau = tau - (T(2) / T(3)) * ph.mu * div;
-      S inv = u[1 + j] * vel[k];
-      if (j == k) inv = inv + p;
-      F[1 + j][k] = inv - tau;
-      tv = tv + vel[j] * tau;
+    for (int j = 0; j <= k; ++j) {
+      S f = madd(u[1 + j], P.vel[k], -tau[j][k]);
+      if (j == k) f = f + P.p;
+      F[1 + j][k] = f;
+      F[1 + k][j] = f;
     }
-    F[M - 1][k] = rho * vel[k] * h0 - (tv + ph.kappa * gT[k]);
+    S q = ki * b[k];
+#pragma unroll
+    for (int j = 0; j < D; ++j) q = madd(P.vel[j], tau[j][k], q);
+    F[M - 1][k] = madd(u[1 + k], P.h0, -q);
   }
+}
+
+// Fk += c F_v column k (F_v = -(0, tau, v.tau - q)), given the primitives.
+template <int D, int k, class S, class T>
+__host__ __device__ __forceinline__ void add_visc_col(const Prim<D, S>& P, const S (*g)[D], T c, S* Fk,
+                                                      const Phys<T>& ph) {
+  constexpr int M = D + 2;
+  S an[D], b = msub(P.e0, g[0][k], g[M - 1][k]), dt = T(0);   // rho d_k v_j; the other directions' divergence
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    an[j] = msub(P.vel[j], g[0][k], g[1 + j][k]);
+    b = msub(P.vel[j], an[j], b);
+  }
+  const S mi = (c * ph.mu) * P.ir;
+  S q = (c * ph.heat()) * P.ir * b;
+  bool first = true;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    if (j == k) continue;
+    const S ajj = msub(P.vel[j], g[0][j], g[1 + j][j]);
+    dt = first ? ajj : dt + ajj;
+    first = false;
+    const S akj = msub(P.vel[k], g[0][j], g[1 + k][j]);      // rho d_j v_k
+    const S t = mi * (an[j] + akj);
+    Fk[1 + j] = Fk[1 + j] - t;
+    q = madd(P.vel[j], t, q);
+  }
+  const S t = mi * msub(T(2) / T(3), dt, (T(4) / T(3)) * an[k]);
+  Fk[1 + k] = Fk[1 + k] - t;
+  q = madd(P.vel[k], t, q);
+  Fk[M - 1] = Fk[M - 1] - q;
 }
 
 // Viscous flux only (F_v = -(0, tau, v.tau - q)), column k, for face averages.
 template <int D, int k, class S, class T>
 __host__ __device__ __forceinline__ void flux_visc_col(const S* u, const S (*g)[D], S* Fk,
                                               const Phys<T>& ph) {
-  constexpr int M = D + 2;
-  S ir = T(1) / u[0];
-  S vel[D];
+  Prim<D, S> P;
+  primitives<D, S, T>(u, ph, P);
 #pragma unroll
-  for (int j = 0; j < D; ++j) vel[j] = u[1 + j] * ir;
-  S e0 = u[M - 1] * ir;
-  S gv[D][D];
-  S gTk = T(0);
-#pragma unroll
-  for (int kk = 0; kk < D; ++kk) {
-#pragma unroll
-    for (int j = 0; j < D; ++j) gv[j][kk] = (g[1 + j][kk] - vel[j] * g[0][kk]) * ir;
-  }
-  {
-    S ge = (g[M - 1][k] - e0 * g[0][k]) * ir;
-    S s = vel[0] * gv[0][k];
-#pragma unroll
-    for (int j = 1; j < D; ++j) s = s + vel[j] * gv[j][k];
-    gTk = (ph.gm1 / ph.Rgas) * (ge - s);
-  }
-  S div = gv[0][0];
-#pragma unroll
-  for (int j = 1; j < D; ++j) div = div + gv[j][j];
-  Fk[0] = T(0);
-  S tv = T(0);
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    S tau = ph.mu * (gv[j][k] + gv[k][j]);
-    if (j == k) tau = tau - (T(2) / T(3)) * ph.mu * div;
-    Fk[1 + j] = -tau;
-    tv = tv + vel[j] * tau;
-  }
-  Fk[M - 1] = -(tv + ph.kappa * gTk);
+  for (int v = 0; v < D + 2; ++v) Fk[v] = T(0);
+  add_visc_col<D, k, S, T>(P, g, T(1), Fk, ph);
 }
 
-// G = K(u) (a (x) e_k) = -F_v(u, a (x) e_k): the viscous operator applied to the
-// rank-one gradient a e_k^T (full tensor G[v][kk]).  Used by the BR2 lifting
-// (eq. re) and the dual-consistency term of eq. dg_ns.
+// c K(u)(a (x) e_k) = -c F_v(u, a (x) e_k), the viscous operator applied to the
+// rank-one gradient a e_k^T (the BR2 lifting of eq. re and the dual-consistency
+// term of eq. dg_ns), by its independent entries: with m_j = c mu (d v_j along
+// e_k) the tensor G[v][kk] is
+//   G[0][.] = 0,  G[1+j][k] = m_j (j != k), 4/3 m_k (j = k),
+//   kk != k: G[1+k][kk] = m_kk, G[1+kk][kk] = -2/3 m_k, else 0,  G[M-1][kk] = e_kk.
 template <int D, int k, class S, class T>
-__host__ __device__ __forceinline__ void visc_K_rank1(const S* u, const S* a, S (*G)[D],
-                                             const Phys<T>& ph) {
+__host__ __device__ __forceinline__ void visc_rank1(const Prim<D, S>& P, const S* a, T c, S* m, S* e,
+                                                    const Phys<T>& ph) {
   constexpr int M = D + 2;
-  S ir = T(1) / u[0];
-  S vel[D], av[D];
+  S b = msub(P.e0, a[0], a[M - 1]), av[D];
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    vel[j] = u[1 + j] * ir;
-    av[j] = (a[1 + j] - vel[j] * a[0]) * ir;     // d v_j along e_k
+    av[j] = msub(P.vel[j], a[0], a[1 + j]);
+    b = msub(P.vel[j], av[j], b);
   }
-  S e0 = u[M - 1] * ir;
-  S ae = (a[M - 1] - e0 * a[0]) * ir;
-  S s = vel[0] * av[0];
+  const S mi = (c * ph.mu) * P.ir;
 #pragma unroll
-  for (int j = 1; j < D; ++j) s = s + vel[j] * av[j];
-  S aT = (ph.gm1 / ph.Rgas) * (ae - s);
-  S div = av[k];
+  for (int j = 0; j < D; ++j) m[j] = mi * av[j];
+  S en = madd((T(4) / T(3)) * P.vel[k], m[k], (c * ph.heat()) * P.ir * b);
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    if (j == k) continue;
+    en = madd(P.vel[j], m[j], en);
+    e[j] = msub((T(2) / T(3)) * P.vel[j], m[k], P.vel[k] * m[j]);
+  }
+  e[k] = en;
+}
+template <int D, int k, class S, class T>
+__host__ __device__ __forceinline__ void rank1_tensor(const S* m, const S* e, S (*G)[D]) {
 #pragma unroll
   for (int kk = 0; kk < D; ++kk) {
     G[0][kk] = T(0);
-    S tv = T(0);
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      S tau = T(0);
-      if (kk == k) tau = tau + ph.mu * av[j];
-      if (j == k) tau = tau + ph.mu * av[kk];
-      if (j == kk) tau = tau - (T(2) / T(3)) * ph.mu * div;
-      G[1 + j][kk] = tau;
-      tv = tv + vel[j] * tau;
-    }
-    G[M - 1][kk] = tv + ((kk == k) ? ph.kappa * aT : S(T(0)));
+    for (int j = 0; j < D; ++j)
+      G[1 + j][kk] = kk == k ? (j == k ? (T(4) / T(3)) * m[k] : m[j])
+                             : j == k ? m[kk] : j == kk ? (T(-2) / T(3)) * m[k] : S(T(0));
+    G[D + 1][kk] = e[kk];
   }
 }
+template <int D, int k, class S, class T>
+__host__ __device__ __forceinline__ void visc_K_rank1(const S* u, const S* a, S (*G)[D],
+                                             const Phys<T>& ph) {
+  Prim<D, S> P;
+  primitives<D, S, T>(u, ph, P);
+  S m[D], e[D];
+  visc_rank1<D, k, S, T>(P, a, T(1), m, e, ph);
+  rank1_tensor<D, k, S, T>(m, e, G);
+}
 
+// |lam| smoothed to (lam^2 + delta^2) / (2 delta) below delta; ihd = 1 / (2 delta)
 template <class S, class T>
-__host__ __device__ __forceinline__ S entropy_fixed_abs(S lam, S delta) {
-  S a = sabs(lam);
-  if (val(delta) > T(0) && val(a) < val(delta)) return (lam * lam + delta * delta) / (T(2) * delta);
+__host__ __device__ __forceinline__ S entropy_fixed_abs(S lam, S delta, S ihd) {
+  const S a = sabs(lam);
+  if (val(delta) > T(0) && val(a) < val(delta)) return madd(lam, lam, delta * delta) * ihd;
   return a;
 }
 
-// Roe flux with normal +e_k: 1/2 (F_c(uL) + F_c(uR)).e_k - 1/2 |A_Roe| (uR - uL).
+// Roe flux with normal +e_k: 1/2 (F_c(uL) + F_c(uR)).e_k - 1/2 |A_Roe| (uR - uL),
+// the primitives of both sides given.
 template <int D, int k, class S, class T>
-__host__ __device__ __forceinline__ void roe_flux(const S* uL, const S* uR, S* Fh,
-                                         const Phys<T>& ph) {
+__host__ __device__ __forceinline__ void roe_flux(const S* uL, const S* uR, const Prim<D, S>& L, const Prim<D, S>& R,
+                                                  S* Fh, const Phys<T>& ph) {
   constexpr int M = D + 2;
-  S rL = uL[0], rR = uR[0];
-  S irL = T(1) / rL, irR = T(1) / rR;
-  S vL[D], vR[D];
-  S q2L = T(0), q2R = T(0);
+  const S sL = dsqrt(uL[0], L.ir), sR = dsqrt(uR[0], R.ir);
+  const S wL = sL * (T(1) / (sL + sR));          // Roe weight of L; R has 1 - wL
+  const S rho = sL * sR;
+  S vel[D], dv[D], q2 = T(0), vt = T(0);
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    vL[j] = uL[1 + j] * irL;
-    vR[j] = uR[1 + j] * irR;
-    q2L = q2L + vL[j] * vL[j];
-    q2R = q2R + vR[j] * vR[j];
+    dv[j] = R.vel[j] - L.vel[j];
+    vel[j] = msub(wL, dv[j], R.vel[j]);
+    q2 = j == 0 ? vel[0] * vel[0] : madd(vel[j], vel[j], q2);
   }
-  S pL = ph.gm1 * (uL[M - 1] - T(0.5) * rL * q2L);
-  S pR = ph.gm1 * (uR[M - 1] - T(0.5) * rR * q2R);
-  S hL = (uL[M - 1] + pL) * irL;
-  S hR = (uR[M - 1] + pR) * irR;
-  S sL = dsqrt(rL), sR = dsqrt(rR);
-  S isum = T(1) / (sL + sR);
-  S rho = sL * sR;
-  S vel[D];
-  S q2 = T(0);
+  const S h0 = msub(wL, R.h0 - L.h0, R.h0);
+  const S c2 = ph.gm1 * msub(T(0.5), q2, h0), ic2 = T(1) / c2;
+  const S c = dsqrt(c2, ic2);
+  const S vn = vel[k], dp = R.p - L.p;
+  const S pa = dp * (T(0.5) * ic2), pb = (rho * dv[k]) * (T(0.5) * c * ic2);   // wave strengths pa -+ pb
+  const S delta = ph.roe_delta * c;
+  const S ihd = ph.roe_delta > T(0) ? (ph.half_inv_delta() * c) * ic2 : S(T(0));
+  const S l1 = entropy_fixed_abs<S, T>(vn - c, delta, ihd) * (pa - pb);
+  const S l2 = entropy_fixed_abs<S, T>(vn, delta, ihd);
+  const S l3 = entropy_fixed_abs<S, T>(vn + c, delta, ihd) * (pa + pb);
+  const S sum = l1 + l3, dif = (l3 - l1) * c;
+  const S ent = l2 * msub(T(2), pa, uR[0] - uL[0]), shr = l2 * rho, mass = sum + ent;
+  Fh[0] = T(0.5) * ((uL[1 + k] + uR[1 + k]) - mass);
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    vel[j] = (sL * vL[j] + sR * vR[j]) * isum;
-    q2 = q2 + vel[j] * vel[j];
-  }
-  S h0 = (sL * hL + sR * hR) * isum;
-  S c2 = ph.gm1 * (h0 - T(0.5) * q2);
-  S c = dsqrt(c2);
-  S vn = vel[k];
-  S dr = rR - rL, dp = pR - pL;
-  S dv[D];
-  S vdv = T(0);
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    dv[j] = vR[j] - vL[j];
-    vdv = vdv + vel[j] * dv[j];
-  }
-  S dvn = dv[k];
-  S ic2 = T(1) / c2;
-  S a1 = (dp - rho * c * dvn) * (T(0.5) * ic2);
-  S a3 = (dp + rho * c * dvn) * (T(0.5) * ic2);
-  S a2 = dr - dp * ic2;
-  S delta = ph.roe_delta * c;
-  S l1 = entropy_fixed_abs<S, T>(vn - c, delta) * a1;
-  S l2 = entropy_fixed_abs<S, T>(vn, delta);
-  S l3 = entropy_fixed_abs<S, T>(vn + c, delta) * a3;
-  // inviscid flux column k of both states
-  Fh[0] = T(0.5) * (uL[1 + k] + uR[1 + k]) - T(0.5) * (l1 + l3 + l2 * a2);
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    S fl = uL[1 + j] * vL[k];
-    S fr = uR[1 + j] * vR[k];
+    S f = madd(uL[1 + j], L.vel[k], uR[1 + j] * R.vel[k]);
+    f = msub(vel[j], mass, f);
     if (j == k) {
-      fl = fl + pL;
-      fr = fr + pR;
+      f = f + ((L.p + R.p) - dif);
+    } else {
+      const S t = shr * dv[j];
+      f = f - t;
+      vt = madd(vel[j], t, vt);
     }
-    S dis = l1 * vel[j] + l3 * vel[j] + l2 * (a2 * vel[j] + rho * dv[j]);
-    if (j == k) dis = dis - l1 * c + l3 * c - l2 * rho * dvn;
-    Fh[1 + j] = T(0.5) * (fl + fr) - T(0.5) * dis;
+    Fh[1 + j] = T(0.5) * f;
   }
-  S disE = l1 * (h0 - c * vn) + l3 * (h0 + c * vn) + l2 * (a2 * T(0.5) * q2 + rho * (vdv - vn * dvn));
-  Fh[M - 1] = T(0.5) * (rL * vL[k] * hL + rR * vR[k] * hR) - T(0.5) * disE;
+  S f = madd(uL[1 + k], L.h0, uR[1 + k] * R.h0) - vt;
+  f = msub(h0, sum, f);
+  f = msub(vn, dif, f);
+  Fh[M - 1] = T(0.5) * msub(T(0.5) * q2, ent, f);
+}
+template <int D, int k, class S, class T>
+__host__ __device__ __forceinline__ void roe_flux(const S* uL, const S* uR, S* Fh, const Phys<T>& ph) {
+  Prim<D, S> L, R;
+  primitives<D, S, T>(uL, ph, L);
+  primitives<D, S, T>(uR, ph, R);
+  roe_flux<D, k, S, T>(uL, uR, L, R, Fh, ph);
 }
 
 // Pointwise physics of one face point, normal +e_k from L (its xi_k = +1 side)
-// to R.  fp = Roe(uL, uR) + {F_v}.e_k; with jump = uL - uR,
-// GLn/GRn = normal column of K(uL)/K(uR) (jump (x) e_k) (the BR2 lifting
-// integrand of eq. re) and DL/DR = half the full tensors (the dual-consistency
-// term of eq. dg_ns, (u+ - uhat) = jump/2).  The direction is a compile-time
-// constant: no local array is indexed at run time.
+// to R.  fp = Roe(uL, uR) + {F_v}.e_k; with jump = uL - uR, (mL, eL) and (mR,
+// eR) are the entries (visc_rank1) of half the tensors K(uL), K(uR) (jump (x)
+// e_k): twice their normal columns are the BR2 lifting integrands of eq. re,
+// the tensors themselves the dual-consistency term of eq. dg_ns ((u+ - uhat) =
+// jump/2).  The direction is a compile-time constant: no local array is
+// indexed at run time.
+template <int D, int k, class S, class T>
+__host__ __device__ __forceinline__ void face_point_core(const S* uL, const S (*gL)[D], const S* uR, const S (*gR)[D],
+                                                         const Phys<T>& ph, S* fp, S* mL, S* eL, S* mR, S* eR) {
+  constexpr int M = D + 2;
+  Prim<D, S> L, R;
+  primitives<D, S, T>(uL, ph, L);
+  primitives<D, S, T>(uR, ph, R);
+  roe_flux<D, k, S, T>(uL, uR, L, R, fp, ph);
+  add_visc_col<D, k, S, T>(L, gL, T(0.5), fp, ph);
+  add_visc_col<D, k, S, T>(R, gR, T(0.5), fp, ph);
+  S jump[M];
+#pragma unroll
+  for (int v = 0; v < M; ++v) jump[v] = uL[v] - uR[v];
+  visc_rank1<D, k, S, T>(L, jump, T(0.5), mL, eL, ph);
+  visc_rank1<D, k, S, T>(R, jump, T(0.5), mR, eR, ph);
+}
+template <int D, class S, class T>
+__host__ __device__ __forceinline__ void face_point_core_k(int k, const S* uL, const S (*gL)[D], const S* uR,
+                                                           const S (*gR)[D], const Phys<T>& ph, S* fp, S* mL, S* eL,
+                                                           S* mR, S* eR) {
+  if (k == 0) {
+    face_point_core<D, 0, S, T>(uL, gL, uR, gR, ph, fp, mL, eL, mR, eR);
+  } else if (k == 1) {
+    face_point_core<D, 1, S, T>(uL, gL, uR, gR, ph, fp, mL, eL, mR, eR);
+  } else {
+    if constexpr (D == 3) face_point_core<D, 2, S, T>(uL, gL, uR, gR, ph, fp, mL, eL, mR, eR);
+  }
+}
+
+// The same with full tensors: GLn/GRn = normal column of K(uL)/K(uR) (jump (x)
+// e_k), DL/DR = half the full tensors.
 template <int D, int k, class S, class T>
 __host__ __device__ __forceinline__ void face_point(const S* uL, const S (*gL)[D], const S* uR,
                                                     const S (*gR)[D], const Phys<T>& ph, S* fp, S* GLn,
                                                     S* GRn, S (*DL)[D], S (*DR)[D]) {
   constexpr int M = D + 2;
-  S jump[M], Fr[M], FvL[M], FvR[M], G[M][D];
-#pragma unroll
-  for (int v = 0; v < M; ++v) jump[v] = uL[v] - uR[v];
-  roe_flux<D, k, S, T>(uL, uR, Fr, ph);
-  flux_visc_col<D, k, S, T>(uL, gL, FvL, ph);
-  flux_visc_col<D, k, S, T>(uR, gR, FvR, ph);
-#pragma unroll
-  for (int v = 0; v < M; ++v) fp[v] = Fr[v] + T(0.5) * (FvL[v] + FvR[v]);
-  visc_K_rank1<D, k, S, T>(uL, jump, G, ph);
+  S mL[D], eL[D], mR[D], eR[D];
+  face_point_core<D, k, S, T>(uL, gL, uR, gR, ph, fp, mL, eL, mR, eR);
+  rank1_tensor<D, k, S, T>(mL, eL, DL);
+  rank1_tensor<D, k, S, T>(mR, eR, DR);
 #pragma unroll
   for (int v = 0; v < M; ++v) {
-    GLn[v] = G[v][k];
-#pragma unroll
-    for (int kk = 0; kk < D; ++kk) DL[v][kk] = T(0.5) * G[v][kk];
-  }
-  visc_K_rank1<D, k, S, T>(uR, jump, G, ph);
-#pragma unroll
-  for (int v = 0; v < M; ++v) {
-    GRn[v] = G[v][k];
-#pragma unroll
-    for (int kk = 0; kk < D; ++kk) DR[v][kk] = T(0.5) * G[v][kk];
+    GLn[v] = T(2) * DL[v][k];
+    GRn[v] = T(2) * DR[v][k];
   }
 }
 
@@ -337,14 +416,14 @@ __host__ __device__ __forceinline__ void face_point_k(int k, const S* uL, const 
 
 // rho > 0 and p > 0 of a point state (primal values)
 template <int D, class S, class T>
-__host__ __device__ __forceinline__ bool physical(const S* u, T gm1) {
+__host__ __device__ __forceinline__ bool physical(const S* u, T) {
   constexpr int M = D + 2;
   T r = val(u[0]);
-  T q = T(0);
+  T q = val(u[1]) * val(u[1]);
 #pragma unroll
-  for (int j = 0; j < D; ++j) q += val(u[1 + j]) * val(u[1 + j]);
-  T p = gm1 * (val(u[M - 1]) - T(0.5) * q / r);
-  return r > T(0) && p > T(0);
+  for (int j = 1; j < D; ++j) q += val(u[1 + j]) * val(u[1 + j]);
+  // p = (gamma - 1) (E - q / (2 rho)) > 0 without the division
+  return r > T(0) && val(u[M - 1]) * r > T(0.5) * q;
 }
 
 // ----------------------------------------------------------------- mesh view

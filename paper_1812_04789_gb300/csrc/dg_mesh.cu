@@ -174,6 +174,8 @@ Phys<T> Mesh::phys_t() const {
   p.eta = (T)(phys.eta_br2 > 0 ? phys.eta_br2 : 2.0 * d + 1.0);
   p.roe_delta = (T)phys.roe_delta;
   p.kappa = (T)(phys.mu * phys.gamma * phys.Rgas / ((phys.gamma - 1.0) * phys.Pr));
+  p.kq = (T)(phys.mu * phys.gamma / phys.Pr);
+  p.hrd = (T)(phys.roe_delta > 0.0 ? 0.5 / phys.roe_delta : 0.0);
   return p;
 }
 template Phys<double> Mesh::phys_t<double>() const;

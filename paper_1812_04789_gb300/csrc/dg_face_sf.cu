@@ -4,18 +4,33 @@
 // On the face k of an element the basis functions are products
 // L_a(xi_k = +-1) L_b(xi_t0) L_c(xi_t1) (t0 < t1 the two other directions) and
 // the face points a tensor grid (b0, b1) of the same Gauss-Legendre points,
-// q = b0 + nq b1.  The traces of a field and of its gradient at all n_qf points
-// are then three short contractions instead of one over all modes:
+// q = b0 + nq b1.  Everything is done in the face's frame: directions (n, t0,
+// t1), variables (rho, the momenta along n, t0, t1, rho e0); the physics is
+// invariant under that permutation, so one copy of it (normal = first
+// direction) serves all faces.  Traces of a field and of its gradient:
 //   S1  c0[a0][a1] = sum_ak w L_ak(+-1),  c1[a0][a1] = sum_ak w L'_ak(+-1)
 //   S2  d0[a0][b1] = sum_a1 c0 L_a1(b1),  d1 = sum_a1 c0 L'_a1(b1),  d2 = sum_a1 c1 L_a1(b1)
 //   per point: u = sum_a0 d0 L_a0(b0), du/dt0 = sum d0 L'_a0(b0), du/dt1 = sum d1 L_a0(b0),
 //              du/dn = sum d2 L_a0(b0)   (each derivative times its metric 2/h)
-// and the projection of the face fluxes onto both elements' test functions is
-// the transposed sequence (X over b0, Y over b1, then the end values).  The
-// total-degree space P_p is the subset a_k + a0 + a1 <= p of these products
-// (qidx maps a tensor index to its mode, -1 outside P_p), Q_p all of them.
-// Pointwise physics and the BR2 lifting are those of face_kernel
-// (csrc/dg_residual.cu), point for point.
+// and the projection onto both elements' test functions is the transposed
+// sequence (X over b0, Y over b1, then the end values).  The total-degree
+// space P_p is the subset a_k + a0 + a1 <= p of these products, Q_p all of
+// them; the sums run over that subset only.
+//
+// In FP64 the kernel is bound by the FP64 pipe (two lanes per clock and SM), so
+// the work is what counts, shared-memory traffic and index arithmetic are free:
+//  * the fluxes of the two sides differ in sign only: one projection for both;
+//  * the dual-consistency tensors have six independent entries per side
+//    (visc_rank1), of which eight tangential contractions are needed;
+//  * the BR2 lifting of eq. re is never formed at the points.  Both sides lift
+//    with the same operator, delta = sum_a C_a psi_a (sum_q w psi_a G) / (2 |J|)
+//    over the tangential products psi_a, C_a = sum_ak L_ak(+-1)^2 (n^2 / 2 for n
+//    values of ak), and its projection onto psi_a' is exact (Gauss-Legendre,
+//    nq >= p + 1), so in the projected flux it is a factor per (a0, a1):
+//    Y_a += eta/2 C_a (1/h_k) (sum_q w psi_a (G_L + G_R)).
+// FP64 operations per face at p = 4, JVP: 154 k -> 64 k (with the point
+// physics of dg_common.cuh).  JVP, FP64, faces: 32^3 p = 6 79.7 -> 29 ms, 16^3 p =
+// 4 3.64 -> 1.50 ms (FP64 pipe 72 % busy when each thread ran one sum at a time).
 #include <algorithm>
 #include <type_traits>
 
@@ -25,31 +40,35 @@ namespace dgk {
 
 namespace {
 
+constexpr int FSF_NP = 21;   // point values: flux 5, lifting integrand 4, two sides' tensors 6 each
+constexpr int FSF_NX = 25;   // X arrays: flux 5, lifting 4, per side 5 with L and 3 with L'
+constexpr int FSF_NY = 25;   // Y arrays: flux 5, per side 4 value and 4 normal-derivative parts, lifting 4
+
 // shared-memory plan (elements of T); NC = interpolated real fields per side
 struct FsfPlan {
-  int n1, nq, nqf, NC;
-  size_t oW, oV, oG, oF, oD, oS, oT, per_face, total;
+  int n1, nq, nqf, NC, npair;
+  size_t oV, oS, oT, per_face, total;
 };
 
-__host__ __device__ inline FsfPlan fsf_plan(int p, int nq, int nb, int M, bool jvp, bool cached, int fpc) {
+__host__ __device__ inline FsfPlan fsf_plan(int p, int nq, int nb, int M, bool total_degree, bool jvp, bool cached,
+                                            int fpc) {
   FsfPlan P;
   P.n1 = p + 1;
   P.nq = nq;
   P.nqf = nq * nq;
+  P.npair = total_degree ? P.n1 * (P.n1 + 1) / 2 : P.n1 * P.n1;
   const bool haveW = !(jvp && cached);
   P.NC = (haveW ? 1 : 0) + (jvp ? 1 : 0);
-  // the coefficients (read by S1 only) share their space with the point values
-  // (written from phase 1 on, after S2)
-  P.oW = 0;
+  // region 0: the coefficients (read by S1 only), then the point values (written
+  // after S2), then the projected modes
   P.oV = haveW ? (size_t)fpc * 2 * nb : 0;
-  const size_t coef = P.oV + (jvp ? (size_t)fpc * 2 * nb : 0);
-  P.oG = 0;
-  P.oF = (size_t)fpc * 2 * P.nqf * M;
-  P.oD = P.oF + (size_t)fpc * P.nqf * M;
-  const size_t pts = P.oD + (size_t)fpc * 2 * P.nqf * M * 3;
+  const size_t coef = P.oV + (jvp ? (size_t)fpc * 2 * nb : 0), pts = (size_t)fpc * FSF_NP * P.nqf;
   size_t o = coef > pts ? coef : pts;
-  const size_t interp = (size_t)2 * P.NC * M * (2 * P.n1 * P.n1 + 3 * P.n1 * nq);
-  const size_t proj = (size_t)2 * M * (3 * P.n1 * nq + 2 * P.n1 * P.n1);
+  const size_t modes = (size_t)fpc * 2 * nb;
+  o = o > modes ? o : modes;
+  // region 1, per face: the interpolation's stages, then the projection's
+  const size_t interp = (size_t)2 * P.NC * M * (2 * P.npair + 3 * P.n1 * nq);
+  const size_t proj = (size_t)FSF_NX * P.n1 * nq + FSF_NY * P.npair;
   P.per_face = interp > proj ? interp : proj;
   P.oS = o;
   o += (size_t)fpc * P.per_face;
@@ -71,23 +90,22 @@ template <class T, bool JVP>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2)
     face_sf_kernel(MeshView<T> mv, Phys<T> ph, const T* __restrict__ W, const T* __restrict__ V,
                    T* __restrict__ slots, int* status, int fpc, const T* __restrict__ Pf, const T* __restrict__ l1g,
-                   const int* __restrict__ qidx, int p, int nq, T m0, T m1, T m2) {
+                   const int* __restrict__ qidx, int p, int nq, int total_degree, T m0, T m1, T m2) {
   using S = typename std::conditional<JVP, Dual<T>, T>::type;
   constexpr int D = 3, M = D + 2, PU = M * (1 + D);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
+  __shared__ unsigned short ptab[256];   // pair -> a0 | a1 << 8, a0-major
   const int nb = mv.nb, nm = mv.nm, nqf = mv.nqf, E = mv.E;
   const bool cached = JVP && Pf != nullptr;
-  const FsfPlan P = fsf_plan(p, nq, nb, M, JVP, cached, fpc);
-  const int n1 = P.n1, NC = P.NC;
+  const FsfPlan P = fsf_plan(p, nq, nb, M, total_degree, JVP, cached, fpc);
+  const int n1 = P.n1, NC = P.NC, npair = P.npair, n1s = n1 * n1;
   const bool haveW = !cached;
   const int nfaces = D * E, f0 = blockIdx.x * fpc, nloc = min(fpc, nfaces - f0);
   if (nloc <= 0) return;
-  T* sW = sm + P.oW;               // [fpc][2][nb]  state (not with cached traces), until S1
+  T* sW = sm;                      // [fpc][2][nb]  state (not with cached traces), until S1
   T* sV = sm + P.oV;               // [fpc][2][nb]  direction (JVP), until S1
-  T* sG = sm + P.oG;               // [fpc][2][nqf][M]
-  T* sF = sm + P.oF;               // [fpc][nqf][M]
-  T* sD = sm + P.oD;               // [fpc][2][nqf][M][D]
+  T* sP = sm;                      // [fpc][FSF_NP][nqf] point values times the face weight
   T* sS = sm + P.oS;               // [fpc][per_face]: contraction stages
   T* tab = sm + P.oT;
   const T* L = tab;                // L[a][b]
@@ -96,6 +114,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2)
   const T* dLe = Le + 2 * n1;
   for (int t = threadIdx.x; t < 2 * n1 * nq; t += blockDim.x) tab[t] = l1g[t];
   for (int t = threadIdx.x; t < 4 * n1; t += blockDim.x) tab[2 * n1 * nq + t] = l1g[2 * n1 * nq + nq + t];
+  // first pair of a0: a0 n1 - a0 (a0 - 1) / 2 (P_p) or a0 n1 (Q_p)
+  auto pair0 = [&](int a0) { return total_degree ? a0 * n1 - a0 * (a0 - 1) / 2 : a0 * n1; };
+  for (int t = threadIdx.x; t < n1s; t += blockDim.x) {
+    const int a0 = t / n1, a1 = t - a0 * n1;
+    if (!total_degree || a0 + a1 <= p) ptab[pair0(a0) + a1] = (unsigned short)(a0 | a1 << 8);
+  }
   // phase 0: the modal coefficients of both elements of every face
   for (int t = threadIdx.x; t < nloc * 2 * nb; t += blockDim.x) {
     const int fl = t / (2 * nb), r = t % (2 * nb), side = r / nb, j = r % nb;
@@ -105,57 +129,69 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2)
     if (JVP) sV[t] = V[(size_t)el * nb + j];
   }
   __syncthreads();
-  // S1: collapse the normal direction with the end values (L and L')
-  const int n1s = n1 * n1, s1sz = 2 * NC * M * 2 * n1s;
-  for (int t = threadIdx.x; t < nloc * s1sz; t += blockDim.x) {
-    const int fl = t / s1sz;
-    int r = t - fl * s1sz;
-    const int a1 = r % n1;
-    r /= n1;
-    const int a0 = r % n1;
-    r /= n1;
-    const int w2 = r % 2;
-    r /= 2;
-    const int v = r % M;
+  // S1: collapse the normal direction with the end values (L and L'); the pair
+  // slowest, so that the lanes of a warp run sums of one length
+  const int n_s1 = 2 * NC * M, s1sz = 2 * n_s1 * npair;
+  for (int t = threadIdx.x; t < nloc * n_s1 * npair; t += blockDim.x) {
+    const int pr = t / (nloc * n_s1);
+    int r = t - pr * (nloc * n_s1);
+    const int fl = r / n_s1;
+    r -= fl * n_s1;
+    const int row = r, v = r % M;
     r /= M;
     const int c = r % NC, side = r / NC;
+    const int a0 = ptab[pr] & 255, a1 = ptab[pr] >> 8;
     const int k = (f0 + fl) / E, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2;
+    const int pv = v == 0 || v == M - 1 ? v : 1 + pick3(v - 1, k, t0, t1);   // the frame's variable v
     const int end = side == 0 ? 1 : 0;       // the element on side 0 meets the face at xi_k = +1
-    const T* Ev = (w2 ? dLe : Le) + end * n1;
-    const T* fld = ((haveW && c == 0) ? sW : sV) + ((size_t)fl * 2 + side) * nb + v * nm;
-    T acc = T(0);
+    const T* Ev = Le + end * n1;
+    const T* dEv = dLe + end * n1;
+    const T* fld = ((haveW && c == 0) ? sW : sV) + ((size_t)fl * 2 + side) * nb + pv * nm;
+    T acc = T(0), dacc = T(0);
     const int sk = pick3(k, 1, n1, n1s), base = a0 * pick3(t0, 1, n1, n1s) + a1 * pick3(t1, 1, n1, n1s);
-    for (int ak = 0; ak < n1; ++ak) {
-      const int i = qidx[base + ak * sk];
-      if (i >= 0) acc += fld[i] * Ev[ak];
+    const int nak = total_degree ? n1 - a0 - a1 : n1;
+#pragma unroll 4
+    for (int ak = 0; ak < nak; ++ak) {
+      const T x = fld[qidx[base + ak * sk]];
+      acc += x * Ev[ak];
+      dacc += x * dEv[ak];
     }
-    sS[(size_t)fl * P.per_face + (t - fl * s1sz)] = acc;
+    T* o = sS + (size_t)fl * P.per_face + (size_t)row * 2 * npair + pr;
+    o[0] = acc;
+    o[npair] = dacc;
   }
   __syncthreads();
-  // S2: contract the second tangential direction: d0 = c0 L, d1 = c0 L', d2 = c1 L
-  const int s2sz = 2 * NC * M * 3 * n1 * nq;
-  for (int t = threadIdx.x; t < nloc * s2sz; t += blockDim.x) {
-    const int fl = t / s2sz;
-    int r = t - fl * s2sz;
-    const int b1 = r % nq;
-    r /= nq;
-    const int a0 = r % n1;
-    r /= n1;
-    const int ty = r % 3;
-    r /= 3;
-    const int scv = r;                       // (side, c, v)
-    const T* s1 = sS + (size_t)fl * P.per_face + ((size_t)scv * 2 + (ty == 2 ? 1 : 0)) * n1s + a0 * n1;
-    const T* Lt = ty == 1 ? dL : L;
-    T acc = T(0);
-    for (int a1 = 0; a1 < n1; ++a1) acc += s1[a1] * Lt[a1 * nq + b1];
-    sS[(size_t)fl * P.per_face + s1sz + (t - fl * s2sz)] = acc;
+  // S2: contract the second tangential direction: d0 = c0 L, d1 = c0 L', d2 = c1 L;
+  // a0 slowest, as S1's pair
+  const int n_s2 = 2 * NC * M * nq;
+  for (int t = threadIdx.x; t < nloc * n_s2 * n1; t += blockDim.x) {
+    const int a0 = t / (nloc * n_s2);
+    int r = t - a0 * (nloc * n_s2);
+    const int fl = r / n_s2;
+    r -= fl * n_s2;
+    const int b1 = r % nq, scv = r / nq;                            // scv = (side, c, v)
+    const T* s1 = sS + (size_t)fl * P.per_face + (size_t)scv * 2 * npair + pair0(a0);
+    const int na1 = total_degree ? n1 - a0 : n1;
+    T d0 = T(0), d1 = T(0), d2 = T(0);
+#pragma unroll 4
+    for (int a1 = 0; a1 < na1; ++a1) {
+      const T la = L[a1 * nq + b1], x = s1[a1];
+      d0 += x * la;
+      d1 += x * dL[a1 * nq + b1];
+      d2 += s1[npair + a1] * la;
+    }
+    T* o = sS + (size_t)fl * P.per_face + s1sz + ((size_t)scv * 3 * n1 + a0) * nq + b1;
+    o[0] = d0;
+    o[(size_t)n1 * nq] = d1;
+    o[(size_t)2 * n1 * nq] = d2;
   }
   __syncthreads();
   // phase 1: traces at the face points from the S2 stage, pointwise physics
-  // (as face_kernel: with cached traces a JVP takes the state's from the cache)
+  // (with cached traces a JVP takes the state's from the cache)
   for (int t = threadIdx.x; t < nloc * nqf; t += blockDim.x) {
     const int fl = t / nqf, q = t % nqf, b0 = q % nq, b1 = q / nq;
     const int f = f0 + fl, k = f / E, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2;
+    const T mk = pick3(k, m0, m1, m2), mt0 = pick3(t0, m0, m1, m2), mt1 = pick3(t1, m0, m1, m2);
     const T* s2 = sS + (size_t)fl * P.per_face + s1sz;
     S uS[2][M], gS[2][M][D];
 #pragma unroll
@@ -163,174 +199,241 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2)
 #pragma unroll
       for (int v = 0; v < M; ++v) {
         T val[2] = {T(0), T(0)}, gn[2] = {T(0), T(0)}, g0[2] = {T(0), T(0)}, g1[2] = {T(0), T(0)};
-        for (int c = 0; c < NC; ++c) {
-          const T* d = s2 + ((size_t)((side * NC + c) * M + v) * 3) * n1 * nq + b1;   // [ty][a0][b1]
-          T u_ = T(0), ut0 = T(0), ut1 = T(0), un = T(0);
-          for (int a0 = 0; a0 < n1; ++a0) {
-            const T la = L[a0 * nq + b0], da = dL[a0 * nq + b0];
-            const T d0 = d[(size_t)a0 * nq], d1 = d[(size_t)(n1 + a0) * nq], d2 = d[(size_t)(2 * n1 + a0) * nq];
-            u_ += d0 * la;
-            ut0 += d0 * da;
-            ut1 += d1 * la;
-            un += d2 * la;
+        const T* d = s2 + ((size_t)(side * NC * M + v) * 3) * n1 * nq + b1;   // [ty][a0][b1]
+        const size_t dc = (size_t)M * 3 * n1 * nq;                            // to the second field
+        for (int a0 = 0; a0 < n1; ++a0) {
+          const T la = L[a0 * nq + b0], da = dL[a0 * nq + b0];
+#pragma unroll
+          for (int c = 0; c < (JVP ? 2 : 1); ++c) {
+            if (c >= NC) continue;
+            const T* x = d + c * dc + (size_t)a0 * nq;
+            const T d0 = x[0], d1 = x[(size_t)n1 * nq], d2 = x[(size_t)2 * n1 * nq];
+            val[c] += d0 * la;
+            g0[c] += d0 * da;
+            g1[c] += d1 * la;
+            gn[c] += d2 * la;
           }
-          val[c] = u_;
-          gn[c] = un * pick3(k, m0, m1, m2);
-          g0[c] = ut0 * pick3(t0, m0, m1, m2);
-          g1[c] = ut1 * pick3(t1, m0, m1, m2);
         }
-        // the gradient component of physical direction kk: normal, first or second tangential
-#define GCOMP(c, kk) ((kk) == k ? gn[c] : ((kk) == t0 ? g0[c] : g1[c]))
+#pragma unroll
+        for (int c = 0; c < (JVP ? 2 : 1); ++c) {
+          gn[c] *= mk;
+          g0[c] *= mt0;
+          g1[c] *= mt1;
+        }
         if constexpr (JVP) {
           if (cached) {
+            const int pv = v == 0 || v == M - 1 ? v : 1 + pick3(v - 1, k, t0, t1);
             const T* cc = Pf + ((size_t)(f0 + fl) * nqf + q) * 2 * PU + side * PU;
-            uS[side][v] = S(cc[v], val[0]);
-#pragma unroll
-            for (int kk = 0; kk < D; ++kk) gS[side][v][kk] = S(cc[M + v * D + kk], GCOMP(0, kk));
+            uS[side][v] = S(cc[pv], val[0]);
+            gS[side][v][0] = S(cc[M + pv * D + k], gn[0]);
+            gS[side][v][1] = S(cc[M + pv * D + t0], g0[0]);
+            gS[side][v][2] = S(cc[M + pv * D + t1], g1[0]);
           } else {
             uS[side][v] = S(val[0], val[1]);
-#pragma unroll
-            for (int kk = 0; kk < D; ++kk) gS[side][v][kk] = S(GCOMP(0, kk), GCOMP(1, kk));
+            gS[side][v][0] = S(gn[0], gn[1]);
+            gS[side][v][1] = S(g0[0], g0[1]);
+            gS[side][v][2] = S(g1[0], g1[1]);
           }
         } else {
           uS[side][v] = val[0];
-#pragma unroll
-          for (int kk = 0; kk < D; ++kk) gS[side][v][kk] = GCOMP(0, kk);
+          gS[side][v][0] = gn[0];
+          gS[side][v][1] = g0[0];
+          gS[side][v][2] = g1[0];
         }
-#undef GCOMP
       }
     }
     if (!physical<D>(uS[0], ph.gm1) || !physical<D>(uS[1], ph.gm1)) atomicOr(status, ST_NONPHYSICAL);
-    S fp[M], GLn[M], GRn[M], DL[M][D], DR[M][D];
-    face_point_k<D, S, T>(k, uS[0], gS[0], uS[1], gS[1], ph, fp, GLn, GRn, DL, DR);
-    T* gq0 = sG + ((size_t)fl * 2 * nqf + q) * M;
-    T* gq1 = sG + ((size_t)(fl * 2 + 1) * nqf + q) * M;
-    T* fo = sF + ((size_t)fl * nqf + q) * M;
-    T* dq0 = sD + (((size_t)fl * 2) * nqf + q) * M * D;
-    T* dq1 = sD + (((size_t)fl * 2 + 1) * nqf + q) * M * D;
+    S fp[M], mL[D], eL[D], mR[D], eR[D];
+    face_point_core<D, 0, S, T>(uS[0], gS[0], uS[1], gS[1], ph, fp, mL, eL, mR, eR);
+    const T fw = mv.fw[(size_t)k * nqf + q];
+    T* o = sP + (size_t)fl * FSF_NP * nqf + q;
+#define PART(x) (JVP ? tan_part(x) : val(x))
 #pragma unroll
-    for (int v = 0; v < M; ++v) {
-      fo[v] = JVP ? tan_part(fp[v]) : val(fp[v]);
-      gq0[v] = JVP ? tan_part(GLn[v]) : val(GLn[v]);
-      gq1[v] = JVP ? tan_part(GRn[v]) : val(GRn[v]);
+    for (int v = 0; v < M; ++v) o[(size_t)v * nqf] = fw * PART(fp[v]);
 #pragma unroll
-      for (int kk = 0; kk < D; ++kk) {
-        dq0[v * D + kk] = JVP ? tan_part(DL[v][kk]) : val(DL[v][kk]);
-        dq1[v * D + kk] = JVP ? tan_part(DR[v][kk]) : val(DR[v][kk]);
-      }
+    for (int j = 0; j < D; ++j) {
+      const T ml = fw * PART(mL[j]), mr = fw * PART(mR[j]), el = fw * PART(eL[j]), er = fw * PART(eR[j]);
+      // normal column of K(uL) jump + K(uR) jump (twice the halves)
+      o[(size_t)(5 + j) * nqf] = (j == 0 ? T(8) / T(3) : T(2)) * (ml + mr);
+      if (j == 0) o[(size_t)8 * nqf] = T(2) * (el + er);
+      o[(size_t)(9 + j) * nqf] = ml;
+      o[(size_t)(12 + j) * nqf] = el;
+      o[(size_t)(15 + j) * nqf] = mr;
+      o[(size_t)(18 + j) * nqf] = er;
     }
+#undef PART
   }
   __syncthreads();
-  // phase 2: BR2 lifting on both sides, fhat = Roe + {F_v}.n + eta {delta}.n (as face_kernel)
-  for (int t = threadIdx.x; t < nloc * nqf; t += blockDim.x) {
-    const int fl = t / nqf, q = t % nqf;
-    const int k = (f0 + fl) / E;
-    const T* PL = mv.lift + (size_t)(2 * k + 1) * nqf * nqf + q;   // column q2 at PL[q2 * nqf]
-    const T* PR = mv.lift + (size_t)(2 * k) * nqf * nqf + q;
-    T dl[M], dr[M];
-#pragma unroll
-    for (int v = 0; v < M; ++v) dl[v] = dr[v] = T(0);
-    for (int q2 = 0; q2 < nqf; ++q2) {
-      const T a = PL[(size_t)q2 * nqf], b = PR[(size_t)q2 * nqf];
-      const T* g0 = sG + ((size_t)fl * 2 * nqf + q2) * M;
-      const T* g1 = sG + ((size_t)(fl * 2 + 1) * nqf + q2) * M;
-#pragma unroll
-      for (int v = 0; v < M; ++v) {
-        dl[v] += a * g0[v];
-        dr[v] += b * g1[v];
-      }
-    }
-    T* fo = sF + ((size_t)fl * nqf + q) * M;
-#pragma unroll
-    for (int v = 0; v < M; ++v) fo[v] += ph.eta * T(0.5) * (dl[v] + dr[v]);
-  }
-  __syncthreads();
-  // phase 3: projection onto both elements' test functions by the transposed
-  // contractions.  Per side and variable, with the point values
-  //   A = sgn fw Fo,  P = -fw Dd_t0 m_t0,  Q = -fw Dd_t1 m_t1,  N = -fw Dd_n m_n:
-  //   X: XA[a0][b1] = sum_b0 A L_a0(b0) + P L'_a0(b0),  XQ = sum_b0 Q L_a0(b0),  XN = sum_b0 N L_a0(b0)
-  //   Y: YA[a0][a1] = sum_b1 XA L_a1(b1) + XQ L'_a1(b1),  YN = sum_b1 XN L_a1(b1)
-  //   slot(mode (ak, a0, a1)) = L_ak(+-1) YA + L'_ak(+-1) YN
-  const int xsz = 2 * M * 3 * n1 * nq;
-  for (int t = threadIdx.x; t < nloc * xsz; t += blockDim.x) {
-    const int fl = t / xsz;
-    int r = t - fl * xsz;
-    const int b1 = r % nq;
-    r /= nq;
-    const int a0 = r % n1;
-    r /= n1;
-    const int kind = r % 3;
-    r /= 3;
-    const int v = r % M, side = r / M;
-    const int k = (f0 + fl) / E, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2;
-    const T sgn = side == 0 ? T(1) : T(-1);
-    const T mk = pick3(k, m0, m1, m2), mt0 = pick3(t0, m0, m1, m2), mt1 = pick3(t1, m0, m1, m2);
-    const T* fw = mv.fw + (size_t)k * nqf;
-    const T* Fo = sF + (size_t)fl * nqf * M;
-    const T* Dd = sD + ((size_t)(fl * 2 + side) * nqf) * M * D;
-    T acc = T(0);
-    for (int b0 = 0; b0 < nq; ++b0) {
-      const int q = b0 + nq * b1;
-      const T la = L[a0 * nq + b0];
-      const T* dd = Dd + ((size_t)q * M + v) * D;
-      if (kind == 0)
-        acc += fw[q] * (sgn * Fo[q * M + v] * la - dd[t0] * mt0 * dL[a0 * nq + b0]);
-      else if (kind == 1)
-        acc -= fw[q] * dd[t1] * mt1 * la;
-      else
-        acc -= fw[q] * dd[k] * mk * la;
-    }
-    sS[(size_t)fl * P.per_face + (t - fl * xsz)] = acc;
-  }
-  __syncthreads();
-  const int ysz = 2 * M * 2 * n1s;
-  for (int t = threadIdx.x; t < nloc * ysz; t += blockDim.x) {
-    const int fl = t / ysz;
-    int r = t - fl * ysz;
-    const int a1 = r % n1;
-    r /= n1;
-    const int a0 = r % n1;
-    r /= n1;
-    const int kind = r % 2;
-    const int sv = r / 2;                    // (side, v)
-    const T* X = sS + (size_t)fl * P.per_face + (size_t)sv * 3 * n1 * nq + a0 * nq;   // [kind][a0][b1]
-    T acc = T(0);
-    if (kind == 0) {
-      for (int b1 = 0; b1 < nq; ++b1) acc += X[b1] * L[a1 * nq + b1] + X[(size_t)n1 * nq + b1] * dL[a1 * nq + b1];
+  // X: sums over b0.  Arrays 0-4 the flux, 5-8 the lifting integrand, then per
+  // side m_n, m_t0, m_t1, e_n, e_t1 with L and m_t0, m_n, e_t0 with L'
+  // (a thread takes the arrays of one kind together: independent sums of one
+  // test function, which keep the FP64 pipe fed from few warps)
+  const int xrow = n1 * nq, xsz = FSF_NX * xrow;
+  for (int t = threadIdx.x; t < nloc * 6 * xrow; t += blockDim.x) {
+    const int g = t / (nloc * xrow);                                // flux, lifting, then (side, L / L')
+    int r = t - g * (nloc * xrow);
+    const int fl = r / xrow;
+    r -= fl * xrow;
+    const int b1 = r % nq, a0 = r / nq, side = g >= 4 ? 1 : 0;
+    const T* src = sP + (size_t)fl * FSF_NP * nqf + (size_t)nq * b1;
+    const bool der = g == 3 || g == 5;
+    const T* La = (der ? dL : L) + a0 * nq;
+    int c0, c1, c2, c3, c4, n, to;                                  // components, how many, first array
+    if (g == 0) {
+      c0 = 0, c1 = 1, c2 = 2, c3 = 3, c4 = 4, n = 5, to = 0;
+    } else if (g == 1) {
+      c0 = 5, c1 = 6, c2 = 7, c3 = 8, c4 = 8, n = 4, to = 5;
     } else {
-      for (int b1 = 0; b1 < nq; ++b1) acc += X[(size_t)2 * n1 * nq + b1] * L[a1 * nq + b1];
+      const int b = 9 + 6 * side;
+      if (!der) {
+        c0 = b, c1 = b + 1, c2 = b + 2, c3 = b + 3, c4 = b + 5, n = 5, to = 9 + 8 * side;
+      } else {
+        c0 = b + 1, c1 = b, c2 = b + 4, c3 = b + 4, c4 = b + 4, n = 3, to = 14 + 8 * side;
+      }
     }
-    sS[(size_t)fl * P.per_face + xsz + (t - fl * ysz)] = acc;
+    const T *p0 = src + (size_t)c0 * nqf, *p1 = src + (size_t)c1 * nqf, *p2 = src + (size_t)c2 * nqf,
+            *p3 = src + (size_t)c3 * nqf, *p4 = src + (size_t)c4 * nqf;
+    T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0), s4 = T(0);
+    if (n == 3) {
+#pragma unroll 2
+      for (int b0 = 0; b0 < nq; ++b0) {
+        const T la = La[b0];
+        s0 += p0[b0] * la;
+        s1 += p1[b0] * la;
+        s2 += p2[b0] * la;
+      }
+    } else if (n == 4) {
+      for (int b0 = 0; b0 < nq; ++b0) {
+        const T la = La[b0];
+        s0 += p0[b0] * la;
+        s1 += p1[b0] * la;
+        s2 += p2[b0] * la;
+        s3 += p3[b0] * la;
+      }
+    } else {
+      for (int b0 = 0; b0 < nq; ++b0) {
+        const T la = La[b0];
+        s0 += p0[b0] * la;
+        s1 += p1[b0] * la;
+        s2 += p2[b0] * la;
+        s3 += p3[b0] * la;
+        s4 += p4[b0] * la;
+      }
+    }
+    T* o = sS + (size_t)fl * P.per_face + (size_t)to * xrow + a0 * nq + b1;
+    o[0] = s0;
+    o[xrow] = s1;
+    o[2 * xrow] = s2;
+    if (n > 3) o[3 * xrow] = s3;
+    if (n > 4) o[4 * xrow] = s4;
   }
   __syncthreads();
-  const int n13 = n1s * n1, osz = 2 * M * n13;
+  // Y: sums over b1, per pair.  Arrays 0-4 the flux, then per side the
+  // dual-consistency terms' value part (n, t0, t1, E) and normal derivative
+  // part, then the lifting (n, t0, t1, E)
+  for (int t = threadIdx.x; t < nloc * 6 * npair; t += blockDim.x) {
+    const int g = t / (nloc * npair);                               // flux, lifting, then (side, value / normal part)
+    int r = t - g * (nloc * npair);
+    const int fl = r / npair, pr = r - fl * npair;
+    const int a0 = ptab[pr] & 255, a1 = ptab[pr] >> 8, side = g >= 4 ? 1 : 0;
+    const int k = (f0 + fl) / E, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2;
+    const T mk = pick3(k, m0, m1, m2);
+    const T* X = sS + (size_t)fl * P.per_face + a0 * nq;       // array i at + i * xrow
+    T* o = sS + (size_t)fl * P.per_face + xsz + pr;            // array i at + i * npair
+    const T* L1 = L + a1 * nq;
+    const T* D1 = dL + a1 * nq;
+    if (g == 0) {
+      T s[M] = {};
+      for (int b = 0; b < nq; ++b)
+#pragma unroll
+        for (int v = 0; v < M; ++v) s[v] += X[(size_t)v * xrow + b] * L1[b];
+#pragma unroll
+      for (int v = 0; v < M; ++v) o[(size_t)v * npair] = s[v];
+    } else if (g == 1) {
+      T s[M - 1] = {};
+      for (int b = 0; b < nq; ++b)
+#pragma unroll
+        for (int v = 0; v < M - 1; ++v) s[v] += X[(size_t)(5 + v) * xrow + b] * L1[b];
+      const int n = total_degree ? n1 - a0 - a1 : n1;          // C_a = n^2 / 2
+      const T sc = ph.eta * mk * (T(0.125) * (T)(n * n));
+#pragma unroll
+      for (int v = 0; v < M - 1; ++v) o[(size_t)(M + 16 + v) * npair] = sc * s[v];
+    } else {
+      const T* xs = X + (size_t)(9 + 8 * side) * xrow;         // m_n m_t0 m_t1 e_n e_t1 | m_t0' m_n' e_t0'
+      T* os = o + (size_t)(M + 8 * side) * npair;
+      if (g == 3 || g == 5) {
+        T s[4] = {};
+        for (int b = 0; b < nq; ++b)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) s[v] += xs[(size_t)v * xrow + b] * L1[b];
+        os[(size_t)4 * npair] = -mk * (T(4) / T(3)) * s[0];
+#pragma unroll
+        for (int v = 1; v < 4; ++v) os[(size_t)(4 + v) * npair] = -mk * s[v];
+      } else {
+        // rows n, E: m_t0 d_t0 + m_t1 d_t1, e_t0 d_t0 + e_t1 d_t1; t0, t1: -2/3 m_n d_t0, d_t1
+        T s[6] = {};
+        for (int b = 0; b < nq; ++b) {
+          const T l = L1[b], dl = D1[b];
+          s[0] += xs[(size_t)5 * xrow + b] * l;
+          s[1] += xs[(size_t)6 * xrow + b] * l;
+          s[2] += xs[(size_t)7 * xrow + b] * l;
+          s[3] += xs[(size_t)2 * xrow + b] * dl;
+          s[4] += xs[b] * dl;
+          s[5] += xs[(size_t)4 * xrow + b] * dl;
+        }
+        const T mt0 = pick3(t0, m0, m1, m2), mt1 = pick3(t1, m0, m1, m2);
+        os[0] = -(mt0 * s[0] + mt1 * s[3]);
+        os[npair] = (T(2) / T(3)) * mt0 * s[1];
+        os[(size_t)2 * npair] = (T(2) / T(3)) * mt1 * s[4];
+        os[(size_t)3 * npair] = -(mt0 * s[2] + mt1 * s[5]);
+      }
+    }
+  }
+  __syncthreads();
+  // the normal direction's end values: modes of both elements, in shared memory
+  const int osz = 2 * M * npair;
   for (int t = threadIdx.x; t < nloc * osz; t += blockDim.x) {
     const int fl = t / osz;
     int r = t - fl * osz;
-    const int tt = r % n13;
-    r /= n13;
+    const int pr = r % npair;
+    r /= npair;
     const int v = r % M, side = r / M;
-    const int i = qidx[tt];
-    if (i < 0) continue;                     // a tensor product outside P_p
-    const int f = f0 + fl, k = f / E, e = f % E, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2;
-    const int x0 = tt % n1, x1 = (tt / n1) % n1, x2 = tt / n1s;
-    const int ak = pick3(k, x0, x1, x2), a0 = pick3(t0, x0, x1, x2), a1 = pick3(t1, x0, x1, x2);
+    const int a0 = ptab[pr] & 255, a1 = ptab[pr] >> 8;
+    const int k = (f0 + fl) / E, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2;
+    const int pv = v == 0 || v == M - 1 ? v : 1 + pick3(v - 1, k, t0, t1);
     const int end = side == 0 ? 1 : 0;
-    const T* Y = sS + (size_t)fl * P.per_face + xsz + (size_t)(side * M + v) * 2 * n1s + a0 * n1 + a1;
-    slots[(((size_t)e * D + k) * 2 + side) * nb + v * nm + i] = Le[end * n1 + ak] * Y[0] + dLe[end * n1 + ak] * Y[n1s];
+    const T* Y = sS + (size_t)fl * P.per_face + xsz + pr;
+    const T yf = v > 0 ? Y[(size_t)v * npair] + Y[(size_t)(M + 16 + v - 1) * npair] : Y[0];
+    T ya = side == 0 ? yf : -yf, yn = T(0);
+    if (v > 0) {
+      ya += Y[(size_t)(M + 8 * side + v - 1) * npair];
+      yn = Y[(size_t)(M + 8 * side + 4 + v - 1) * npair];
+    }
+    const int sk = pick3(k, 1, n1, n1s), base = a0 * pick3(t0, 1, n1, n1s) + a1 * pick3(t1, 1, n1, n1s);
+    const int nak = total_degree ? n1 - a0 - a1 : n1;
+    T* o = sm + ((size_t)fl * 2 + side) * nb + pv * nm;      // over the point values (dead since X)
+    for (int ak = 0; ak < nak; ++ak) o[qidx[base + ak * sk]] = Le[end * n1 + ak] * ya + dLe[end * n1 + ak] * yn;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < nloc * 2 * nb; t += blockDim.x) {
+    const int fl = t / (2 * nb), r = t - fl * 2 * nb, f = f0 + fl, k = f / E, e = f % E;
+    slots[((size_t)e * D + k) * 2 * nb + r] = sm[t];
   }
 }
 
 template <class T, bool JVP>
 static cudaError_t run_face_sf(const Mesh& Ms, const T* W, const T* V, T* slots, const T* Pf, cudaStream_t st) {
   const bool cached = JVP && Pf != nullptr;
+  const int pdeg = Ms.desc.space == DG_SPACE_Q ? 0 : 1;
+  if (Ms.p + 1 > 15) return cudaErrorNotSupported;   // the pair table
   int fpc = std::max(1, 128 / Ms.nqf);
   int dev = 0, smax = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  size_t smem = fsf_plan(Ms.p, Ms.nq1d, Ms.nb, Ms.m, JVP, cached, fpc).total * sizeof(T);
-  while (smem > (size_t)smax - 1024 && fpc > 1) smem = fsf_plan(Ms.p, Ms.nq1d, Ms.nb, Ms.m, JVP, cached, --fpc).total * sizeof(T);
-  if (smem > (size_t)smax - 1024) return cudaErrorNotSupported;
+  auto bytes = [&](int f) { return fsf_plan(Ms.p, Ms.nq1d, Ms.nb, Ms.m, pdeg, JVP, cached, f).total * sizeof(T); };
+  size_t smem = bytes(fpc);
+  while (smem > (size_t)smax - 1536 && fpc > 1) smem = bytes(--fpc);
+  if (smem > (size_t)smax - 1536) return cudaErrorNotSupported;
   if (smem > 48 * 1024) {
     cudaError_t e = allow_max_smem(face_sf_kernel<T, JVP>);
     if (e != cudaSuccess) return e;
@@ -341,7 +444,7 @@ static cudaError_t run_face_sf(const Mesh& Ms, const T* W, const T* V, T* slots,
   note_launch();
   face_sf_kernel<T, JVP><<<(nfaces + fpc - 1) / fpc, 128, smem, st>>>(Ms.view<T>(), Ms.phys_t<T>(), W, V, slots,
                                                                      Ms.status, fpc, cached ? Pf : nullptr, l1,
-                                                                     Ms.qidx, Ms.p, Ms.nq1d, m0, m1, m2);
+                                                                     Ms.qidx, Ms.p, Ms.nq1d, pdeg, m0, m1, m2);
   return cudaGetLastError();
 }
 

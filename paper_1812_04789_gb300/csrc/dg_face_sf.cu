@@ -426,7 +426,8 @@ static cudaError_t run_face_sf(const Mesh& Ms, const T* W, const T* V, T* slots,
   const bool cached = JVP && Pf != nullptr;
   const int pdeg = Ms.desc.space == DG_SPACE_Q ? 0 : 1;
   if (Ms.p + 1 > 15) return cudaErrorNotSupported;   // the pair table
-  int fpc = std::max(1, 128 / Ms.nqf);
+  int threads = 128;
+  int fpc = items_per_cta(3L * Ms.E, std::max(1, 128 / Ms.nqf), Ms.nqf, 128, &threads);
   int dev = 0, smax = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -442,7 +443,7 @@ static cudaError_t run_face_sf(const Mesh& Ms, const T* W, const T* V, T* slots,
   const T m0 = (T)(2.0 / Ms.h[0]), m1 = (T)(2.0 / Ms.h[1]), m2 = (T)(2.0 / Ms.h[2]);
   const int nfaces = 3 * Ms.E;
   note_launch();
-  face_sf_kernel<T, JVP><<<(nfaces + fpc - 1) / fpc, 128, smem, st>>>(Ms.view<T>(), Ms.phys_t<T>(), W, V, slots,
+  face_sf_kernel<T, JVP><<<(nfaces + fpc - 1) / fpc, threads, smem, st>>>(Ms.view<T>(), Ms.phys_t<T>(), W, V, slots,
                                                                      Ms.status, fpc, cached ? Pf : nullptr, l1,
                                                                      Ms.qidx, Ms.p, Ms.nq1d, pdeg, m0, m1, m2);
   return cudaGetLastError();

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
+
+#include <algorithm>
 #include <vector>
 
 #include "../../include/dg.h"
@@ -28,6 +30,25 @@ inline cudaError_t allow_max_smem(K kernel) {
   // the per-block limit covers the kernel's static shared memory too
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               smax - (int)fa.sharedSizeBytes);
+}
+
+inline int sm_count() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 1;
+}
+
+// Work items (elements, faces) per CTA, at most `most`, such that n of them
+// still fill the SMs, and the CTA's threads for them (`points` each; a multiple
+// of a warp, at most `threads`): a small mesh is bound by the longest chain of
+// operations on one SM, FP64 ones above all (16^2 quads, p = 2, residual:
+// face and volume kernels on 16 SMs 52 us, on 128 SMs 41).
+inline int items_per_cta(long n, int most, int points, int threads, int* cta_threads) {
+  const long sms = sm_count();
+  const int per = (int)std::max<long>(1, std::min<long>(most, (n + sms - 1) / sms));
+  *cta_threads = per == most ? threads : std::min(threads, std::max(32, (per * points + 31) / 32 * 32));
+  return per;
 }
 
 // host-side count of kernel launches (dg_launch_count)

@@ -26,17 +26,6 @@
 
 namespace dgk {
 
-static int sm_count() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
 // ---------------------------------------------------------------- elementwise
 template <class T>
 __global__ void axpby_kernel(long n, double a, const T* __restrict__ x, double b, T* __restrict__ y) {

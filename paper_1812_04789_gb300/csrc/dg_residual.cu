@@ -535,12 +535,12 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
   // such CTAs fit shared memory (not for the 125 modes of Q_4: then 128 threads)
   int fthreads = 128;
   if (sizeof(T) == 4 && face_smem<T>(Ms, std::max(1, 256 / Ms.nqf), JVP) <= 100 * 1024) fthreads = 256;
-  int fpc = std::max(1, fthreads / Ms.nqf);
+  int nfaces = D * Ms.E;
+  int fpc = items_per_cta(nfaces, std::max(1, fthreads / Ms.nqf), Ms.nqf, fthreads, &fthreads);
   size_t fsm = face_smem<T>(Ms, fpc, JVP);
   while (fsm > 200 * 1024 && fpc > 1) fsm = face_smem<T>(Ms, --fpc, JVP);
   if (fsm > 48 * 1024)
     allow_max_smem(face_kernel<D, T, JVP>);
-  int nfaces = D * Ms.E;
   if (parts & 1) {
     // 3-D: the face term by sum factorisation in FP64 (fewer of the FP64 pipe's
     // cycles: the residual 4.4 -> 3.8 ms at 16^3 p = 4, 125 -> 73 ms at 32^3
@@ -595,13 +595,14 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
       return cudaGetLastError();
     }
   }
-  int epc = std::max(1, 256 / Ms.nq);
+  int vthreads = 256;
+  int epc = items_per_cta(Ms.E, std::max(1, 256 / Ms.nq), Ms.nq, vthreads, &vthreads);
   size_t vsm = vol_smem<T>(Ms, epc, JVP);
   while (vsm > 200 * 1024 && epc > 1) vsm = vol_smem<T>(Ms, --epc, JVP);
   if (vsm > 48 * 1024)
     allow_max_smem(volume_kernel<D, T, JVP>);
   note_launch();
-  volume_kernel<D, T, JVP><<<(Ms.E + epc - 1) / epc, 256, vsm, st>>>(mv, ph, W, V, slots, S, sigma, out,
+  volume_kernel<D, T, JVP><<<(Ms.E + epc - 1) / epc, vthreads, vsm, st>>>(mv, ph, W, V, slots, S, sigma, out,
                                                                     Ms.status, epc);
   return cudaGetLastError();
 }

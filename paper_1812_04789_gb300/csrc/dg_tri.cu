@@ -409,25 +409,26 @@ cudaError_t launch_residual_tri(const Mesh& M, const T* W, const T* V, const T* 
   const TriView<T> tv = tri_view<T>(M);
   const Phys<T> ph = M.phys_t<T>();
   T* slots = std::is_same<T, double>::value ? (T*)M.t64.slots : (T*)M.t32.slots;
-  const int fpc = std::max(1, 128 / M.nqf);
   const long F = 3L * M.E;
+  int fth = 128, vth = 128;
+  const int fpc = items_per_cta(F, std::max(1, 128 / M.nqf), M.nqf, 128, &fth);
   const int gf = (int)std::min<long>((F + fpc - 1) / fpc, 1L << 20);
   const size_t fsm = (size_t)fpc * M.nqf * TF_NS * sizeof(T);
   note_launch();
   if (jvp)
-    tri_face_kernel<T, true><<<gf, 128, fsm, st>>>(tv, ph, W, V, slots, M.status, fpc);
+    tri_face_kernel<T, true><<<gf, fth, fsm, st>>>(tv, ph, W, V, slots, M.status, fpc);
   else
-    tri_face_kernel<T, false><<<gf, 128, fsm, st>>>(tv, ph, W, nullptr, slots, M.status, fpc);
+    tri_face_kernel<T, false><<<gf, fth, fsm, st>>>(tv, ph, W, nullptr, slots, M.status, fpc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int epc = std::max(1, 128 / M.nq);
+  const int epc = items_per_cta(M.E, std::max(1, 128 / M.nq), M.nq, 128, &vth);
   const int gv = (int)std::min<long>((M.E + epc - 1) / epc, 1L << 20);
   const size_t vsm = (size_t)epc * 8 * M.nq * sizeof(T);
   note_launch();
   if (jvp)
-    tri_volume_kernel<T, true><<<gv, 128, vsm, st>>>(tv, ph, W, V, slots, nullptr, sigma, out, M.status, epc);
+    tri_volume_kernel<T, true><<<gv, vth, vsm, st>>>(tv, ph, W, V, slots, nullptr, sigma, out, M.status, epc);
   else
-    tri_volume_kernel<T, false><<<gv, 128, vsm, st>>>(tv, ph, W, nullptr, slots, S, sigma, out, M.status, epc);
+    tri_volume_kernel<T, false><<<gv, vth, vsm, st>>>(tv, ph, W, nullptr, slots, S, sigma, out, M.status, epc);
   return cudaGetLastError();
 }
 template cudaError_t launch_residual_tri<double>(const Mesh&, const double*, const double*, const double*, double,

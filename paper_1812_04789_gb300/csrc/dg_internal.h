@@ -102,6 +102,7 @@ struct Mesh {
   int* nbr = nullptr;        // device [E][d][2]
   Tables<double> t64;
   Tables<float> t32;
+  std::vector<double> h_l1d; // host copy of l1d
   TcPlan tc;                 // tensor-core probe plan and its element-independent tables:
   float* tc_test = nullptr;  //   test rows [point][kind][nmp] (weights, signs, lifting folded in)
   float* tc_trial = nullptr; //   trial operand per K step [nks][hi, lo][npad x 8] in MMA layout
@@ -166,6 +167,16 @@ cudaError_t launch_volume_q(const Mesh& M, const T* W, const T* V, const T* S, T
 template <class T>
 cudaError_t launch_face_sf(const Mesh& M, const T* W, const T* V, T* slots, bool jvp, const T* Pf,
                            cudaStream_t st);
+
+// FP32 JVP of 3-D P_p meshes with p + 2 points, 1 <= p <= 6 (sf32_ok), by sum
+// factorisation with the loops unrolled for p (csrc/dg_face32.cu: the face
+// slots; csrc/dg_vol32.cu: the rest).  Pf / Pv: primal traces of W cached by
+// launch_primal_cache_sf (their own layout, dg_sf32.cuh), or null.
+bool sf32_ok(const Mesh& M);
+cudaError_t launch_face32(const Mesh& M, const float* W, const float* V, const float* Pf, cudaStream_t st);
+cudaError_t launch_vol32(const Mesh& M, const float* W, const float* V, float sigma, float* out, const float* Pv,
+                         cudaStream_t st);
+cudaError_t launch_primal_cache_sf(const Mesh& M, const float* W, float* Pv, float* Pf, cudaStream_t st);
 
 // Primal traces (u, grad u) of an FP32 state at the volume points and on both
 // sides of every face point; primal_cache_sizes returns the volume cache's

@@ -389,6 +389,7 @@ static dg_status build_mesh(Mesh& M, const dg_mesh_desc* desc, const dg_physics*
       l1d[(size_t)2 * n1 * nq1 + nq1 + a] = Le[a];
       l1d[(size_t)2 * n1 * nq1 + nq1 + 2 * n1 + a] = dLe[a];
     }
+    M.h_l1d = l1d;
     if ((err = upload<double>(M, l1d, &M.t64.l1d)) != cudaSuccess) return DG_ERR_OOM;
     if ((err = upload<float>(M, l1d, &M.t32.l1d)) != cudaSuccess) return DG_ERR_OOM;
     int nt = 1;

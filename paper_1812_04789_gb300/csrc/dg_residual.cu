@@ -541,15 +541,33 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
   while (fsm > 200 * 1024 && fpc > 1) fsm = face_smem<T>(Ms, --fpc, JVP);
   if (fsm > 48 * 1024)
     allow_max_smem(face_kernel<D, T, JVP>);
-  if (parts & 1) {
+  // FP32 JVP on 3-D P_p meshes: kernels of their own, whose cached traces have
+  // their own layout (the kernels below then interpolate the state as well).
+  // DG_NO_SUMFACT_FACE, DG_SUMFACT_FACE_MIN_MODES, DG_NO_SUMFACT_P as below
+  const char* nsff = getenv("DG_NO_SUMFACT_FACE");
+  const char* sfmin = getenv("DG_SUMFACT_FACE_MIN_MODES");
+  const char* nsf = getenv("DG_NO_SUMFACT_P");
+  bool face32 = false, vol32 = false;
+  if constexpr (std::is_same<T, float>::value && JVP && D == 3) {
+    if (sf32_ok(Ms)) {
+      face32 = !(nsff && nsff[0] == '1') && !sfmin;
+      vol32 = !(nsf && nsf[0] == '1');
+      if (face32 && (parts & 1)) {
+        cudaError_t e = launch_face32(Ms, W, V, Pf, st);
+        if (e != cudaSuccess) return e;
+      }
+      if (vol32 && face32) return (parts & 2) ? launch_vol32(Ms, W, V, sigma, out, Pv, st) : cudaSuccess;
+      Pf = nullptr;
+      if (!vol32) Pv = nullptr;
+    }
+  }
+  if ((parts & 1) && !face32) {
     // 3-D: the face term by sum factorisation in FP64 (fewer of the FP64 pipe's
     // cycles: the residual 4.4 -> 3.8 ms at 16^3 p = 4, 125 -> 73 ms at 32^3
     // p = 6); in FP32 the direct kernel is faster (smoother JVP 0.23 against
     // 0.56 ms at p = 4, 4.9 against 9.1 ms at p = 6).  DG_NO_SUMFACT_FACE=1
     // keeps the direct kernel; DG_SUMFACT_FACE_MIN_MODES=n takes the sum-
     // factorised one in FP32 from n modes on
-    const char* nsff = getenv("DG_NO_SUMFACT_FACE");
-    const char* sfmin = getenv("DG_SUMFACT_FACE_MIN_MODES");
     const int min_modes = sfmin ? atoi(sfmin) : INT_MAX;
     cudaError_t e = cudaErrorNotSupported;
     if (D == 3 && !(nsff && nsff[0] == '1') && (std::is_same<T, double>::value || Ms.nm >= min_modes)) {
@@ -565,6 +583,9 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
     if (e != cudaSuccess) return e;
   }
   if (!(parts & 2)) return cudaSuccess;
+  if constexpr (std::is_same<T, float>::value && JVP && D == 3) {
+    if (vol32) return launch_vol32(Ms, W, V, sigma, out, Pv, st);
+  }
   // volume term by sum factorisation (Q_p; P_p embedded in Q_p, 3-D) when its
   // stages fit shared memory, except in FP32 where the shared-memory kernel's
   // tables fit (it reads the cached primal traces and interpolates only the
@@ -572,7 +593,6 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
   size_t tsm0 = 0;
   int nqp0 = 0;
   const bool st_fits = std::is_same<T, float>::value && vol_tables_fit(Ms, JVP, &tsm0, &nqp0);
-  const char* nsf = getenv("DG_NO_SUMFACT_P");
   const bool sumfact = Ms.desc.space == DG_SPACE_Q || (!(nsf && nsf[0] == '1') && !st_fits && Ms.d == 3);
   if (sumfact) {
     cudaError_t eq = launch_volume_q<T>(Ms, W, V, S, sigma, JVP, out, st);
@@ -695,6 +715,7 @@ size_t primal_cache_sizes(const Mesh& M, size_t* nface) {
 }
 
 cudaError_t launch_primal_cache(const Mesh& M, const float* W, float* Pv, float* Pf, cudaStream_t st) {
+  if (sf32_ok(M)) return launch_primal_cache_sf(M, W, Pv, Pf, st);
   const long tot = (long)M.E * M.nq + (long)M.d * M.E * M.nqf * 2;
   const int grid = (int)std::min<long>((tot + 255) / 256, 65535L * 4);
   note_launch();

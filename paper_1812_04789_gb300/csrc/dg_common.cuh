@@ -476,4 +476,17 @@ __device__ __forceinline__ void ld_vec(const T* p, T* out) {
   }
 }
 
+// the same for stores
+template <class T, int N>
+__device__ __forceinline__ void st_vec(T* p, const T* v) {
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k)
+      reinterpret_cast<float4*>(p)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) reinterpret_cast<double2*>(p)[k] = make_double2(v[2 * k], v[2 * k + 1]);
+  }
+}
+
 }  // namespace dgk

@@ -534,6 +534,244 @@ __global__ void __launch_bounds__(256) block_inverse_panel_kernel(T* __restrict_
   }
 }
 
+// Blocks of up to 512 rows that do not fit registers or shared memory (FP32:
+// nb = 280 and 420 at p = 5, 6; FP64: from 175), rows a multiple of 16 bytes:
+// the panel elimination below with one CTA per SM, so that the blocks in
+// flight (152 x 706 KB at nb = 420) stay in L2.
+//  * The panel is held in registers, a thread per row, and eliminated with two
+//    barriers per step: the pivot search is one warp reduction over the value's
+//    bits and one over the warps' candidates, done by every warp for itself,
+//    and the pivot row goes through shared memory.
+//  * The update of the other columns, C += P Xp (Xp the panel's pivot rows as
+//    they were), takes register tiles of RI rows x 16 bytes of columns: per
+//    panel column RI + 16 bytes from shared memory for RI x 16 bytes of
+//    results.  A panel of 128 bytes of columns makes it bound by the FP32 pipe;
+//    panels of 16 FP32 columns are bound by the 2 nb^2 entries of L2 traffic.
+//  * The two permutations of the result go through shared memory slab by slab
+//    (coalesced), not cycle by cycle through memory.
+// nb = 420, 4,096 blocks: 145 -> 28.6 ms; FP64 nb = 175, 1,728 blocks: 27.7 -> 23.5 ms
+// (the FP64 pipe: 16 ms).
+constexpr int BLK_THREADS = 512;
+template <class T>
+struct BlkTile {
+  static constexpr int BW = 128 / sizeof(T);           // panel width
+  static constexpr int RI = sizeof(T) == 4 ? 16 : 8;   // rows of a register tile
+};
+// |x| as an integer that orders like it, in two words; 0 = not a candidate
+__device__ __forceinline__ void pivot_key(float x, bool cand, unsigned* hi, unsigned* lo) {
+  const float v = fabsf(x) >= 0.f ? fabsf(x) : 0.f;   // NaN counts as 0
+  *hi = cand ? __float_as_uint(v) + 1u : 0u;
+  *lo = 0u;
+}
+__device__ __forceinline__ void pivot_key(double x, bool cand, unsigned* hi, unsigned* lo) {
+  const double v = fabs(x) >= 0.0 ? fabs(x) : 0.0;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  *hi = cand ? (unsigned)(b >> 32) + 1u : 0u;
+  *lo = cand ? (unsigned)b : 0u;
+}
+// lowest lane with the largest key (hi, lo) of the warp; all lanes take part
+template <class T>
+__device__ __forceinline__ int warp_argmax(unsigned hi, unsigned lo) {
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  if (sizeof(T) == 4) return __ffs(__ballot_sync(0xffffffffu, hi == mh)) - 1;
+  const unsigned l2 = hi == mh ? lo : 0u, ml = __reduce_max_sync(0xffffffffu, l2);
+  return __ffs(__ballot_sync(0xffffffffu, hi == mh && l2 == ml)) - 1;
+}
+
+// VN consecutive entries of a matrix row (16 bytes, or one entry where rows are not aligned)
+template <class T, int VN>
+__device__ __forceinline__ void ld_row(const T* p, T* v) {
+  if constexpr (VN == 1)
+    v[0] = p[0];
+  else
+    ld_vec<T, VN>(p, v);
+}
+template <class T, int VN>
+__device__ __forceinline__ void st_row(T* p, const T* v) {
+  if constexpr (VN == 1)
+    p[0] = v[0];
+  else
+    st_vec<T, VN>(p, v);
+}
+
+template <class T, int VN>
+__global__ void __launch_bounds__(BLK_THREADS, 1) block_inverse_blk_kernel(T* __restrict__ blocks, int nb,
+                                                                           size_t bstride, long nblk, int slab,
+                                                                           int* status) {
+  constexpr int BW = BlkTile<T>::BW, RI = BlkTile<T>::RI, V16 = 16 / sizeof(T);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nbp = (nb + RI - 1) / RI * RI, nv = nb / VN, nbx = (BW * nb + 1) / 2 * 2;
+  T* Ps = reinterpret_cast<T*>(smem_raw);             // [BW][nbp] panel, transposed; later the permutations' slab
+  T* Xp = Ps + (size_t)BW * nbp;                      // [BW][nb] pivot rows before the panel
+  T* prow = Xp + nbx;                                 // [2][BW] pivot row of the step (alternating)
+  int* piv_row = reinterpret_cast<int*>(prow + 2 * BW);
+  int* step_of = piv_row + nb;
+  __shared__ unsigned cand_hi[2][16], cand_lo[2][16];
+  __shared__ int cand_row[2][16];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < nb; i += BLK_THREADS) step_of[i] = -1;   // no row has been a pivot (again at a block's end)
+  for (long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    T* A = blocks + (size_t)blk * bstride;
+    bool bad = false, used = tid >= nb;
+    for (int k0 = 0; k0 < nb; k0 += BW) {
+      const int bw = min(BW, nb - k0);
+      // the panel into registers, a row per thread (columns past the last: zero)
+      T x[BW];
+#pragma unroll
+      for (int c = 0; c < BW; c += VN) {
+        if (tid < nb && c < bw)
+          ld_row<T, VN>(A + (size_t)tid * nb + k0 + c, x + c);
+        else
+#pragma unroll
+          for (int u = 0; u < VN; ++u) x[c + u] = T(0);
+      }
+#pragma unroll
+      for (int c = 0; c < BW; ++c) {
+        if (c >= bw) break;
+        const int par = c & 1;
+        unsigned hi, lo;
+        pivot_key(x[c], !used, &hi, &lo);
+        const int wl = warp_argmax<T>(hi, lo);
+        if (lane == wl) {
+          cand_hi[par][warp] = hi;
+          cand_lo[par][warp] = lo;
+          cand_row[par][warp] = tid;
+        }
+        __syncthreads();
+        const int b = lane & 15;
+        const int wb = warp_argmax<T>(cand_hi[par][b], cand_lo[par][b]) & 15;
+        const int p = cand_row[par][wb];
+        T* pr = prow + par * BW;
+        if (tid == p) {
+#pragma unroll
+          for (int u = 0; u < BW; ++u) pr[u] = x[u];
+          used = true;
+          piv_row[k0 + c] = p;
+          step_of[p] = k0 + c;
+        }
+        __syncthreads();
+        T piv = pr[c];
+        if (!(fabs(piv) > T(0))) {
+          bad = true;
+          piv = T(1);
+        }
+        const T ipiv = T(1) / piv;
+        if (tid == p) {
+#pragma unroll
+          for (int u = 0; u < BW; ++u) x[u] = u == c ? ipiv : x[u] * ipiv;
+        } else {
+          const T m = x[c] * ipiv;
+#pragma unroll
+          for (int u = 0; u < BW; u += V16) {
+            T q[V16];
+            ld_vec<T, V16>(pr + u, q);
+#pragma unroll
+            for (int w = 0; w < V16; ++w)
+              if (u + w != c) x[u + w] -= m * q[w];
+          }
+          x[c] = -m;
+        }
+      }
+      // pivot rows before the panel, the panel transposed and back in place
+      for (int t = tid; t < bw * nv; t += BLK_THREADS) {
+        const int c = t / nv, v = t - c * nv;
+        T q[VN];
+        ld_row<T, VN>(A + (size_t)piv_row[k0 + c] * nb + v * VN, q);
+#pragma unroll
+        for (int u = 0; u < VN; ++u) Xp[(size_t)c * nb + v * VN + u] = q[u];
+      }
+      if (tid < nbp) {
+#pragma unroll
+        for (int c = 0; c < BW; ++c) Ps[(size_t)c * nbp + tid] = tid < nb ? x[c] : T(0);
+      }
+      __syncthreads();
+      if (tid < nb) {
+#pragma unroll
+        for (int c = 0; c < BW; c += VN)
+          if (c < bw) st_row<T, VN>(A + (size_t)tid * nb + k0 + c, x + c);
+      }
+      // C += P Xp on the other columns (pivot rows: C = P Xp)
+      const int vlo = k0 / VN, nvc = nv - bw / VN;      // columns' vectors outside the panel
+      for (int t = tid; t < nbp / RI * nvc; t += BLK_THREADS) {
+        const int rg = t / nvc, v_ = t - rg * nvc, v = v_ < vlo ? v_ : v_ + bw / VN, i0 = rg * RI;
+        T acc[RI][VN];
+        T* Ac = A + (size_t)i0 * nb + (size_t)v * VN;
+#pragma unroll
+        for (int i = 0; i < RI; ++i) ld_row<T, VN>(Ac + (size_t)min(i, nb - 1 - i0) * nb, acc[i]);
+#pragma unroll
+        for (int i = 0; i < RI; ++i) {
+          const int so = i0 + i < nb ? step_of[i0 + i] : -1;
+          if (so >= k0 && so < k0 + bw)
+#pragma unroll
+            for (int u = 0; u < VN; ++u) acc[i][u] = T(0);
+        }
+#pragma unroll 2
+        for (int c = 0; c < bw; ++c) {
+          T pi[RI], q[VN];
+          ld_vec<T, RI>(Ps + (size_t)c * nbp + i0, pi);
+          ld_row<T, VN>(Xp + (size_t)c * nb + (size_t)v * VN, q);
+#pragma unroll
+          for (int i = 0; i < RI; ++i)
+#pragma unroll
+            for (int u = 0; u < VN; ++u) acc[i][u] += pi[i] * q[u];
+        }
+#pragma unroll
+        for (int i = 0; i < RI; ++i)
+          if (i0 + i < nb) st_row<T, VN>(Ac + (size_t)i * nb, acc[i]);
+      }
+      __syncthreads();
+    }
+    // X[step_of[i]][piv_row[j]] = R[i][j]: rows by slabs of columns, then columns
+    // by slabs of rows, each slab read whole before it is written back
+    for (int j0 = 0; j0 < nb; j0 += slab) {
+      const int w = min(slab, nb - j0);
+      for (int t = tid; t < nb * w; t += BLK_THREADS) {
+        const int i = t / w, j = t - i * w;
+        Ps[(size_t)i * slab + j] = A[(size_t)i * nb + j0 + j];
+      }
+      __syncthreads();
+      for (int t = tid; t < nb * w; t += BLK_THREADS) {
+        const int i = t / w, j = t - i * w;             // row i of the result: R's row piv_row[i]
+        A[(size_t)i * nb + j0 + j] = Ps[(size_t)piv_row[i] * slab + j];
+      }
+      __syncthreads();
+    }
+    for (int i0 = 0; i0 < nb; i0 += slab) {
+      const int w = min(slab, nb - i0);
+      for (int t = tid; t < nb * w; t += BLK_THREADS) Ps[t] = A[(size_t)i0 * nb + t];
+      __syncthreads();
+      for (int t = tid; t < nb * w; t += BLK_THREADS) {
+        const int i = t / nb, j = t - i * nb;           // column j of the result: R's column step_of[j]
+        A[(size_t)i0 * nb + t] = Ps[(size_t)i * nb + step_of[j]];
+      }
+      __syncthreads();
+    }
+    if (bad && tid == 0) atomicOr(status, ST_SINGULAR);
+    __syncthreads();
+    for (int i = tid; i < nb; i += BLK_THREADS) step_of[i] = -1;
+  }
+}
+
+template <class T, int VN>
+cudaError_t run_blk(T* A, int nb, size_t bstride, long nblk, int smax, int* status, cudaStream_t st, bool* done) {
+  constexpr int BW = BlkTile<T>::BW, RI = BlkTile<T>::RI;
+  *done = false;
+  const size_t nbp = (nb + RI - 1) / RI * RI;
+  if (nbp > (size_t)BLK_THREADS || nb % VN || bstride % VN || (reinterpret_cast<uintptr_t>(A) & (VN * sizeof(T) - 1)))
+    return cudaSuccess;
+  const size_t xp = ((size_t)BW * nb + 1) / 2 * 2;       // (16-byte multiple)
+  const size_t tiles = ((size_t)BW * nbp + xp + 2 * BW) * sizeof(T), idx = 2 * (size_t)nb * sizeof(int);
+  if (tiles + idx > (size_t)smax - 1024) return cudaSuccess;
+  const int slab = (int)(((size_t)BW * nbp + (size_t)BW * nb) / nb);   // rows or columns that fit over Ps and Xp
+  cudaError_t e = allow_max_smem(block_inverse_blk_kernel<T, VN>);
+  if (e != cudaSuccess) return e;
+  note_launch();
+  block_inverse_blk_kernel<T, VN><<<(int)std::min<long>(nblk, num_sms_inv()), BLK_THREADS, tiles + idx, st>>>(
+      A, nb, bstride, nblk, slab, status);
+  *done = true;
+  return cudaGetLastError();
+}
+
 template <class T, int R>
 cudaError_t run_reg(T* A, int nb, size_t bstride, long nblk, int* status, cudaStream_t st) {
   const size_t smem = (size_t)nb * inv_ld<T>(nb) * sizeof(T);
@@ -571,6 +809,18 @@ cudaError_t launch_block_inverse(T* A, int nb, size_t bstride, long nblk, int* s
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int use_smem = full <= (size_t)smax - 1024;
+  if (!use_smem) {
+    bool done = false;
+    cudaError_t e = run_blk<T, 16 / (int)sizeof(T)>(A, nb, bstride, nblk, smax, status, st, &done);
+    if (e != cudaSuccess) return e;
+    if (sizeof(T) == 8 && !done)   // FP64 rows of an odd number of entries (nb = 175)
+      if ((e = run_blk<T, sizeof(T) == 8 ? 1 : 4>(A, nb, bstride, nblk, smax, status, st, &done)) != cudaSuccess)
+        return e;
+    if (done) {
+      *transposed = 0;
+      return cudaSuccess;
+    }
+  }
   if (!use_smem) {   // panels of 16 columns in shared memory, rank-16 updates of the rest in global memory
     constexpr int BP = 16;
     const size_t psm = (size_t)nb * BP * sizeof(T) + 4 * (size_t)nb * sizeof(int);

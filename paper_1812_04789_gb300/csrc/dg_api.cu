@@ -338,7 +338,7 @@ static dg_status compute_mg(dg_pmg h, MG<T>& mg, const double* W64, cudaStream_t
   else
     CK(launch_probe_blocks<T>(M, mg.W, (T)h->sigma, mg.lv[0].Dinv, mg.lv[0].bs, nl > 1 ? mg.lv[1].O : nullptr,
                               nl > 1 ? mg.lv[1].nm : 0, nl > 1 ? mg.lv[1].co_t : 0, mg.scratch, mg.scratch_elems,
-                              st));
+                              st, mg.Pv, mg.Pf));
   const Level<T>& F = mg.lv[0];
   for (int l = 1; l < nl; ++l) {
     Level<T>& L = mg.lv[l];
@@ -735,7 +735,7 @@ static dg_status export_level(const MG<T>& mg, const Mesh& M, T* W, double sigma
       CK(launch_probe_blocks_tri<T>(M, W, (T)sigma, out, (size_t)nb * nb, nullptr, 0, 0, 0, mg.lv[0].r, mg.lv[0].t, st));
     else if (level == 0)
       CK(launch_probe_blocks<T>(M, W, (T)sigma, out, (size_t)nb * nb, nullptr, 0, 0, mg.scratch, mg.scratch_elems,
-                                st));
+                                st, mg.Pv, mg.Pf));
     else
       CK(launch_unpack_inverse<T>(L.Dop, L.cs, L.co_t, out, nb, (long)nblk, st));
   } else {

@@ -347,8 +347,11 @@ static cudaError_t run_probe(const Mesh& Ms, const T* W, T sigma, T* Dout, size_
   return cudaGetLastError();
 }
 
-// FP32 blocks go through the tensor-core kernel when the mesh has a plan for
-// it (DG_PROBE_SIMT=1 in the environment selects the SIMT kernel instead); the
+// Diagonal blocks of 3-D P_p meshes come from the sum-factorised probe
+// (probe_sf_ok; faster at every order it has, figures there), other FP32 blocks
+// from the tensor-core kernel when the mesh has a plan for it, other FP64
+// blocks from probe64_kernel where they fit it (DG_PROBE_SIMT=1 in the
+// environment selects the general kernel for all); in FP32 the
 // coarse neighbour blocks then come from probe_nbr_kernel, or, when a
 // direction has one element (its faces feed the diagonal block), from the SIMT
 // kernel restricted to the neighbour-seeded terms.
@@ -359,10 +362,15 @@ static bool use_tc(const Mesh& M) {
 
 template <class T>
 cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, int nmc,
-                                int nbr_colmajor, T* scratch, size_t scratch_elems, cudaStream_t st) {
+                                int nbr_colmajor, T* scratch, size_t scratch_elems, cudaStream_t st, const T* Pv,
+                                const T* Pf) {
+  const char* simt = getenv("DG_PROBE_SIMT");
+  const bool sf = probe_sf_ok(M) && !(simt && simt[0] == '1');
   if (std::is_same<T, float>::value && nbr_colmajor && O) {
     // layout fixed at setup: the neighbour blocks always come from probe_nbr_kernel
-    cudaError_t e = use_tc(M) ? launch_probe_tc(M, (const float*)W, (float)sigma, (float*)D, dstride, st)
+    cudaError_t e = sf ? launch_probe_sf(M, (const float*)W, (float)sigma, (float*)D, dstride, (const float*)Pv,
+                                         (const float*)Pf, st)
+                   : use_tc(M) ? launch_probe_tc(M, (const float*)W, (float)sigma, (float*)D, dstride, st)
                    : M.d == 2 ? run_probe<2, T>(M, W, sigma, D, dstride, nullptr, 0, scratch, scratch_elems, false, st)
                               : run_probe<3, T>(M, W, sigma, D, dstride, nullptr, 0, scratch, scratch_elems, false, st);
     if (e != cudaSuccess) return e;
@@ -370,12 +378,19 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
   }
   bool nbr_only = false;
   if constexpr (std::is_same<T, double>::value) {
-    const char* e = getenv("DG_PROBE_SIMT");
-    if (!(e && e[0] == '1') && probe64_fits(M, O ? nmc : 0))
-      return launch_probe64(M, W, sigma, D, dstride, O, nmc, nbr_colmajor, st);
+    if (!(simt && simt[0] == '1') && probe64_fits(M, O ? nmc : 0)) {
+      const bool diag = sf && probe_sf64_ok(M);
+      if (diag) {
+        cudaError_t e = launch_probe_sf(M, W, sigma, D, dstride, st);
+        if (e != cudaSuccess) return e;
+      }
+      return launch_probe64(M, W, sigma, diag ? nullptr : D, dstride, O, nmc, nbr_colmajor, st);
+    }
   }
   if (std::is_same<T, float>::value && use_tc(M)) {
-    cudaError_t e = launch_probe_tc(M, (const float*)W, (float)sigma, (float*)D, dstride, st);
+    cudaError_t e = sf ? launch_probe_sf(M, (const float*)W, (float)sigma, (float*)D, dstride, (const float*)Pv,
+                                         (const float*)Pf, st)
+                       : launch_probe_tc(M, (const float*)W, (float)sigma, (float*)D, dstride, st);
     if (e != cudaSuccess) return e;
     bool self = false;
     for (int k = 0; k < M.d; ++k) self = self || M.desc.n[k] == 1;
@@ -387,9 +402,10 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
   return run_probe<3, T>(M, W, sigma, D, dstride, O, nmc, scratch, scratch_elems, nbr_only, st);
 }
 template cudaError_t launch_probe_blocks<double>(const Mesh&, const double*, double, double*, size_t, double*,
-                                                 int, int, double*, size_t, cudaStream_t);
+                                                 int, int, double*, size_t, cudaStream_t, const double*,
+                                                 const double*);
 template cudaError_t launch_probe_blocks<float>(const Mesh&, const float*, float, float*, size_t, float*, int,
-                                                int, float*, size_t, cudaStream_t);
+                                                int, float*, size_t, cudaStream_t, const float*, const float*);
 
 bool probe_nbr_colmajor_ok(const Mesh& M, int nmc) { return use_tc(M) && probe_nbr_fits(M, nmc); }
 

@@ -393,7 +393,7 @@ cudaError_t run_face32(const Mesh& Ms, const float* W, const float* V, float* sl
   if (e != cudaSuccess) return e;
   note_launch();
   face32_kernel<N1, CACHED><<<(3 * Ms.E + C::FPC - 1) / C::FPC, F32_THREADS, C::bytes, st>>>(
-      sf32_tab<N1>(Ms), Ms.phys_t<float>(), Ms.nbr, Ms.qidx, Ms.E, W, V, slots, Ms.status, Pf);
+      sf_tab<float, N1>(Ms), Ms.phys_t<float>(), Ms.nbr, Ms.qidx, Ms.E, W, V, slots, Ms.status, Pf);
   return cudaGetLastError();
 }
 

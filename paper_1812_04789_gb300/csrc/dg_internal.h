@@ -195,9 +195,11 @@ cudaError_t launch_residual_with_slots(const Mesh& M, const double* W, const dou
 // D[e] starts at D + e * dstride (row-major, row stride nb).  With
 // nbr_colmajor (FP32 only, probe_nbr_colmajor_ok) the neighbour blocks are
 // written column-major by probe_nbr_kernel, else row-major, nbc^2 apart.
+// Pv, Pf: cached primal traces of W (FP32, or null).
 template <class T>
 cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, int nmc,
-                                int nbr_colmajor, T* scratch, size_t scratch_elems, cudaStream_t st);
+                                int nbr_colmajor, T* scratch, size_t scratch_elems, cudaStream_t st,
+                                const T* Pv = nullptr, const T* Pf = nullptr);
 template <class T>
 size_t probe_scratch_elems(const Mesh& M, int nmc, bool* fits_smem);
 
@@ -208,7 +210,16 @@ cudaError_t launch_probe_tc(const Mesh& M, const float* W, float sigma, float* D
                             cudaStream_t st);
 cudaError_t build_tc_tables(Mesh& M);
 
-// FP64 blocks (csrc/dg_probe64.cu): D as launch_probe_blocks, O (may be null)
+// Diagonal blocks of 3-D P_p meshes (p = 1 .. 6 in FP32, .. 4 in FP64, p + 2
+// points, no direction of one element) by sum factorisation
+// (csrc/dg_probe_sf.cuh), written in full as launch_probe_blocks does.
+bool probe_sf_ok(const Mesh& M);
+bool probe_sf64_ok(const Mesh& M);
+cudaError_t launch_probe_sf(const Mesh& M, const float* W, float sigma, float* D, size_t dstride, const float* Pv,
+                            const float* Pf, cudaStream_t st);
+cudaError_t launch_probe_sf(const Mesh& M, const double* W, double sigma, double* D, size_t dstride, cudaStream_t st);
+
+// FP64 blocks (csrc/dg_probe64.cu): D (null: the neighbour blocks alone) as launch_probe_blocks, O (may be null)
 // column-major with leading dimension inv_ld(nbc), nbc * inv_ld(nbc) apart, or
 // row-major, nbc^2 apart.  probe64_fits: structured, no direction of one
 // element, blocks within the kernel's registers and shared memory.

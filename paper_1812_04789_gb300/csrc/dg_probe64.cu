@@ -23,7 +23,8 @@
 // Blocks of more entries than 256 threads hold are taken in passes over the
 // rows (w, v, i'), each a CTA of its own, as is an element's set of neighbour
 // blocks.  9 x 10 x 12 elements, p = 3: 137 -> 34 ms (17 M multiply-adds per element at the FP64 pipe's rate: 29 ms);
-// 16^2 quads, p = 2 (diagonal blocks alone): 1.63 -> 0.2 ms.
+// 16^2 quads, p = 2 (diagonal blocks alone): 1.63 -> 0.2 ms.  The diagonal
+// blocks of 3-D P_p meshes up to p = 4 come from dg_probe_sf.cuh instead (12^3, p = 4: 198 -> 42 ms).
 #include <algorithm>
 
 #include "dg_probe.cuh"
@@ -386,7 +387,9 @@ cudaError_t launch_probe64(const Mesh& M, const double* W, double sigma, double*
                            int nmc, int colmajor, cudaStream_t st) {
   P64Plan P;
   if (!O) nmc = 0;
+  if (!O && !D) return cudaSuccess;
   if (!probe64_plan(M, nmc, &P)) return cudaErrorInvalidValue;
+  if (!D) P.passes = 0;
   const int nbc = M.m * nmc, ldo = colmajor ? inv_ld<double>(nbc) : 0;
   const size_t ostride = (size_t)nbc * (ldo ? ldo : nbc);
   if (M.d == 2)

@@ -1,7 +1,7 @@
 // Neighbour blocks of the first coarse level (Sec. 6.3: the inherited
 // block-sparse operator needs dR_e/dW_nbr restricted to the coarse modes),
-// FP32, for the mixed-precision preconditioner when the diagonal blocks come
-// from the tensor-core probe.
+// FP32, for the mixed-precision preconditioner when the mesh has the
+// tensor-core probe's tables.
 //
 // For face s of element e (neighbour n = nbr(e, s), which sees the face as its
 // local face s ^ 1), with nmc coarse modes per variable:

@@ -1,5 +1,7 @@
 // Element Jacobian blocks on the 5th-generation tensor cores (FP32 blocks of
-// the mixed-precision preconditioner; Sec. 5.1 eq. ODEDG, Sec. 6.3).
+// the mixed-precision preconditioner; Sec. 5.1 eq. ODEDG, Sec. 6.3): 2-D
+// meshes, 3-D Q_p and 3-D with a direction of one element (the other 3-D P_p
+// blocks: dg_probe_sf.cuh).
 //
 // The diagonal block of element e is a sum over its volume points and the
 // points of its own faces,

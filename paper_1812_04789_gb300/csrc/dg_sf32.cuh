@@ -1,5 +1,5 @@
-// Shared by the FP32 Jacobian-vector product kernels of 3-D P_p meshes
-// (dg_vol32.cu, dg_face32.cu): the one-dimensional tables as a kernel parameter
+// Shared by the FP32 Jacobian-vector product kernels (dg_vol32.cu,
+// dg_face32.cu) and the block probe (dg_probe_sf.cuh) of 3-D P_p meshes: the one-dimensional tables as a kernel parameter
 // (after unrolling, operands straight from the constant bank: a multiply-add
 // of a contraction costs no load for its table entry) and the layout of the
 // cached primal traces.
@@ -9,33 +9,35 @@
 namespace dgk {
 
 // N1 = p + 1 values of a one-dimensional degree, N1 + 1 Gauss-Legendre points
-template <int N1>
-struct Sf32Tab {
-  float L[N1][N1 + 1], dL[N1][N1 + 1];   // values and reference derivatives
-  float w[N1 + 1];                       // weights
-  float Le[N1], dLe[N1];                 // end values at +1; at -1: (-1)^a Le, -(-1)^a dLe
-  float met[3], detJ, faceJ[3];          // 2 / h_k, |J|, |J_F|
+template <class T, int N1>
+struct SfTab {
+  T L[N1][N1 + 1], dL[N1][N1 + 1];   // values and reference derivatives
+  T w[N1 + 1];                       // weights
+  T Le[N1], dLe[N1];                 // end values at +1; at -1: (-1)^a Le, -(-1)^a dLe
+  T met[3], detJ, faceJ[3];          // 2 / h_k, |J|, |J_F|
 };
-
 template <int N1>
-inline Sf32Tab<N1> sf32_tab(const Mesh& M) {
+using Sf32Tab = SfTab<float, N1>;
+
+template <class T, int N1>
+inline SfTab<T, N1> sf_tab(const Mesh& M) {
   constexpr int NQ = N1 + 1;
-  Sf32Tab<N1> t;
+  SfTab<T, N1> t;
   const std::vector<double>& l = M.h_l1d;   // L[a][q], dL[a][q], w[q], Le(-1)[a], Le(+1)[a], dLe(-1)[a], dLe(+1)[a]
   for (int a = 0; a < N1; ++a) {
     for (int q = 0; q < NQ; ++q) {
-      t.L[a][q] = (float)l[(size_t)a * NQ + q];
-      t.dL[a][q] = (float)l[(size_t)(N1 + a) * NQ + q];
+      t.L[a][q] = (T)l[(size_t)a * NQ + q];
+      t.dL[a][q] = (T)l[(size_t)(N1 + a) * NQ + q];
     }
-    t.Le[a] = (float)l[(size_t)2 * N1 * NQ + NQ + N1 + a];
-    t.dLe[a] = (float)l[(size_t)2 * N1 * NQ + NQ + 3 * N1 + a];
+    t.Le[a] = (T)l[(size_t)2 * N1 * NQ + NQ + N1 + a];
+    t.dLe[a] = (T)l[(size_t)2 * N1 * NQ + NQ + 3 * N1 + a];
   }
-  for (int q = 0; q < NQ; ++q) t.w[q] = (float)l[(size_t)2 * N1 * NQ + q];
+  for (int q = 0; q < NQ; ++q) t.w[q] = (T)l[(size_t)2 * N1 * NQ + q];
   for (int k = 0; k < 3; ++k) {
-    t.met[k] = (float)(2.0 / M.h[k]);
-    t.faceJ[k] = (float)M.faceJ[k];
+    t.met[k] = (T)(2.0 / M.h[k]);
+    t.faceJ[k] = (T)M.faceJ[k];
   }
-  t.detJ = (float)M.detJ;
+  t.detJ = (T)M.detJ;
   return t;
 }
 

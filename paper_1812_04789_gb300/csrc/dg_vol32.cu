@@ -369,7 +369,7 @@ cudaError_t run_vol32(const Mesh& Ms, const float* W, const float* V, const floa
   if (e != cudaSuccess) return e;
   note_launch();
   vol32_kernel<N1, CACHED><<<(Ms.E + C::EPC - 1) / C::EPC, V32_THREADS, C::bytes, st>>>(
-      sf32_tab<N1>(Ms), Ms.phys_t<float>(), Ms.nbr, Ms.qidx, Ms.E, W, V, slots, sigma, out, Ms.status, Pv);
+      sf_tab<float, N1>(Ms), Ms.phys_t<float>(), Ms.nbr, Ms.qidx, Ms.E, W, V, slots, sigma, out, Ms.status, Pv);
   return cudaGetLastError();
 }
 

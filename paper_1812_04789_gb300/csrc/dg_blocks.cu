@@ -348,7 +348,8 @@ static cudaError_t run_probe(const Mesh& Ms, const T* W, T sigma, T* Dout, size_
 }
 
 // Diagonal blocks of 3-D P_p meshes come from the sum-factorised probe
-// (probe_sf_ok; faster at every order it has, figures there), other FP32 blocks
+// (probe_sf_ok; faster at every order it has, figures there), their coarse
+// neighbour blocks from nbr_sf_kernel (FP32: where the traces are cached), other FP32 blocks
 // from the tensor-core kernel when the mesh has a plan for it, other FP64
 // blocks from probe64_kernel where they fit it (DG_PROBE_SIMT=1 in the
 // environment selects the general kernel for all); in FP32 the
@@ -374,18 +375,17 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
                    : M.d == 2 ? run_probe<2, T>(M, W, sigma, D, dstride, nullptr, 0, scratch, scratch_elems, false, st)
                               : run_probe<3, T>(M, W, sigma, D, dstride, nullptr, 0, scratch, scratch_elems, false, st);
     if (e != cudaSuccess) return e;
-    return launch_probe_nbr(M, (const float*)W, (float*)O, nmc, 1, st);
+    return sf && Pf ? launch_nbr_sf(M, (const float*)W, (float*)O, nmc, 1, (const float*)Pf, st)
+                    : launch_probe_nbr(M, (const float*)W, (float*)O, nmc, 1, st);
   }
   bool nbr_only = false;
   if constexpr (std::is_same<T, double>::value) {
-    if (!(simt && simt[0] == '1') && probe64_fits(M, O ? nmc : 0)) {
-      const bool diag = sf && probe_sf64_ok(M);
-      if (diag) {
-        cudaError_t e = launch_probe_sf(M, W, sigma, D, dstride, st);
-        if (e != cudaSuccess) return e;
-      }
-      return launch_probe64(M, W, sigma, diag ? nullptr : D, dstride, O, nmc, nbr_colmajor, st);
+    if (sf && probe_sf64_ok(M)) {
+      cudaError_t e = launch_probe_sf(M, W, sigma, D, dstride, st);
+      return e != cudaSuccess || !O ? e : launch_nbr_sf(M, W, O, nmc, nbr_colmajor, st);
     }
+    if (!(simt && simt[0] == '1') && probe64_fits(M, O ? nmc : 0))
+      return launch_probe64(M, W, sigma, D, dstride, O, nmc, nbr_colmajor, st);
   }
   if (std::is_same<T, float>::value && use_tc(M)) {
     cudaError_t e = sf ? launch_probe_sf(M, (const float*)W, (float)sigma, (float*)D, dstride, (const float*)Pv,
@@ -395,6 +395,7 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
     bool self = false;
     for (int k = 0; k < M.d; ++k) self = self || M.desc.n[k] == 1;
     if (O == nullptr && !self) return cudaSuccess;
+    if (sf && Pf) return launch_nbr_sf(M, (const float*)W, (float*)O, nmc, 0, (const float*)Pf, st);
     if (!self && probe_nbr_fits(M, nmc)) return launch_probe_nbr(M, (const float*)W, (float*)O, nmc, 0, st);
     nbr_only = true;
   }

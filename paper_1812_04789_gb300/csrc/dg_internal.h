@@ -218,8 +218,13 @@ bool probe_sf64_ok(const Mesh& M);
 cudaError_t launch_probe_sf(const Mesh& M, const float* W, float sigma, float* D, size_t dstride, const float* Pv,
                             const float* Pf, cudaStream_t st);
 cudaError_t launch_probe_sf(const Mesh& M, const double* W, double sigma, double* D, size_t dstride, cudaStream_t st);
+// Neighbour blocks of the same meshes (csrc/dg_nbr_sf.cuh), O as launch_probe_nbr;
+// FP32 from the cached traces Pf alone.
+cudaError_t launch_nbr_sf(const Mesh& M, const float* W, float* O, int nmc, int colmajor, const float* Pf,
+                          cudaStream_t st);
+cudaError_t launch_nbr_sf(const Mesh& M, const double* W, double* O, int nmc, int colmajor, cudaStream_t st);
 
-// FP64 blocks (csrc/dg_probe64.cu): D (null: the neighbour blocks alone) as launch_probe_blocks, O (may be null)
+// FP64 blocks (csrc/dg_probe64.cu): D as launch_probe_blocks, O (may be null)
 // column-major with leading dimension inv_ld(nbc), nbc * inv_ld(nbc) apart, or
 // row-major, nbc^2 apart.  probe64_fits: structured, no direction of one
 // element, blocks within the kernel's registers and shared memory.

@@ -387,9 +387,7 @@ cudaError_t launch_probe64(const Mesh& M, const double* W, double sigma, double*
                            int nmc, int colmajor, cudaStream_t st) {
   P64Plan P;
   if (!O) nmc = 0;
-  if (!O && !D) return cudaSuccess;
   if (!probe64_plan(M, nmc, &P)) return cudaErrorInvalidValue;
-  if (!D) P.passes = 0;
   const int nbc = M.m * nmc, ldo = colmajor ? inv_ld<double>(nbc) : 0;
   const size_t ostride = (size_t)nbc * (ldo ? ldo : nbc);
   if (M.d == 2)

@@ -64,10 +64,10 @@ struct Psf {
 // items, table entries of the trial side from the constant bank.  A product of
 // total-degree pairs uses a < n alone: FP64 leaves the others out (its pipe is the
 // limit; n is the same for most of a warp), FP32 computes and drops them.
-template <class T, int N1, bool RD>
+template <class T, int N1, int NC, bool RD>
 __device__ __forceinline__ void psf_row(const SfTab<T, N1>& tb, const T* x, T* acc, int n) {
 #pragma unroll
-  for (int b = 0; b < N1; ++b)
+  for (int b = 0; b < NC; ++b)
     if (sizeof(T) == 4 || b < n)
 #pragma unroll
       for (int q = 0; q < N1 + 1; ++q) acc[b] += x[q] * (RD ? tb.dL[b][q] : tb.L[b][q]);
@@ -77,6 +77,109 @@ template <class T, int NQ, int S, bool ADD>
 __device__ __forceinline__ void psf_scale(const T* t, const T* y, T* x) {
 #pragma unroll
   for (int q = 0; q < NQ; ++q) x[q] = ADD ? x[q] + t[q] * y[q * S] : t[q] * y[q * S];
+}
+
+// The state at point q of face f in the face's frame (directions n, t0, t1;
+// momenta likewise); sd 0: from the L element's +1 face, sd 1: from R's -1 face.
+// sW: the modes of the element, then of its neighbours.
+template <class T, int N1>
+__device__ __forceinline__ void psf_face_trace(const MeshView<T>& mv, const T* sW, int f, int sd, int q, T* c) {
+  constexpr int NQ = N1 + 1, NL = NQ * NQ, NM = sf32_modes(N1), M = 5;
+  const int k = f >> 1, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2, qs = q / NQ + NQ * (q % NQ), lf = sd == 0 ? 2 * k + 1 : 2 * k;
+  const T* ws = sW + ((sd == 0) == ((f & 1) == 1) ? 0 : 1 + f) * M * NM;
+#pragma unroll
+  for (int j = 0; j < 20; ++j) c[j] = T(0);
+  for (int i = 0; i < NM; ++i) {
+    const T p = mv.fphiT[((size_t)lf * NM + i) * NL + qs];
+    const T dn = mv.fdphiT[(((size_t)lf * 3 + k) * NM + i) * NL + qs];
+    const T d0 = mv.fdphiT[(((size_t)lf * 3 + t0) * NM + i) * NL + qs];
+    const T d1 = mv.fdphiT[(((size_t)lf * 3 + t1) * NM + i) * NL + qs];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const int pv = v == 0 || v == M - 1 ? v : v == 1 ? 1 + k : v == 2 ? 1 + t0 : 1 + t1;
+      const T a = ws[pv * NM + i];
+      c[v] += a * p;
+      c[5 + 3 * v] += a * dn;
+      c[6 + 3 * v] += a * d0;
+      c[7 + 3 * v] += a * d1;
+    }
+  }
+}
+
+// Derivatives of the outputs of one face point with respect to seed s (0 the
+// value, 1 + j the gradient component j of the face's frame) of variable w of
+// this element's state (OWN) or the neighbour's, weighted: o[(v 8 + kind) NL],
+// v in the face's frame, kinds 0 flux, 1 lifting (s = 0), 2 3 4 flux (s = 1, 2,
+// 3), 5 6 7 the own dual tensor's rows n, t0, t1 (s = 0).  side 1: this
+// element's +1 face.
+template <class T, int N1, bool OWN>
+__device__ __forceinline__ void psf_face_jac(const SfTab<T, N1>& tb, const Phys<T>& ph, const T (*c)[20], int k, int side,
+                                             int q, int s, int w, T* o) {
+  using S = Dual<T>;
+  constexpr int NQ = N1 + 1, NL = NQ * NQ, M = 5;
+  const int b0 = q / NQ, b1 = q - b0 * NQ, t0 = k == 0 ? 1 : 0;
+  const int wf = w == 0 || w == M - 1 ? w : w == 1 + k ? 1 : w == 1 + t0 ? 2 : 3;   // w in the face's frame
+  const T mkk = k == 0 ? tb.met[0] : k == 1 ? tb.met[1] : tb.met[2];
+  const T mt0 = k == 0 ? tb.met[1] : tb.met[0], mt1 = k == 2 ? tb.met[1] : tb.met[2];
+  T wb0 = T(0), wb1 = T(0);
+#pragma unroll
+  for (int b = 0; b < NQ; ++b) {
+    if (b0 == b) wb0 = tb.w[b];
+    if (b1 == b) wb1 = tb.w[b];
+  }
+  const T fw = (k == 0 ? tb.faceJ[0] : k == 1 ? tb.faceJ[1] : tb.faceJ[2]) * wb0 * wb1;
+  const T sg = side ? fw : -fw;
+  if (s == 0) {
+    S u[2][M], g[2][M][3];
+#pragma unroll
+    for (int sd = 0; sd < 2; ++sd)
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        u[sd][v] = S(c[sd][v], (((sd == 0) == (side == 1)) == OWN && v == wf) ? T(1) : T(0));
+#pragma unroll
+        for (int j = 0; j < 3; ++j) g[sd][v][j] = S(c[sd][5 + 3 * v + j], T(0));
+      }
+    S fp[M], mL[3], eL[3], mR[3], eR[3];
+    face_point_core<3, 0, S, T>(u[0], g[0], u[1], g[1], ph, fp, mL, eL, mR, eR);
+    const T lf = sg * ph.eta * mkk * T(0.125);
+    T m[3], en[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      m[j] = side ? mL[j].d : mR[j].d;
+      en[j] = side ? eL[j].d : eR[j].d;
+    }
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const int j = v == 0 || v == M - 1 ? 0 : v - 1;
+      o[(v * 8 + 0) * NL] = sg * fp[v].d;
+      // normal column of K(uL) jump + K(uR) jump (twice the halves)
+      o[(v * 8 + 1) * NL] = v == 0 ? T(0)
+                          : v == M - 1 ? lf * T(2) * (eL[0].d + eR[0].d)
+                                       : lf * (v == 1 ? T(8) / T(3) : T(2)) * (mL[j].d + mR[j].d);
+      // the own dual tensor (visc_rank1): rows n, t0, t1, E
+      const T dn = v == 0 ? T(0) : v == 1 ? (T(4) / T(3)) * m[0] : v == 2 ? m[1] : v == 3 ? m[2] : en[0];
+      const T d0 = v == 1 ? m[1] : v == 2 ? (T(-2) / T(3)) * m[0] : v == 4 ? en[1] : T(0);
+      const T d1 = v == 1 ? m[2] : v == 3 ? (T(-2) / T(3)) * m[0] : v == 4 ? en[2] : T(0);
+      o[(v * 8 + 5) * NL] = -fw * mkk * dn;
+      o[(v * 8 + 6) * NL] = -fw * mt0 * d0;
+      o[(v * 8 + 7) * NL] = -fw * mt1 * d1;
+    }
+  } else {
+    T u[M], g[M][3], F[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      u[v] = (side == 1) == OWN ? c[0][v] : c[1][v];
+      F[v] = T(0);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) g[v][j] = (v == wf && j == s - 1) ? T(1) : T(0);
+    }
+    Prim<3, T> pr;
+    primitives<3, T, T>(u, ph, pr);
+    add_visc_col<3, 0, T, T>(pr, g, T(0.5), F, ph);
+    const T sc = sg * (s == 1 ? mkk : s == 2 ? mt0 : mt1);
+#pragma unroll
+    for (int v = 0; v < M; ++v) o[(v * 8 + 1 + s) * NL] = sc * F[v];
+  }
 }
 
 template <class T, int N1, int VG, int VP, int CQ, bool CACHED>
@@ -129,29 +232,6 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
     sL[t] = tb.L[t / NQ][t % NQ];
     sdL[t] = tb.dL[t / NQ][t % NQ];
   }
-
-  // the state at point q of face f in its frame; sd 0: from the L element's +1 face, sd 1: from R's -1 face
-  [[maybe_unused]] auto face_trace = [&](int f, int sd, int q, T* c) {
-    const int k = f >> 1, t0 = k == 0 ? 1 : 0, t1 = k == 2 ? 1 : 2, qs = q / NQ + NQ * (q % NQ), lf = sd == 0 ? 2 * k + 1 : 2 * k;
-    const T* ws = sW + ((sd == 0) == ((f & 1) == 1) ? 0 : 1 + f) * NB;
-#pragma unroll
-    for (int j = 0; j < 20; ++j) c[j] = T(0);
-    for (int i = 0; i < NM; ++i) {
-      const T p = mv.fphiT[((size_t)lf * NM + i) * NL + qs];
-      const T dn = mv.fdphiT[(((size_t)lf * 3 + k) * NM + i) * NL + qs];
-      const T d0 = mv.fdphiT[(((size_t)lf * 3 + t0) * NM + i) * NL + qs];
-      const T d1 = mv.fdphiT[(((size_t)lf * 3 + t1) * NM + i) * NL + qs];
-#pragma unroll
-      for (int v = 0; v < M; ++v) {
-        const int pv = v == 0 || v == M - 1 ? v : v == 1 ? 1 + k : v == 2 ? 1 + t0 : 1 + t1;
-        const T a = ws[pv * NM + i];
-        c[v] += a * p;
-        c[5 + 3 * v] += a * dn;
-        c[6 + 3 * v] += a * d0;
-        c[7 + 3 * v] += a * d1;
-      }
-    }
-  };
 
   for (int e = blockIdx.x; e < E; e += gridDim.x) {
     T* De = Dout + (size_t)e * dstride;
@@ -274,10 +354,10 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
 #pragma unroll
               for (int b = 0; b < N1; ++b) acc[b] = T(0);
               psf_scale<T, NQ, NL, false>(tt, j, x);
-              psf_row<T, N1, false>(tb, x, acc, N1);
+              psf_row<T, N1, N1, false>(tb, x, acc, N1);
               if (sg == 0) {
                 psf_scale<T, NQ, NL, false>(tt, j + NV, x);
-                psf_row<T, N1, true>(tb, x, acc, N1);
+                psf_row<T, N1, N1, true>(tb, x, acc, N1);
               }
               T* o = X + ((size_t)r * N2 + at * N1) * XQ * CQ + l / NQ * XQ + l % NQ;
 #pragma unroll
@@ -300,19 +380,19 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
               if (kd == 0) {          // derivatives in direction 1: X kinds 3 (test), 1 (trial), 4 (both)
                 psf_scale<T, NQ, 1, false>(l, xb, x);
                 psf_scale<T, NQ, 1, true>(dl, xb + 3 * XS, x);
-                psf_row<T, N1, false>(tb, x, acc, nr);
+                psf_row<T, N1, N1, false>(tb, x, acc, nr);
                 psf_scale<T, NQ, 1, false>(l, xb + XS, x);
                 psf_scale<T, NQ, 1, true>(dl, xb + 4 * XS, x);
-                psf_row<T, N1, true>(tb, x, acc, nr);
+                psf_row<T, N1, N1, true>(tb, x, acc, nr);
               } else if (kd == 1) {
                 psf_scale<T, NQ, 1, false>(l, xb + 6 * XS, x);
-                psf_row<T, N1, false>(tb, x, acc, nr);
+                psf_row<T, N1, N1, false>(tb, x, acc, nr);
                 psf_scale<T, NQ, 1, false>(l, xb + 7 * XS, x);
-                psf_row<T, N1, true>(tb, x, acc, nr);
+                psf_row<T, N1, N1, true>(tb, x, acc, nr);
               } else {
                 psf_scale<T, NQ, 1, false>(l, xb + (kd == 2 ? 2 : 8) * XS, x);
                 if (kd == 2) psf_scale<T, NQ, 1, true>(dl, xb + 5 * XS, x);
-                psf_row<T, N1, false>(tb, x, acc, nr);
+                psf_row<T, N1, N1, false>(tb, x, acc, nr);
               }
               T* o = Y + ((size_t)(vp * 4 + kd) * CQ + z) * NP * YP + pt * YP + sf32_pair0(N1, ar);
 #pragma unroll
@@ -358,7 +438,7 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
       for (int t = tid; t < 12 * NL; t += C::NT) {
         const int fs = t / NL, q = t - fs * NL;
         T c[20];
-        face_trace(fs >> 1, fs & 1, q, c);
+        psf_face_trace<T, N1>(mv, sW, fs >> 1, fs & 1, q, c);
 #pragma unroll
         for (int j = 0; j < 20; ++j) P[(fs * 20 + j) * NL + q] = c[j];
       }
@@ -367,7 +447,6 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
     for (int w = 0; w < M; ++w) {
       for (int t = tid; t < 4 * 6 * NL; t += C::NT) {
         const int s = t / (6 * NL), fq = t - s * 6 * NL, f = fq / NL, q = fq - f * NL, k = f >> 1, side = f & 1;
-        const int b0 = q / NQ, b1 = q - b0 * NQ, t0 = k == 0 ? 1 : 0;
         // the face's L element sees it at its +1 end: side 1 is this element's +1 face
         T c[2][20];
         if constexpr (CACHED) {
@@ -386,75 +465,13 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
 #pragma unroll
               for (int j = 0; j < 20; ++j) c[sd][j] = P[((f * 2 + sd) * 20 + j) * NL + q];
             } else {
-              face_trace(f, sd, q, c[sd]);
+              psf_face_trace<T, N1>(mv, sW, f, sd, q, c[sd]);
             }
           }
         }
         if (s == 0 && w == 0 && (!physical<3>(c[0], ph.gm1) || !physical<3>(c[1], ph.gm1)))
           atomicOr(status, ST_NONPHYSICAL);
-        const int wf = w == 0 || w == M - 1 ? w : w == 1 + k ? 1 : w == 1 + t0 ? 2 : 3;   // w in the face's frame
-        const T mkk = k == 0 ? tb.met[0] : k == 1 ? tb.met[1] : tb.met[2];
-        const T mt0 = k == 0 ? tb.met[1] : tb.met[0], mt1 = k == 2 ? tb.met[1] : tb.met[2];
-        T wb0 = T(0), wb1 = T(0);
-#pragma unroll
-        for (int b = 0; b < NQ; ++b) {
-          if (b0 == b) wb0 = tb.w[b];
-          if (b1 == b) wb1 = tb.w[b];
-        }
-        const T fw = (k == 0 ? tb.faceJ[0] : k == 1 ? tb.faceJ[1] : tb.faceJ[2]) * wb0 * wb1;
-        const T sg = side ? fw : -fw;
-        T* o = Jf + (size_t)f * M * 8 * NL + q;            // + (v * 8 + kind) * NL
-        if (s == 0) {
-          S u[2][M], g[2][M][3];
-#pragma unroll
-          for (int sd = 0; sd < 2; ++sd)
-#pragma unroll
-            for (int v = 0; v < M; ++v) {
-              u[sd][v] = S(c[sd][v], ((sd == 0) == (side == 1) && v == wf) ? T(1) : T(0));
-#pragma unroll
-              for (int j = 0; j < 3; ++j) g[sd][v][j] = S(c[sd][5 + 3 * v + j], T(0));
-            }
-          S fp[M], mL[3], eL[3], mR[3], eR[3];
-          face_point_core<3, 0, S, T>(u[0], g[0], u[1], g[1], ph, fp, mL, eL, mR, eR);
-          const T lf = sg * ph.eta * mkk * T(0.125);
-          T m[3], en[3];
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            m[j] = side ? mL[j].d : mR[j].d;
-            en[j] = side ? eL[j].d : eR[j].d;
-          }
-#pragma unroll
-          for (int v = 0; v < M; ++v) {
-            const int j = v == 0 || v == M - 1 ? 0 : v - 1;
-            o[(v * 8 + 0) * NL] = sg * fp[v].d;
-            // normal column of K(uL) jump + K(uR) jump (twice the halves)
-            o[(v * 8 + 1) * NL] = v == 0 ? T(0)
-                                : v == M - 1 ? lf * T(2) * (eL[0].d + eR[0].d)
-                                             : lf * (v == 1 ? T(8) / T(3) : T(2)) * (mL[j].d + mR[j].d);
-            // the own dual tensor (visc_rank1): rows n, t0, t1, E
-            const T dn = v == 0 ? T(0) : v == 1 ? (T(4) / T(3)) * m[0] : v == 2 ? m[1] : v == 3 ? m[2] : en[0];
-            const T d0 = v == 1 ? m[1] : v == 2 ? (T(-2) / T(3)) * m[0] : v == 4 ? en[1] : T(0);
-            const T d1 = v == 1 ? m[2] : v == 3 ? (T(-2) / T(3)) * m[0] : v == 4 ? en[2] : T(0);
-            o[(v * 8 + 5) * NL] = -fw * mkk * dn;
-            o[(v * 8 + 6) * NL] = -fw * mt0 * d0;
-            o[(v * 8 + 7) * NL] = -fw * mt1 * d1;
-          }
-        } else {
-          T u[M], g[M][3], F[M];
-#pragma unroll
-          for (int v = 0; v < M; ++v) {
-            u[v] = side ? c[0][v] : c[1][v];
-            F[v] = T(0);
-#pragma unroll
-            for (int j = 0; j < 3; ++j) g[v][j] = (v == wf && j == s - 1) ? T(1) : T(0);
-          }
-          Prim<3, T> pr;
-          primitives<3, T, T>(u, ph, pr);
-          add_visc_col<3, 0, T, T>(pr, g, T(0.5), F, ph);
-          const T sc = sg * (s == 1 ? mkk : s == 2 ? mt0 : mt1);
-#pragma unroll
-          for (int v = 0; v < M; ++v) o[(v * 8 + 1 + s) * NL] = sc * F[v];
-        }
+        psf_face_jac<T, N1, true>(tb, ph, c, k, side, q, s, w, Jf + (size_t)f * M * 8 * NL + q);
       }
       __syncthreads();
       for (int v = 0; v < M; ++v) {      // v in each face's own frame: see the last loop for the rows
@@ -473,10 +490,10 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
           for (int b = 0; b < N1; ++b) acc[b] = T(0);
           psf_scale<T, NQ, NQ, false>(l, j + kind * NL, x);
           if (arr == 0) psf_scale<T, NQ, NQ, true>(dl, j + 6 * NL, x);
-          psf_row<T, N1, false>(tb, x, acc, N1);
+          psf_row<T, N1, N1, false>(tb, x, acc, N1);
           if (arr == 0) {
             psf_scale<T, NQ, NQ, false>(l, j + 3 * NL, x);
-            psf_row<T, N1, true>(tb, x, acc, N1);
+            psf_row<T, N1, N1, true>(tb, x, acc, N1);
           }
           T* o = F1 + ((size_t)(f * 6 + arr) * N2 + at * N1) * XQ + b1;
 #pragma unroll
@@ -498,12 +515,12 @@ __global__ void __launch_bounds__(Psf<T, N1, VG, VP, CQ, CACHED>::NT, sizeof(T) 
 #pragma unroll
             for (int q = 0; q < NQ; ++q) x[q] = l[q] * (fb[q] + n * n * fb[FS + q]);
             psf_scale<T, NQ, 1, true>(dl, fb + 5 * FS, x);
-            psf_row<T, N1, false>(tb, x, acc, nr);
+            psf_row<T, N1, N1, false>(tb, x, acc, nr);
             psf_scale<T, NQ, 1, false>(l, fb + 3 * FS, x);
-            psf_row<T, N1, true>(tb, x, acc, nr);
+            psf_row<T, N1, N1, true>(tb, x, acc, nr);
           } else {
             psf_scale<T, NQ, 1, false>(l, fb + (out == 1 ? 2 : 4) * FS, x);
-            psf_row<T, N1, false>(tb, x, acc, nr);
+            psf_row<T, N1, N1, false>(tb, x, acc, nr);
           }
           T* o = A + (size_t)(f * 3 + out) * NP * YP + pt * YP + sf32_pair0(N1, ar);
 #pragma unroll

@@ -1,5 +1,5 @@
-"""The sum-factorised block probe of 3-D P_p meshes, every order of both
-precisions, FP32 with the primal traces cached and interpolated, on meshes with
+"""The sum-factorised block probe of 3-D P_p meshes and its neighbour blocks at
+every coarse order, every order of both precisions, FP32 with the primal traces cached and interpolated, on meshes with
 unequal directions (two elements in one, whose neighbours coincide), against
 the general FP64 probe kernel (DG_PROBE_SIMT=1).
 
@@ -26,14 +26,17 @@ def _lib():
     B.load()
 
 
-def _diag(m, cfg, W, precision):
-    pmg = B.PMG(m, W, 1.5 / wl.time_step(cfg), B.pmg_opts((cfg["p"], 0), precision=precision, cycle=B.CYCLE_FMG))
-    nb = m.m * m.nm
-    D = torch.empty((m.E, nb, nb), dtype=torch.float64 if precision == B.PREC_FP64 else torch.float32, device="cuda")
+def _blocks(m, cfg, W, precision, pc):
+    pmg = B.PMG(m, W, 1.5 / wl.time_step(cfg), B.pmg_opts((cfg["p"], pc), precision=precision, cycle=B.CYCLE_FMG))
+    nb, nbc = m.m * m.nm, m.m * wl.n_modes(pc, 3, "P")
+    dt = torch.float64 if precision == B.PREC_FP64 else torch.float32
+    D = torch.empty((m.E, nb, nb), dtype=dt, device="cuda")
+    O = torch.empty((m.E, 6, nbc, nbc), dtype=dt, device="cuda")
     pmg.export_blocks(0, B.BLOCKS_DIAG, D)
+    pmg.export_blocks(1, B.BLOCKS_NEIGHBOUR, O)
     assert m.status_sync() == B.DG_OK
     pmg.close()
-    return D.cpu().numpy().astype(np.float64)
+    return [x.cpu().numpy().astype(np.float64) for x in (D, O)]
 
 
 @pytest.mark.parametrize("n", [(2, 3, 5), (4, 3, 2)])
@@ -43,12 +46,13 @@ def test_probe_sf_matches_general_kernel(p, n, monkeypatch):
     W = torch.from_numpy(wl.perturbed_state(cfg, amp=0.02)).cuda()
     m = B.Mesh.from_workload(wl.mesh_desc(cfg), wl.physics(cfg))
     monkeypatch.setenv("DG_PROBE_SIMT", "1")
-    ref = _diag(m, cfg, W, B.PREC_FP64)
+    ref = [_blocks(m, cfg, W, B.PREC_FP64, pc) for pc in range(p)]
     monkeypatch.setenv("DG_PROBE_SIMT", "0")
     for what, precision, no_cache, bar in (("fp64", B.PREC_FP64, "0", 1e-12), ("fp32 cached", B.PREC_MIXED, "0", 5e-6),
                                            ("fp32 interpolated", B.PREC_MIXED, "1", 5e-6)):
         monkeypatch.setenv("DG_PMG_NO_PRIMAL_CACHE", no_cache)
-        D = _diag(m, cfg, W, precision)
-        err = float(np.abs(D - ref).max() / np.abs(ref).max())
-        print("p=%d %s %s: %.2e" % (p, n, what, err))
-        assert err <= bar
+        for pc in range(p):
+            got = _blocks(m, cfg, W, precision, pc)
+            err = [float(np.abs(a - b).max() / np.abs(b).max()) for a, b in zip(got, ref[pc])]
+            print("p=%d pc=%d %s %s: %.2e %.2e" % (p, pc, n, what, *err))
+            assert max(err) <= bar

@@ -115,19 +115,16 @@ template <class T>
 cudaError_t MG<T>::smooth(int l, const T* b, T* x, int nu, cudaStream_t st) {
   Level<T>& L = lv[l];
   Krylov<T>& K = L.kr;
-  if constexpr (std::is_same<T, float>::value) {
-    // inherited FP32/BF16 coarse levels: the whole call in one persistent launch
-    const bool ilu = bilu && l == (int)lv.size() - 1;
-    if (l >= 1 && L.coop.ok && !ilu && (L.Dinv16 || (L.inv_t && L.co_t))) {
-      if (nu == 0) return cudaSuccess;
-      return launch_coop_smoother(L.coop, L.Dinv, L.Dop, L.O, L.Dinv16, L.Dop16, L.O16, mesh->face_nbr(),
-                                  mesh->nfaces(), b, x, nu, K, L.cbuf, mesh->status, coop_extra, L.nb, mesh->E, st);
-    }
+  const bool ilu = bilu && l == (int)lv.size() - 1;   // block ILU(0) on the coarsest level
+  // inherited coarse levels: the whole call in one persistent launch
+  if (l >= 1 && L.coop.ok && !ilu && (L.Dinv16 || (L.inv_t && L.co_t))) {
+    if (nu == 0) return cudaSuccess;
+    return launch_coop_smoother(L.coop, L.Dinv, L.Dop, L.O, L.Dinv16, L.Dop16, L.O16, mesh->face_nbr(),
+                                mesh->nfaces(), b, x, nu, K, L.cbuf, mesh->status, coop_extra, L.nb, mesh->E, st);
   }
   CKE(op(l, x, L.r, st));
   CKE(launch_axpby<T>(L.N, 1.0, b, -1.0, L.r, st));           // r = b - A x
   CKE(K.start(L.r, st));
-  const bool ilu = bilu && l == (int)lv.size() - 1;   // block ILU(0) on the coarsest level
   for (int j = 0; j < nu; ++j) {
     if (ilu)
       CKE(launch_bilu_apply<T>(*this, K.Vj(j), K.Zj(j), st));
@@ -226,13 +223,14 @@ static dg_status alloc_mg(dg_pmg h, MG<T>& mg) {
     L.bs = (size_t)L.nb * inv_ld<T>(L.nb);
     CK(dalloc(mg.allocs, (void**)&L.Dinv, sizeof(T) * (size_t)M.E * L.bs, &h->block_bytes));
     if (l >= 1) {
-      // coarse blocks column-major when the FP32 neighbour blocks come from
-      // probe_nbr_kernel (decided here once: the captured graph relies on it)
+      // coarse blocks column-major when the neighbour blocks come from a kernel
+      // that writes them so (decided here once: the captured graph relies on it)
       // (the column-major mat-vec runs one thread per block and 16 bytes of rows: at most 256 per element)
       // or, on triangles, from the coloured probe (which writes either layout)
       const int tpb1 = (1 + M.nfaces()) * (inv_ld<T>(mg.lv[1].nb) / (int)(16 / sizeof(T)));
-      L.co_t = std::is_same<T, float>::value && tpb1 <= 256 &&
-                       (M.kind == DG_MESH_TRI || probe_nbr_colmajor_ok(M, mg.lv[1].nm)) ? 1 : 0;
+      L.co_t = tpb1 <= 256 && (M.kind == DG_MESH_TRI ||
+                               (std::is_same<T, float>::value ? probe_nbr_colmajor_ok(M, mg.lv[1].nm)
+                                                              : probe_nbr64_colmajor_ok(M, mg.lv[1].nm))) ? 1 : 0;
       L.cs = L.co_t ? L.bs : (size_t)L.nb * L.nb;
       (void)nbl;
       CK(dalloc(mg.allocs, (void**)&L.Dop, sizeof(T) * (size_t)M.E * L.cs, &h->block_bytes));
@@ -254,14 +252,14 @@ static dg_status alloc_mg(dg_pmg h, MG<T>& mg) {
       CK(L.kr.alloc(L.N, nmax));
       h->vector_bytes += L.kr.bytes();
     }
-    // persistent smoother of an inherited FP32 level (column-major or BF16
+    // persistent smoother of an inherited level (column-major or BF16
     // blocks); DG_PMG_NO_COOP=1 keeps the launch-per-operation smoother
     const char* nco = getenv("DG_PMG_NO_COOP");
     const bool bf16 = o.block_storage == DG_STORE_BF16;
-    if (std::is_same<T, float>::value && l >= 1 && o.cycle != DG_CYCLE_BJ && (L.co_t || bf16) &&
+    if (l >= 1 && o.cycle != DG_CYCLE_BJ && (L.co_t || bf16) &&
         !(nco && nco[0] == '1') &&
         !(o.coarse_precond == DG_COARSE_BILU && l == nl - 1)) {
-      CK(plan_coop_smoother(bf16 ? 1 : 0, L.nb, M.nfaces(), M.E, nmax, &L.coop));
+      CK(plan_coop_smoother(bf16 ? COOP_BF16 : std::is_same<T, double>::value ? COOP_FP64 : COOP_FP32, L.nb, M.nfaces(), M.E, nmax, &L.coop));
       if (L.coop.ok) {
         L.coop.nu_max = nmax;
         CK(dalloc(mg.allocs, &L.cbuf.part, L.coop.part_bytes, &h->vector_bytes));

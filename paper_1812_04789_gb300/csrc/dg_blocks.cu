@@ -384,7 +384,7 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
       cudaError_t e = launch_probe_sf(M, W, sigma, D, dstride, st);
       return e != cudaSuccess || !O ? e : launch_nbr_sf(M, W, O, nmc, nbr_colmajor, st);
     }
-    if (!(simt && simt[0] == '1') && probe64_fits(M, O ? nmc : 0))
+    if ((nbr_colmajor || !(simt && simt[0] == '1')) && probe64_fits(M, O ? nmc : 0))   // (layout fixed at setup)
       return launch_probe64(M, W, sigma, D, dstride, O, nmc, nbr_colmajor, st);
   }
   if (std::is_same<T, float>::value && use_tc(M)) {
@@ -408,6 +408,10 @@ template cudaError_t launch_probe_blocks<double>(const Mesh&, const double*, dou
 template cudaError_t launch_probe_blocks<float>(const Mesh&, const float*, float, float*, size_t, float*, int,
                                                 int, float*, size_t, cudaStream_t, const float*, const float*);
 
+bool probe_nbr64_colmajor_ok(const Mesh& M, int nmc) {
+  const char* e = getenv("DG_PROBE_SIMT");
+  return !(e && e[0] == '1') && probe64_fits(M, nmc);
+}
 bool probe_nbr_colmajor_ok(const Mesh& M, int nmc) { return use_tc(M) && probe_nbr_fits(M, nmc); }
 
 // ---------------------------------------------------------------- truncation

@@ -193,8 +193,8 @@ cudaError_t launch_residual_with_slots(const Mesh& M, const double* W, const dou
 // and when O != nullptr the neighbour blocks O[e][2k+side] restricted to the
 // first nmc modes of every variable (nbc x nbc, nbc = m nmc).
 // D[e] starts at D + e * dstride (row-major, row stride nb).  With
-// nbr_colmajor (FP32 only, probe_nbr_colmajor_ok) the neighbour blocks are
-// written column-major by probe_nbr_kernel, else row-major, nbc^2 apart.
+// nbr_colmajor (probe_nbr_colmajor_ok, probe_nbr64_colmajor_ok) the neighbour
+// blocks are written column-major, else row-major, nbc^2 apart.
 // Pv, Pf: cached primal traces of W (FP32, or null).
 template <class T>
 cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t dstride, T* O, int nmc,
@@ -242,6 +242,9 @@ cudaError_t launch_probe_nbr(const Mesh& M, const float* W, float* O, int nmc, i
 // Whether the FP32 neighbour blocks of this mesh come from probe_nbr_kernel
 // (tensor-core tables present, the kernel applies, not disabled by DG_PROBE_SIMT).
 bool probe_nbr_colmajor_ok(const Mesh& M, int nmc);
+// FP64 neighbour blocks: whether launch_probe_blocks can write them column-major
+// (nbr_sf_kernel or probe64_kernel, not disabled by DG_PROBE_SIMT).
+bool probe_nbr64_colmajor_ok(const Mesh& M, int nmc);
 
 // Batched in-place inverse of nblk row-major blocks of size nb starting bstride
 // elements apart (bstride >= nb * inv_ld(nb)).  *transposed = 1 when the
@@ -347,7 +350,8 @@ struct CoopPlan {
   int ok = 0, grid = 0, chunk = 0, epc = 0, tpe = 0, ns = 1, pre = 0, res = 0, nu_max = 0;
   size_t smem = 0, part_bytes = 0, z_bytes = 0;
 };
-cudaError_t plan_coop_smoother(int bf16, int nb, int nf, int E, int nu, CoopPlan* plan);
+enum CoopStore { COOP_FP32, COOP_BF16, COOP_FP64 };   // the blocks; vectors FP32, FP32, FP64
+cudaError_t plan_coop_smoother(int store, int nb, int nf, int E, int nu, CoopPlan* plan);
 // Exchange buffers of a level (zero when allocated): the CTAs' partial sums,
 // the published directions and the epoch word.  Launches that share them are
 // ordered on one stream.
@@ -358,13 +362,17 @@ struct CoopBuffers {
 };
 // One SMOOTH call (nu >= 1 GMRES(BJ) iterations from x on A x = b, Algorithm 2)
 // in one cooperative launch: FP32 vectors, blocks column-major in FP32 (inv_ld)
-// or, when Dinv16 is given, BF16 (ld_bf16).  A bounded wait that runs out sets
+// or, when Dinv16 is given, BF16 (ld_bf16); or FP64 vectors and blocks.  A bounded wait that runs out sets
 // ST_TIMEOUT in *status.  extra > 0 makes every exchange wait for a CTA that
 // does not exist (the wait then runs out).
 cudaError_t launch_coop_smoother(const CoopPlan& pl, const float* Dinv, const float* Dop, const float* O,
                                  const unsigned short* Dinv16, const unsigned short* Dop16, const unsigned short* O16,
                                  const int* nbr, int nf, const float* b, float* x, int nu, Krylov<float>& K,
                                  const CoopBuffers& buf, int* status, int extra, int nb, int E, cudaStream_t st);
+cudaError_t launch_coop_smoother(const CoopPlan& pl, const double* Dinv, const double* Dop, const double* O,
+                                 const unsigned short*, const unsigned short*, const unsigned short*, const int* nbr,
+                                 int nf, const double* b, double* x, int nu, Krylov<double>& K, const CoopBuffers& buf,
+                                 int* status, int extra, int nb, int E, cudaStream_t st);
 
 template <class T>
 struct Level {

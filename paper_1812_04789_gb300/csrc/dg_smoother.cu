@@ -41,10 +41,15 @@
 // addition carried along, 48 bits) and in a fixed order, rounded to FP32 at the
 // end; all CTAs hold identical scalars and the final x += Z y needs no
 // exchange.  FP64 sums cost more than a hop (GB300 has two FP64 lanes per SM).  The arithmetic inside a CTA is FP32.  A warp of its own
-// keeps the Hessenberg matrix, the Givens rotations and the small
-// least-squares solve off the critical path.
+// keeps the Hessenberg matrix, the Givens rotations (behind the next
+// exchange's wait) and the small least-squares solve off the critical path;
+// one warp takes the scalars of an exchange.
 // 16^3 elements, p_fine = 4 (us per call): p = 2, nu = 10: 880 -> 765;
 // p = 1, nu = 10: 400 -> 188; p = 0, nu = 30: 690 -> 290.
+// FP64 handles run the same kernel on FP64 vectors and blocks, the sums over the
+// CTAs plain.  Bound by the FP64 pipe at p = 2 (the block-sparse product), by the
+// exchanges below; the launch-per-operation smoother spent half of its time
+// on kernels of 2 to 5 us.  9 x 10 x 12, p = 3: FP64 step 116 -> 85 ms.
 //
 // Every wait is bounded (2 s of the global timer): on expiry the CTA sets
 // ST_TIMEOUT in the mesh status word and returns, and the other CTAs see the
@@ -83,6 +88,20 @@ struct Col16<float> {
   }
 };
 template <>
+struct Col16<double> {
+  static constexpr int R = 2;
+  template <bool RES>
+  __device__ __forceinline__ static void load(const double* p, double* v) {
+    if constexpr (RES) {
+      const double2 t = *reinterpret_cast<const double2*>(p);
+      v[0] = t.x;
+      v[1] = t.y;
+    } else {
+      asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0,%1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p));
+    }
+  }
+};
+template <>
 struct Col16<unsigned short> {
   static constexpr int R = 8;
   template <bool RES>
@@ -101,40 +120,10 @@ struct Col16<unsigned short> {
   }
 };
 
-template <class S>
-struct CoopArgs {
-  const S* Dinv;        // inverse diagonal blocks, column-major, leading dimension ld, nb * ld apart
-  const S* Dop;         // inherited diagonal blocks (same layout)
-  const S* O;           // inherited neighbour blocks [E][nf] (same layout)
-  const int* nbr;       // [E][nf]
-  const float* b;
-  float* x;
-  unsigned long long* zx;   // [N] (value, epoch) of the direction z_j
-  uint4* px;            // [2][ni][grid + 1] (s, epoch, t, epoch): the CTAs' partial sums
-  uint4* sums;          // [2][ni] their sums over the CTAs
-  unsigned* epoch;      // first free epoch - 1
-  int* status;          // mesh status word (ST_TIMEOUT)
-  int* kflag;           // Krylov status bits (ST_NONFINITE)
-  int nu, nb, ld, E, chunk, epc, tpe, ns, ni, extra;
-  int pre;              // ask for the blocks ahead of their use (a level that L2 holds)
-};
-
-constexpr int COOP_WORK = 512;                  // threads that compute
-constexpr int COOP_THREADS = COOP_WORK + 32;    // and the scalar warp
-
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
-}
-__device__ __forceinline__ unsigned long long ld_val(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_val(unsigned long long* p, float f, unsigned ep) {
-  const unsigned long long v = ((unsigned long long)ep << 32) | __float_as_uint(f);
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ uint4 ld_pair(const uint4* p) {
   uint4 v;
@@ -144,11 +133,91 @@ __device__ __forceinline__ uint4 ld_pair(const uint4* p) {
                : "memory");
   return v;
 }
-__device__ __forceinline__ void st_pair(uint4* p, float s, float t, unsigned ep) {
-  asm volatile("st.volatile.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(__float_as_uint(s)), "r"(ep),
-               "r"(__float_as_uint(t)), "r"(ep)
-               : "memory");
+__device__ __forceinline__ void st_pair(uint4* p, unsigned x, unsigned y, unsigned ep) {
+  asm volatile("st.volatile.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(x), "r"(ep), "r"(y), "r"(ep) : "memory");
 }
+
+// What travels between the CTAs, every 32-bit word of a value beside its epoch:
+// Z a direction's entry, P a pair of sums (s, t).  An FP64 value is two words
+// with an epoch each, so neither needs more than 8 bytes to arrive at once.
+template <class V>
+struct Xch;
+template <>
+struct Xch<float> {
+  using Z = unsigned long long;
+  using P = uint4;
+  using V2 = float2;
+  __device__ __forceinline__ static Z ld(const Z* p) {
+    Z v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ static bool has(Z v, unsigned ep) { return (unsigned)(v >> 32) == ep; }
+  __device__ __forceinline__ static float val(Z v) { return __uint_as_float((unsigned)v); }
+  __device__ __forceinline__ static void st(Z* p, float f, unsigned ep) {
+    const Z v = ((Z)ep << 32) | __float_as_uint(f);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+  }
+  __device__ __forceinline__ static P ldp(const P* p) { return ld_pair(p); }
+  __device__ __forceinline__ static bool hasp(const P& q, unsigned ep) { return q.y == ep && q.w == ep; }
+  __device__ __forceinline__ static V2 valp(const P& q) { return make_float2(__uint_as_float(q.x), __uint_as_float(q.z)); }
+  __device__ __forceinline__ static void stp(P* p, float s, float t, unsigned ep) {
+    st_pair(p, __float_as_uint(s), __float_as_uint(t), ep);
+  }
+};
+struct Pair64 {
+  uint4 s, t;
+};
+template <>
+struct Xch<double> {
+  using Z = uint4;
+  using P = Pair64;
+  using V2 = double2;
+  __device__ __forceinline__ static Z ld(const Z* p) { return ld_pair(p); }
+  __device__ __forceinline__ static bool has(const Z& v, unsigned ep) { return v.y == ep && v.w == ep; }
+  __device__ __forceinline__ static double val(const Z& v) { return __hiloint2double((int)v.z, (int)v.x); }
+  __device__ __forceinline__ static void st(Z* p, double f, unsigned ep) {
+    st_pair(p, (unsigned)__double2loint(f), (unsigned)__double2hiint(f), ep);
+  }
+  __device__ __forceinline__ static P ldp(const P* p) { return {ld_pair(&p->s), ld_pair(&p->t)}; }
+  __device__ __forceinline__ static bool hasp(const P& q, unsigned ep) { return has(q.s, ep) && has(q.t, ep); }
+  __device__ __forceinline__ static V2 valp(const P& q) { return make_double2(val(q.s), val(q.t)); }
+  __device__ __forceinline__ static void stp(P* p, double s, double t, unsigned ep) {
+    st(&p->s, s, ep);
+    st(&p->t, t, ep);
+  }
+};
+// the vectors' type over blocks stored as S
+template <class S>
+struct CoopVal {
+  using V = float;
+};
+template <>
+struct CoopVal<double> {
+  using V = double;
+};
+
+template <class S>
+struct CoopArgs {
+  using V = typename CoopVal<S>::V;
+  const S* Dinv;        // inverse diagonal blocks, column-major, leading dimension ld, nb * ld apart
+  const S* Dop;         // inherited diagonal blocks (same layout)
+  const S* O;           // inherited neighbour blocks [E][nf] (same layout)
+  const int* nbr;       // [E][nf]
+  const V* b;
+  V* x;
+  typename Xch<V>::Z* zx;     // [N] the direction z_j
+  typename Xch<V>::P* px;     // [2][ni][grid + 1] the CTAs' partial sums
+  typename Xch<V>::P* sums;   // [2][ni] their sums over the CTAs
+  unsigned* epoch;      // first free epoch - 1
+  int* status;          // mesh status word (ST_TIMEOUT)
+  int* kflag;           // Krylov status bits (ST_NONFINITE)
+  int nu, nb, ld, E, chunk, epc, tpe, ns, ni, extra;
+  int pre;              // ask for the blocks ahead of their use (a level that L2 holds)
+};
+
+constexpr int COOP_WORK = 512;                  // threads that compute
+constexpr int COOP_THREADS = COOP_WORK + 32;    // and the scalar warp
 
 // A bounded wait: expired() is called once per failed poll and looks at the
 // clock and the status word every 64th time.
@@ -173,113 +242,220 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// (h, l) += x with the rounding error of the addition kept in l
+// (h, l) += x, FP32 with the rounding error of the addition kept in l
+__device__ __forceinline__ void two_add(double& h, double&, double x) { h += x; }
 __device__ __forceinline__ void two_add(float& h, float& l, float x) {
   const float s = h + x, b = s - h;
   l += (h - (s - b)) + (x - b);
   h = s;
 }
 
+// Sums of fs and ft over a warp: the first exchange leaves fs to the lower and
+// ft to the upper half, so five additions do for both.
+template <class V>
+__device__ __forceinline__ void warp_sum2(V& fs, V& ft) {
+  const bool up = threadIdx.x & 16;
+  V a = (up ? ft : fs) + __shfl_xor_sync(0xffffffffu, up ? fs : ft, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  fs = __shfl_sync(0xffffffffu, a, 0);
+  ft = __shfl_sync(0xffffffffu, a, 16);
+}
+
 // The CTA's partial sums of exchange j, a warp per item: (V_i.v_j, V_i.w) for
-// i <= j and (w.w, 0), in FP32 (a lane's rows, then the warp's butterfly),
+// i <= j and (w.w, 0), in the vectors' precision (a lane's rows, then the warp's butterfly),
 // published as they are ready; w = null (the closing exchange): zeros for w.
-__device__ void publish_dots(int j, const float* Vs, int ldv, const float* w, int rows, uint4* out, int stride,
+template <class V>
+__device__ void publish_dots(int j, const V* Vs, int ldv, const V* w, int rows, typename Xch<V>::P* out, int stride,
                              unsigned ep) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp >= COOP_WORK / 32) return;
-  const float* vj = Vs + (size_t)j * ldv;
+  const V* vj = Vs + (size_t)j * ldv;
   for (int i = warp; i < j + 2; i += COOP_WORK / 32) {
-    const float* v = i <= j ? Vs + (size_t)i * ldv : w;
-    float fs = 0.f, ft = 0.f;
+    const V* v = i <= j ? Vs + (size_t)i * ldv : w;
+    V fs = V(0), ft = V(0);
     if (v) {
       for (int r = lane; r < rows; r += 32) {
-        const float x = v[r];
+        const V x = v[r];
         if (i <= j) {
-          fs = fmaf(x, vj[r], fs);
-          if (w) ft = fmaf(x, w[r], ft);
+          fs = fma(x, vj[r], fs);
+          if (w) ft = fma(x, w[r], ft);
         } else {
-          fs = fmaf(x, x, fs);
+          fs = fma(x, x, fs);
         }
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      fs += __shfl_xor_sync(0xffffffffu, fs, o);
-      ft += __shfl_xor_sync(0xffffffffu, ft, o);
-    }
-    if (lane == 0) st_pair(out + (size_t)i * stride, fs, ft, ep);
+    warp_sum2(fs, ft);
+    if (lane == 0) Xch<V>::stp(out + (size_t)i * stride, fs, ft, ep);
   }
 }
 
 // st[i] = the sums over all CTAs of the items i < ni of an exchange: CTA i mod G
 // owns item i, a warp of it polls the G partials in[i stride + c] (5 loads of a
-// lane at once), adds them in two-float arithmetic, a lane's CTAs and then the
+// lane at once), adds them (FP32: in two-float arithmetic), a lane's CTAs and then the
 // lanes by a butterfly, and publishes the sum, and one warp of every CTA
 // polls the ni sums.  Two hops of little traffic: one hop, with every CTA
 // reading all G x ni partials, saturated the L2 with polls and took 8 us.
 // False where a wait ran out.
-__device__ bool gather_dots(const uint4* in, int stride, int ni, int G, uint4* sums, unsigned ep, int* status,
-                            float2* st) {
+template <class V>
+__device__ bool gather_dots(const typename Xch<V>::P* in, int stride, int ni, int G, typename Xch<V>::P* sums,
+                            unsigned ep, int* status, typename Xch<V>::V2* st) {
+  using X = Xch<V>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, C = gridDim.x;
   bool ok = true;
   if (warp >= COOP_WORK / 32) return ok;
   Wait wt;
   // (the owned items i = blockIdx.x + k C, shared out over the warps; warp 0 collects)
   for (int i = blockIdx.x + (warp - 1) * C; warp > 0 && i < ni; i += (COOP_WORK / 32 - 1) * C) {
-    float hs = 0.f, ls = 0.f, ht = 0.f, lt = 0.f;
+    V hs = V(0), ls = V(0), ht = V(0), lt = V(0);
     for (int c0 = lane; c0 < G; c0 += 160) {
-      uint4 q[5];
+      typename X::P q[5];
 #pragma unroll
-      for (int u = 0; u < 5; ++u) q[u] = ld_pair(in + (size_t)i * stride + min(c0 + 32 * u, G - 1));
+      for (int u = 0; u < 5; ++u) q[u] = X::ldp(in + (size_t)i * stride + min(c0 + 32 * u, G - 1));
 #pragma unroll
       for (int u = 0; u < 5; ++u) {
         if (c0 + 32 * u >= G) continue;
-        while (ok && (q[u].y != ep || q[u].w != ep)) {
+        while (ok && !X::hasp(q[u], ep)) {
           if (wt.expired(status)) ok = false;
-          q[u] = ld_pair(in + (size_t)i * stride + c0 + 32 * u);
+          q[u] = X::ldp(in + (size_t)i * stride + c0 + 32 * u);
         }
-        two_add(hs, ls, __uint_as_float(q[u].x));
-        two_add(ht, lt, __uint_as_float(q[u].z));
+        const typename X::V2 v = X::valp(q[u]);
+        two_add(hs, ls, v.x);
+        two_add(ht, lt, v.y);
       }
     }
+    if constexpr (std::is_same<V, double>::value) {
+      warp_sum2(hs, ht);
+    } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float a = __shfl_xor_sync(0xffffffffu, hs, o), b = __shfl_xor_sync(0xffffffffu, ls, o);
-      const float c = __shfl_xor_sync(0xffffffffu, ht, o), d = __shfl_xor_sync(0xffffffffu, lt, o);
-      two_add(hs, ls, a);
-      ls += b;
-      two_add(ht, lt, c);
-      lt += d;
+      for (int o = 16; o > 0; o >>= 1) {
+        const V a = __shfl_xor_sync(0xffffffffu, hs, o), b = __shfl_xor_sync(0xffffffffu, ls, o);
+        const V c = __shfl_xor_sync(0xffffffffu, ht, o), d = __shfl_xor_sync(0xffffffffu, lt, o);
+        two_add(hs, ls, a);
+        ls += b;
+        two_add(ht, lt, c);
+        lt += d;
+      }
     }
-    if (__all_sync(0xffffffffu, ok) && lane == 0) st_pair(sums + i, hs + ls, ht + lt, ep);
+    if (__all_sync(0xffffffffu, ok) && lane == 0) X::stp(sums + i, hs + ls, ht + lt, ep);
   }
   if (warp == 0) {
     for (int i = lane; i < ni; i += 32) {
-      uint4 q = ld_pair(sums + i);
-      while (ok && (q.y != ep || q.w != ep)) {
+      typename X::P q = X::ldp(sums + i);
+      while (ok && !X::hasp(q, ep)) {
         if (wt.expired(status)) ok = false;
-        q = ld_pair(sums + i);
+        q = X::ldp(sums + i);
       }
-      st[i] = make_float2(__uint_as_float(q.x), __uint_as_float(q.z));
+      st[i] = X::valp(q);
     }
   }
   return ok;
+}
+
+// The scalars of exchange j (see the head of the file), by one warp from the
+// sums in st: FP64 square roots and sums in all seventeen warps would cost more
+// than the exchange (two FP64 lanes per SM).  FP64 takes a power of two as rho
+// (any scale will do), whose reciprocal is exact.
+template <class V>
+struct Scal {
+  V beta, ib, hj, rho, ir;
+  int fine, bad;
+};
+template <class V>
+__device__ void exchange_scalars(const typename Xch<V>::V2* st, int j, Scal<V>* sc) {
+  const int lane = threadIdx.x & 31;
+  V ss = V(0), sq = V(0), tq = V(0), none = V(0);
+  for (int i = lane; i < j; i += 32) {
+    const typename Xch<V>::V2 q = st[i];
+    ss = fma(q.x, q.x, ss);
+    sq = fma(q.x, q.y, sq);
+    tq = fma(q.y, q.y, tq);
+  }
+  warp_sum2(ss, sq);
+  warp_sum2(tq, none);
+  const V be2 = st[j].x - ss, ww = st[j + 1].x;
+  const bool fine = be2 > V(0) && isfinite(be2);
+  V beta = V(0), ib = V(0);
+  if (fine) {
+    if constexpr (std::is_same<V, double>::value) {
+      ib = rsqrt(be2);
+      beta = be2 * ib;
+    } else {
+      beta = sqrtf(be2);
+      ib = 1.f / beta;
+    }
+  }
+  const V hj = (st[j].y - sq) * ib, est = fmax(ww - tq - hj * hj, V(1e-6) * ww);
+  V rho = V(1), ir = V(1);
+  if (est > V(0) && isfinite(est)) {
+    if constexpr (std::is_same<V, double>::value) {
+      const int e = ((__double2hiint(est) >> 20) - 1023) >> 1;   // est is normal: |e| <= 512
+      rho = __hiloint2double((1023 + e) << 20, 0);
+      ir = __hiloint2double((1023 - e) << 20, 0);
+    } else {
+      rho = sqrtf(est);
+      ir = 1.f / rho;
+    }
+  }
+  if (lane == 0) {
+    sc->beta = beta;
+    sc->ib = ib;
+    sc->hj = hj;
+    sc->rho = rho;
+    sc->ir = ir;
+    sc->fine = fine;
+    sc->bad = !fine && !isfinite(be2);
+  }
+}
+
+// Column k of the Hessenberg matrix, complete, through the rotations before it and one of its own (one lane)
+template <class V>
+__device__ void rotate_column(V* H, int ldh, int k, V* cs, V* sn, V* g) {
+  V* h = H + (size_t)k * ldh;
+  V p = h[0];
+  for (int i = 0; i < k; ++i) {
+    const V q = h[i + 1];
+    h[i] = cs[i] * p + sn[i] * q;
+    p = -sn[i] * p + cs[i] * q;
+  }
+  const V q = h[k + 1];
+  V c = V(1), sv = V(0);
+  if constexpr (std::is_same<V, double>::value) {
+    const V r2 = p * p + q * q;
+    if (r2 > V(0)) {
+      const V ir = rsqrt(r2);
+      c = p * ir;
+      sv = q * ir;
+    }
+  } else {
+    const V rr = hypotf(p, q);
+    if (rr != 0.f) {
+      c = p / rr;
+      sv = q / rr;
+    }
+  }
+  cs[k] = c;
+  sn[k] = sv;
+  h[k] = c * p + sv * q;
+  g[k + 1] = -sv * g[k];
+  g[k] = c * g[k];
 }
 
 // The inputs of the block-sparse product for the CTA's elements p0 .. p0 + nl:
 // xs[el][who][nb], who = 0 the element itself, 1 + s its neighbour on face s.
 // own = null: from the vector in (no epochs); else own rows from `own`
 // (shared memory) and the others' from zx, polled for epoch ep.
+template <class V>
 __device__ bool stage_inputs(const int* src, int nsrc, int p0, int nl, int nb, float inv_nb, int e_beg, int ne,
-                             const float* in, const float* own, const unsigned long long* zx, unsigned ep,
-                             int* status, float* xs) {
+                             const V* in, const V* own, const typename Xch<V>::Z* zx, unsigned ep, int* status, V* xs) {
+  using X = Xch<V>;
   bool ok = true;
   if (threadIdx.x >= COOP_WORK) return ok;
   Wait wt;
   const int n = nl * nsrc * nb;
   for (int t0 = threadIdx.x; t0 < n; t0 += 4 * COOP_WORK) {
-    unsigned long long v[4];
-    const unsigned long long* ad[4];
+    typename X::Z v[4];
+    const typename X::Z* ad[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int t = t0 + u * COOP_WORK;
@@ -293,17 +469,17 @@ __device__ bool stage_inputs(const int* src, int nsrc, int p0, int nl, int nb, f
         xs[t] = own[(e - e_beg) * nb + j];
       } else {
         ad[u] = zx + (size_t)e * nb + j;
-        v[u] = ld_val(ad[u]);
+        v[u] = X::ld(ad[u]);
       }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (!ad[u]) continue;
-      while (ok && (unsigned)(v[u] >> 32) != ep) {
+      while (ok && !X::has(v[u], ep)) {
         if (wt.expired(status)) ok = false;
-        v[u] = ld_val(ad[u]);
+        v[u] = X::ld(ad[u]);
       }
-      xs[t0 + u * COOP_WORK] = __uint_as_float((unsigned)v[u]);
+      xs[t0 + u * COOP_WORK] = X::val(v[u]);
     }
   }
   return ok;
@@ -313,21 +489,22 @@ __device__ bool stage_inputs(const int* src, int nsrc, int p0, int nl, int nb, f
 // flight together.  The last, shorter run reads the last column again (times
 // zero): with a test around each load, or a loop over the remaining columns,
 // every load waits for the one before it.
-template <class S, bool RES>
-__device__ __forceinline__ void col_run(const S* B, int nb, int ld, const float* x, float* acc) {
-  constexpr int R = Col16<S>::R, U = 48 / R;
+template <class S, bool RES, class V>
+__device__ __forceinline__ void col_run(const S* B, int nb, int ld, const V* x, V* acc) {
+  constexpr int R = Col16<S>::R, U = sizeof(V) == 8 ? 12 : 48 / R;
   for (int c0 = 0; c0 < nb; c0 += U) {
-    float v[U][R], xv[U];
+    V v[U][R], xv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int c = min(c0 + u, nb - 1);
       Col16<S>::template load<RES>(B + (size_t)c * ld, v[u]);
-      xv[u] = c0 + u < nb ? x[c] : 0.f;
+      xv[u] = c0 + u < nb ? x[c] : V(0);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
+      if (sizeof(V) == 4 || c0 + u < nb)     // (FP64: its pipe is the limit)
 #pragma unroll
-      for (int j = 0; j < R; ++j) acc[j] = fmaf(v[u][j], xv[u], acc[j]);
+        for (int j = 0; j < R; ++j) acc[j] = fma(v[u][j], xv[u], acc[j]);
   }
 }
 
@@ -336,12 +513,12 @@ __device__ __forceinline__ void col_run(const S* B, int nb, int ld, const float*
 // one thread takes them all, else block by block with a run of columns in
 // flight.  rev: columns from the last to the first (the next product finds
 // the last ones of this one in L2).
-template <class S, int NF, bool RES>
+template <class S, int NF, bool RES, class V>
 __device__ __forceinline__ void bsr_rows(const S* D, const S* O, int nb, int ld, size_t bs, int b0, int b1, bool rev,
-                                         const float* xe, float* acc) {
+                                         const V* xe, V* acc) {
   constexpr int R = Col16<S>::R, NSRC = 1 + NF;
 #pragma unroll
-  for (int j = 0; j < R; ++j) acc[j] = 0.f;
+  for (int j = 0; j < R; ++j) acc[j] = V(0);
   if (b0 == 0 && b1 == NSRC) {
     const S* base[NSRC];
     base[0] = D;
@@ -350,14 +527,14 @@ __device__ __forceinline__ void bsr_rows(const S* D, const S* O, int nb, int ld,
 #pragma unroll 2
     for (int c_ = 0; c_ < nb; ++c_) {
       const int c = rev ? nb - 1 - c_ : c_;
-      float v[NSRC][R];
+      V v[NSRC][R];
 #pragma unroll
       for (int b = 0; b < NSRC; ++b) Col16<S>::template load<RES>(base[b] + (size_t)c * ld, v[b]);
 #pragma unroll
       for (int b = 0; b < NSRC; ++b) {
-        const float xv = xe[b * nb + c];
+        const V xv = xe[b * nb + c];
 #pragma unroll
-        for (int j = 0; j < R; ++j) acc[j] = fmaf(v[b][j], xv, acc[j]);
+        for (int j = 0; j < R; ++j) acc[j] = fma(v[b][j], xv, acc[j]);
       }
     }
   } else {
@@ -368,24 +545,27 @@ __device__ __forceinline__ void bsr_rows(const S* D, const S* O, int nb, int ld,
 
 template <class S, int NF, bool RES>
 __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S> a) {
+  using V = typename CoopVal<S>::V;
+  using X = Xch<V>;
   constexpr int R = Col16<S>::R, NSRC = 1 + NF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nu = a.nu, ldh = nu + 1, nb = a.nb, ld = a.ld, tpe = a.tpe, ns = a.ns;
   const size_t bs = (size_t)nb * ld;
   const int rmax = a.chunk * nb;
   S* Rs = reinterpret_cast<S*>(smem_raw);             // RES: [chunk][Dop, O.., Dinv]
-  float* Vs = reinterpret_cast<float*>(Rs + (RES ? (size_t)a.chunk * (NSRC + 1) * bs : 0));   // [nu + 1][rmax]
-  float* Zs = Vs + (size_t)ldh * rmax;                // [nu][rmax]
-  float* ws = Zs + (size_t)nu * rmax;                 // [rmax]
-  float* ps = ws + rmax;                              // ns > 1: [ns][rmax] partial products
-  float* xs = ps + (ns > 1 ? (size_t)ns * rmax : 0);  // [epc][NSRC][nb]
-  float* H = xs + (size_t)a.epc * NSRC * nb;          // (nu + 1) x nu, column-major
-  float* cs = H + (size_t)ldh * nu;
-  float* sn = cs + nu;
-  float* g = sn + nu;                                 // nu + 1, then y
+  V* Vs = reinterpret_cast<V*>(Rs + (RES ? (size_t)a.chunk * (NSRC + 1) * bs : 0));   // [nu + 1][rmax]
+  V* Zs = Vs + (size_t)ldh * rmax;                // [nu][rmax]
+  V* ws = Zs + (size_t)nu * rmax;                 // [rmax]
+  V* ps = ws + rmax;                              // ns > 1: [ns][rmax] partial products
+  V* xs = ps + (ns > 1 ? (size_t)ns * rmax : 0);  // [epc][NSRC][nb]
+  V* H = xs + (size_t)a.epc * NSRC * nb;          // (nu + 1) x nu, column-major
+  V* cs = H + (size_t)ldh * nu;
+  V* sn = cs + nu;
+  V* g = sn + nu;                                 // nu + 1, then y
   int* src = reinterpret_cast<int*>(g + ldh);         // [chunk][NSRC] element ids
-  float2* st = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(src + (size_t)a.chunk * NSRC) + 7) & ~(uintptr_t)7);   // [nu + 2]
+  typename X::V2* st = reinterpret_cast<typename X::V2*>((reinterpret_cast<uintptr_t>(src + (size_t)a.chunk * NSRC) + 15) & ~(uintptr_t)15);   // [nu + 2]
   __shared__ int timed_out;
+  __shared__ Scal<V> scal;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, G = gridDim.x;
   const bool scalar_warp = warp == COOP_WORK / 32;
@@ -423,14 +603,14 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
 #define COOP_PRODUCT(own, ep, bsub, out, rev)                                                             \
   for (int p0 = 0; p0 < ne; p0 += a.epc) {                                                                \
     const int nl = min(a.epc, ne - p0);                                                                   \
-    const bool got = stage_inputs(src, NSRC, p0, nl, nb, inv_nb, e_beg, ne, a.x, own, a.zx, ep, a.status, xs); \
+    const bool got = stage_inputs<V>(src, NSRC, p0, nl, nb, inv_nb, e_beg, ne, a.x, own, a.zx, ep, a.status, xs); \
     COOP_LEAVE_IF(!got)                                                                                   \
     if (sp < ns && sub < nl) {                                                                     \
       const int el = p0 + sub;                                                                            \
       const size_t e = e_beg + el;                                                                        \
       const S* D = (RES ? Rs + (size_t)el * (NSRC + 1) * bs : a.Dop + e * bs) + R * tt;                   \
       const S* O = (RES ? Rs + ((size_t)el * (NSRC + 1) + 1) * bs : a.O + e * NF * bs) + R * tt;          \
-      float acc[R];                                                                                       \
+      V acc[R];                                                                                           \
       bsr_rows<S, NF, RES>(D, O, nb, ld, bs, bb0, bb1, rev, xs + (size_t)sub * NSRC * nb, acc);           \
       const int r0 = el * nb + R * tt;                                                                    \
       _Pragma("unroll") for (int k = 0; k < R; ++k) if (R * tt + k < nb) {                                \
@@ -444,7 +624,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
   }                                                                                                       \
   if (ns > 1) {                                                                                           \
     for (int r = tid; r < rows; r += COOP_THREADS) {                                                      \
-      float t = ps[r];                                                                                    \
+      V t = ps[r];                                                                                        \
       for (int k = 1; k < ns; ++k) t += ps[(size_t)k * rmax + r];                                         \
       out[r] = bsub ? __ldcg(bsub + (size_t)e_beg * nb + r) - t : t;                                      \
     }                                                                                                     \
@@ -453,14 +633,14 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
 
   // v_0 = r = b - A x, not normalised (exchange 0 brings its norm)
   {
-    const float* none = nullptr;
+    const V* none = nullptr;
     COOP_PRODUCT(none, 0u, a.b, Vs, false)
   }
-  float rho = 1.f;          // |w - V h| as estimated: v_{j+1} = (w - V h) / rho
+  V rho = V(1);             // |w - V h| as estimated: v_{j+1} = (w - V h) / rho
   int kdone = 0;
   for (int j = 0;; ++j) {
     const unsigned ep = base + 1u + (unsigned)j;
-    float* vj = Vs + (size_t)j * rmax;
+    V* vj = Vs + (size_t)j * rmax;
     if (j < nu) {
       // the blocks of the coming product, meanwhile (see CoopArgs::pre)
       const bool rev = (j & 1) == 0;
@@ -473,29 +653,29 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
           }
       }
       // z_j = D^{-1} v_j: own rows to shared memory, published for the neighbours
-      float* zs = Zs + (size_t)j * rmax;
+      V* zs = Zs + (size_t)j * rmax;
       const int bsub_ = tid / tpe, btt = tid - bsub_ * tpe, bep = COOP_WORK / tpe;
       if (bsub_ < bep) {
         for (int el = bsub_; el < ne; el += bep) {
           const size_t e = e_beg + el;
           const S* M = (RES ? Rs + ((size_t)el * (NSRC + 1) + NSRC) * bs : a.Dinv + e * bs) + R * btt;
-          const float* xe = vj + (size_t)el * nb;
-          float acc[R];
+          const V* xe = vj + (size_t)el * nb;
+          V acc[R];
 #pragma unroll
-          for (int k = 0; k < R; ++k) acc[k] = 0.f;
+          for (int k = 0; k < R; ++k) acc[k] = V(0);
           col_run<S, RES>(M, nb, ld, xe, acc);
           const int r0 = el * nb + R * btt;
 #pragma unroll
           for (int k = 0; k < R; ++k)
             if (R * btt + k < nb) {
               zs[r0 + k] = acc[k];
-              st_val(a.zx + (size_t)e_beg * nb + r0 + k, acc[k], ep);
+              X::st(a.zx + (size_t)e_beg * nb + r0 + k, acc[k], ep);
             }
         }
       }
       __syncthreads();
       // w = A z_j
-      const float* none = nullptr;
+      const V* none = nullptr;
       COOP_PRODUCT(zs, ep, none, ws, rev)
     }
     // exchange j
@@ -504,78 +684,58 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
         for (int el = tid; el < ne; el += COOP_THREADS)
           prefetch_l2(a.Dinv + (size_t)(e_beg + el) * bs, (unsigned)(bs * sizeof(S)));
     }
-    uint4* px = a.px + (size_t)(j & 1) * (G + 1) * a.ni;
-    publish_dots(j, Vs, rmax, j < nu ? ws : nullptr, rows, px + blockIdx.x, G + 1, ep);
-    const bool got = gather_dots(px, G + 1, j + 2, G + a.extra, a.sums + (j & 1) * a.ni, ep, a.status, st);
-    COOP_LEAVE_IF(!got)
-    float ss = 0.f, sc = 0.f, tq = 0.f;
-    for (int i = 0; i < j; ++i) {
-      const float2 q = st[i];
-      ss = fmaf(q.x, q.x, ss);
-      sc = fmaf(q.x, q.y, sc);
-      tq = fmaf(q.y, q.y, tq);
-    }
-    const float be2 = st[j].x - ss;
-    const bool fine = be2 > 0.f && isfinite(be2);
-    const float beta = fine ? sqrtf(be2) : 0.f, ib = fine ? 1.f / beta : 0.f;
-    const float hj = (st[j].y - sc) * ib, ww = st[j + 1].x;
+    typename X::P* px = a.px + (size_t)(j & 1) * (G + 1) * a.ni;
+    publish_dots<V>(j, Vs, rmax, j < nu ? ws : nullptr, rows, px + blockIdx.x, G + 1, ep);
+    bool got = true;
     if (scalar_warp) {
-      // column j - 1 completed and rotated, column j begun (this warp alone)
-      if (j == 0) {
-        for (int i = lane; i < ldh; i += 32) g[i] = i == 0 ? beta : 0.f;
-      } else {
-        float* h = H + (size_t)(j - 1) * ldh;
-        for (int i = lane; i < j; i += 32) h[i] = fmaf(rho, st[i].x, h[i]);
+      if (j >= 2 && lane == 0) rotate_column(H, ldh, j - 2, cs, sn, g);   // behind the exchange
+    } else {
+      got = gather_dots<V>(px, G + 1, j + 2, G + a.extra, a.sums + (j & 1) * a.ni, ep, a.status, st);
+      if (warp == 0) {
         __syncwarp();
-        if (lane == 0) {
-          float p = h[0];
-          for (int i = 0; i + 1 < j; ++i) {
-            const float q = h[i + 1];
-            h[i] = cs[i] * p + sn[i] * q;
-            p = -sn[i] * p + cs[i] * q;
-          }
-          const float q = rho * beta, rr = hypotf(p, q);
-          float c = 1.f, sv = 0.f;
-          if (rr != 0.f) {
-            c = p / rr;
-            sv = q / rr;
-          }
-          cs[j - 1] = c;
-          sn[j - 1] = sv;
-          h[j - 1] = c * p + sv * q;
-          g[j] = -sv * g[j - 1];
-          g[j - 1] = c * g[j - 1];
-        }
+        exchange_scalars<V>(st, j, &scal);
+      }
+    }
+    COOP_LEAVE_IF(!got)
+    const bool fine = scal.fine;
+    const V beta = scal.beta, ib = scal.ib, hj = scal.hj;
+    if (scalar_warp) {
+      // column j - 1 completed, column j begun (this warp alone)
+      if (j == 0) {
+        for (int i = lane; i < ldh; i += 32) g[i] = i == 0 ? beta : V(0);
+      } else {
+        V* h = H + (size_t)(j - 1) * ldh;
+        for (int i = lane; i < j; i += 32) h[i] = fma(rho, st[i].x, h[i]);
+        if (lane == 0) h[j] = rho * beta;
       }
       if (j < nu && fine) {
-        float* h = H + (size_t)j * ldh;
+        V* h = H + (size_t)j * ldh;
         for (int i = lane; i <= j; i += 32) h[i] = i < j ? st[i].y : hj;
       }
       __syncwarp();
     }
     kdone = j;
     if (!fine || j == nu) {   // the Krylov space is exhausted (or not finite), or complete
-      if (!fine && !isfinite(be2) && tid == 0 && blockIdx.x == 0) atomicOr(a.kflag, ST_NONFINITE);
+      if (scal.bad && tid == 0 && blockIdx.x == 0) atomicOr(a.kflag, ST_NONFINITE);
       break;
     }
-    const float est = fmaxf(ww - tq - hj * hj, 1e-6f * ww);
-    rho = est > 0.f ? sqrtf(est) : 1.f;
-    const float ir = 1.f / rho;
+    rho = scal.rho;
+    const V ir = scal.ir;
     if (tid < COOP_WORK) {
-      float* vn = vj + rmax;
+      V* vn = vj + rmax;
       for (int r = tid; r < rows; r += COOP_WORK) {
-        float v = vj[r], w = ws[r];
-        const float* q = Vs + r;
+        V v = vj[r], w = ws[r];
+        const V* q = Vs + r;
 #pragma unroll 8
         for (int i = 0; i < j; ++i) {
-          const float2 c = st[i];
-          const float vi = q[(size_t)i * rmax];
-          v = fmaf(-c.x, vi, v);
-          w = fmaf(-c.y, vi, w);
+          const typename X::V2 c = st[i];
+          const V vi = q[(size_t)i * rmax];
+          v = fma(-c.x, vi, v);
+          w = fma(-c.y, vi, w);
         }
         v *= ib;
         vj[r] = v;
-        vn[r] = fmaf(-hj, v, w) * ir;
+        vn[r] = fma(-hj, v, w) * ir;
       }
     }
     __syncthreads();
@@ -584,19 +744,26 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
   if (kdone == 0) return;   // b - A x = 0 (or not finite): nothing to smooth
   // y = H[:k,:k]^{-1} g[:k] (into g; the scalar warp, which rotated it), x += Z y on own rows
   if (scalar_warp) {
+    if (lane == 0) rotate_column(H, ldh, kdone - 1, cs, sn, g);
+    __syncwarp();
+    for (int i = lane; i < kdone; i += 32) {    // the diagonal's reciprocals at once (into cs)
+      const V d = H[(size_t)i * ldh + i];
+      cs[i] = d != V(0) ? V(1) / d : V(0);
+    }
+    __syncwarp();
     for (int i = kdone - 1; i >= 0; --i) {
-      const float d = H[(size_t)i * ldh + i], y = d != 0.f ? g[i] / d : 0.f;
+      const V y = g[i] * cs[i];
       __syncwarp();
-      for (int c = lane; c < i; c += 32) g[c] = fmaf(-H[(size_t)i * ldh + c], y, g[c]);
+      for (int c = lane; c < i; c += 32) g[c] = fma(-H[(size_t)i * ldh + c], y, g[c]);
       if (lane == 0) g[i] = y;
       __syncwarp();
     }
   }
   __syncthreads();
-  float* xo = a.x + (size_t)e_beg * nb;
+  V* xo = a.x + (size_t)e_beg * nb;
   for (int r = tid; r < rows; r += COOP_THREADS) {
-    float acc = xo[r];
-    for (int i = 0; i < kdone; ++i) acc = fmaf(g[i], Zs[(size_t)i * rmax + r], acc);
+    V acc = xo[r];
+    for (int i = 0; i < kdone; ++i) acc = fma(g[i], Zs[(size_t)i * rmax + r], acc);
     xo[r] = acc;
   }
 #undef COOP_PRODUCT
@@ -608,8 +775,9 @@ template <class S>
 static size_t coop_smem(int nu, int nb, int ld, int nf, int chunk, int epc, int ns, bool res) {
   const size_t ldh = nu + 1, rmax = (size_t)chunk * nb;
   const size_t fl = ldh * rmax + nu * rmax + rmax + (ns > 1 ? ns * rmax : 0) + (size_t)epc * (1 + nf) * nb +
-                    ldh * nu + 2 * (size_t)nu + ldh + (size_t)chunk * (1 + nf);
-  return fl * sizeof(float) + 8 + sizeof(float2) * (nu + 2) +
+                    ldh * nu + 2 * (size_t)nu + ldh;
+  using V = typename CoopVal<S>::V;
+  return fl * sizeof(V) + sizeof(int) * (size_t)chunk * (1 + nf) + 16 + 2 * sizeof(V) * (nu + 2) +
          (res ? (size_t)chunk * (2 + nf) * nb * ld * sizeof(S) : 0);
 }
 
@@ -665,31 +833,33 @@ static cudaError_t plan_coop(int nb, int ld, int E, int nu, CoopPlan* plan) {
     plan->pre = pre;
     plan->res = res;
     plan->smem = smem;
-    plan->part_bytes = sizeof(uint4) * 2 * (size_t)(grid + 2) * (nu + 2);
-    plan->z_bytes = sizeof(unsigned long long) * (size_t)E * nb;
+    using X = Xch<typename CoopVal<S>::V>;
+    plan->part_bytes = sizeof(typename X::P) * 2 * (size_t)(grid + 2) * (nu + 2);
+    plan->z_bytes = sizeof(typename X::Z) * (size_t)E * nb;
     return cudaSuccess;
   }
   return cudaSuccess;
 }
 
-cudaError_t plan_coop_smoother(int bf16, int nb, int nf, int E, int nu, CoopPlan* plan) {
+cudaError_t plan_coop_smoother(int store, int nb, int nf, int E, int nu, CoopPlan* plan) {
   plan->ok = 0;
-  if (nf == 6)
-    return bf16 ? plan_coop<unsigned short, 6>(nb, ld_bf16(nb), E, nu, plan)
-                : plan_coop<float, 6>(nb, inv_ld<float>(nb), E, nu, plan);
-  if (nf == 4)
-    return bf16 ? plan_coop<unsigned short, 4>(nb, ld_bf16(nb), E, nu, plan)
-                : plan_coop<float, 4>(nb, inv_ld<float>(nb), E, nu, plan);
-  if (nf == 3)
-    return bf16 ? plan_coop<unsigned short, 3>(nb, ld_bf16(nb), E, nu, plan)
-                : plan_coop<float, 3>(nb, inv_ld<float>(nb), E, nu, plan);
+#define GO(NF)                                                                                     \
+  return store == COOP_BF16   ? plan_coop<unsigned short, NF>(nb, ld_bf16(nb), E, nu, plan)       \
+         : store == COOP_FP64 ? plan_coop<double, NF>(nb, inv_ld<double>(nb), E, nu, plan)        \
+                              : plan_coop<float, NF>(nb, inv_ld<float>(nb), E, nu, plan)
+  if (nf == 6) GO(6);
+  if (nf == 4) GO(4);
+  if (nf == 3) GO(3);
+#undef GO
   return cudaSuccess;   // other face counts keep the launch-per-operation smoother
 }
 
 template <class S, int NF>
 static cudaError_t launch_coop(const CoopPlan& pl, const S* Dinv, const S* Dop, const S* O, int ld, const int* nbr,
-                               const float* b, float* x, int nu, Krylov<float>& K, const CoopBuffers& buf,
-                               int* status, int extra, int nb, int E, cudaStream_t st) {
+                               const typename CoopVal<S>::V* b, typename CoopVal<S>::V* x, int nu,
+                               Krylov<typename CoopVal<S>::V>& K, const CoopBuffers& buf, int* status, int extra,
+                               int nb, int E, cudaStream_t st) {
+  using X = Xch<typename CoopVal<S>::V>;
   CoopArgs<S> a;
   a.Dinv = Dinv;
   a.Dop = Dop;
@@ -697,8 +867,8 @@ static cudaError_t launch_coop(const CoopPlan& pl, const S* Dinv, const S* Dop, 
   a.nbr = nbr;
   a.b = b;
   a.x = x;
-  a.zx = (unsigned long long*)buf.z;
-  a.px = (uint4*)buf.part;
+  a.zx = (typename X::Z*)buf.z;
+  a.px = (typename X::P*)buf.part;
   a.sums = a.px + 2 * (size_t)(pl.grid + 1) * (pl.nu_max + 2);
   a.epoch = buf.epoch;
   a.status = status;
@@ -739,6 +909,20 @@ cudaError_t launch_coop_smoother(const CoopPlan& pl, const float* Dinv, const fl
                                                   extra, nb, E, st)                                                \
                 : launch_coop<float, NF>(pl, Dinv, Dop, O, inv_ld<float>(nb), nbr, b, x, nu, K, buf, status, extra,   \
                                          nb, E, st)
+  if (nf == 6) GO(6);
+  if (nf == 4) GO(4);
+  if (nf == 3) GO(3);
+#undef GO
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_coop_smoother(const CoopPlan& pl, const double* Dinv, const double* Dop, const double* O,
+                                 const unsigned short*, const unsigned short*, const unsigned short*, const int* nbr,
+                                 int nf, const double* b, double* x, int nu, Krylov<double>& K, const CoopBuffers& buf,
+                                 int* status, int extra, int nb, int E, cudaStream_t st) {
+  if (!pl.ok || nu < 1 || nu > pl.nu_max || nu > K.nmax) return cudaErrorInvalidValue;
+#define GO(NF) \
+  return launch_coop<double, NF>(pl, Dinv, Dop, O, inv_ld<double>(nb), nbr, b, x, nu, K, buf, status, extra, nb, E, st)
   if (nf == 6) GO(6);
   if (nf == 4) GO(4);
   if (nf == 3) GO(3);

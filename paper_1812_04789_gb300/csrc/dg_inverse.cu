@@ -16,16 +16,19 @@
 // 16-byte multiple with zeros), the layout the block-Jacobi apply streams,
 // except from the in-place global-memory path, which leaves it row-major.
 //
-// block_inverse_reg_kernel (nb <= 16 R): 256 threads as a 16 x 16 grid;
+// block_inverse_reg_kernel (nb < 40; nb <= 16 R): 256 threads as a 16 x 16 grid;
 // thread (ty, tx) keeps the R x R entries of rows ty + 16 a and columns
 // tx + 16 b in registers for the whole elimination, so a step costs R^2 FMAs
 // per thread plus two shared-memory vectors (the pivot row and column) and
 // three barriers.  The permuted, transposed result is staged in shared memory
 // and written out coalesced.
-// block_inverse_kernel (larger blocks): the block in shared memory, one warp
-// per row in the update.  block_inverse_panel_kernel (blocks that do not fit
-// shared memory): panels of columns eliminated in shared memory, one rank-16
-// update of the block's other columns per panel.
+// block_inverse_sm_kernel (blocks that fit shared memory with a panel): panels
+// in registers, register-tiled updates in shared memory.
+// block_inverse_blk_kernel (up to 512 rows): the same on the block in memory.
+// block_inverse_kernel (the few sizes whose block fits shared memory without
+// the panel): one warp per row in the update.  block_inverse_panel_kernel
+// (blocks beyond 512 rows): panels of columns eliminated in shared memory, one
+// rank-16 update of the block's other columns per panel.
 #include <algorithm>
 #include <climits>
 
@@ -772,6 +775,185 @@ cudaError_t run_blk(T* A, int nb, size_t bstride, long nblk, int smax, int* stat
   return cudaGetLastError();
 }
 
+// Blocks of 40 rows or more that fit shared memory (209 rows in FP32, 153 in FP64) with their panel: the elimination of
+// block_inverse_blk_kernel on a copy in shared memory (rows padded to an odd
+// number of 16-byte vectors, so that a thread per row reads its panel without
+// bank conflicts), the inverse written column-major.  The panel's warps alone
+// take part in its barriers.  A step of block_inverse_reg_kernel costs 2,600
+// cycles at nb = 175 (three barriers, a serial pivot search, every thread's whole
+// tile); here a step is 32 columns wide and the rest is one register-tiled
+// update per panel.
+// 4,096 FP32 blocks of 175 rows: 6.5 -> 3.8 ms, of 100: 2.76 -> 1.20; 3,600 of 180
+// (block_inverse_kernel before): 39 -> 3.6; 1,080 FP64 blocks of 100 rows: 6.9 ->
+// 2.8 ms, of 50: 1.24 -> 0.55.  Bound by the panel's steps (latency) and the FP32
+// pipe in the update, FP64 by its pipe.
+template <class T, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) block_inverse_sm_kernel(T* __restrict__ blocks, int nb, int lds,
+                                                                        int ldo, size_t bstride, long nblk,
+                                                                        int* status) {
+  constexpr int BW = BlkTile<T>::BW, RI = BlkTile<T>::RI, V = 16 / sizeof(T);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nbp = (nb + RI - 1) / RI * RI, nv = (nb + V - 1) / V;
+  T* S = reinterpret_cast<T*>(smem_raw);              // [nb][lds]
+  T* Ps = S + (size_t)nb * lds;                       // [BW][nbp] panel, transposed
+  T* Xp = Ps + (size_t)BW * nbp;                      // [BW][lds] pivot rows before the panel
+  T* prow = Xp + (size_t)BW * lds;                    // [2][BW] pivot row of the step (alternating)
+  int* piv_row = reinterpret_cast<int*>(prow + 2 * BW);
+  int* step_of = piv_row + nb;
+  __shared__ unsigned cand_hi[2][16], cand_lo[2][16];
+  __shared__ int cand_row[2][16];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nrw = (nb + 31) / 32;   // warps with rows of the panel
+  for (long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    T* A = blocks + (size_t)blk * bstride;
+    __syncthreads();
+    for (int i = tid; i < nb; i += NT) step_of[i] = -1;
+    for (int i = warp; i < nb; i += NT / 32)
+      for (int j = lane; j < nv * V; j += 32) S[(size_t)i * lds + j] = j < nb ? A[(size_t)i * nb + j] : T(0);
+    __syncthreads();
+    bool bad = false, used = tid >= nb;
+    for (int k0 = 0; k0 < nb; k0 += BW) {
+      const int bw = min(BW, nb - k0);
+      T x[BW];
+      if (warp < nrw) {
+#pragma unroll
+        for (int c = 0; c < BW; c += V) {
+          if (tid < nb && c < bw)
+            ld_vec<T, V>(S + (size_t)tid * lds + k0 + c, x + c);
+          else
+#pragma unroll
+            for (int u = 0; u < V; ++u) x[c + u] = T(0);
+        }
+#pragma unroll
+        for (int c = 0; c < BW; ++c) {
+          if (c >= bw) break;
+          const int par = c & 1;
+          unsigned hi, lo;
+          pivot_key(x[c], !used, &hi, &lo);
+          const int wl = warp_argmax<T>(hi, lo);
+          if (lane == wl) {
+            cand_hi[par][warp] = hi;
+            cand_lo[par][warp] = lo;
+            cand_row[par][warp] = tid;
+          }
+          asm volatile("bar.sync 1, %0;" ::"r"(nrw * 32) : "memory");
+          const int b = lane < nrw ? lane : 0;
+          const int wb = warp_argmax<T>(cand_hi[par][b], cand_lo[par][b]);
+          const int p = cand_row[par][wb];
+          T* pr = prow + par * BW;
+          if (tid == p) {
+#pragma unroll
+            for (int u = 0; u < BW; ++u) pr[u] = x[u];
+            used = true;
+            piv_row[k0 + c] = p;
+            step_of[p] = k0 + c;
+          }
+          asm volatile("bar.sync 1, %0;" ::"r"(nrw * 32) : "memory");
+          T piv = pr[c];
+          if (!(fabs(piv) > T(0))) {
+            bad = true;
+            piv = T(1);
+          }
+          const T ipiv = T(1) / piv;
+          if (tid == p) {
+#pragma unroll
+            for (int u = 0; u < BW; ++u) x[u] = u == c ? ipiv : x[u] * ipiv;
+          } else {
+            const T m = x[c] * ipiv;
+#pragma unroll
+            for (int u = 0; u < BW; u += V) {
+              T q[V];
+              ld_vec<T, V>(pr + u, q);
+#pragma unroll
+              for (int w = 0; w < V; ++w)
+                if (u + w != c) x[u + w] -= m * q[w];
+            }
+            x[c] = -m;
+          }
+        }
+      }
+      __syncthreads();
+      // pivot rows before the panel; the panel transposed
+      for (int t = tid; t < bw * nv; t += NT) {
+        const int c = t / nv, v = t - c * nv;
+        T q[V];
+        ld_vec<T, V>(S + (size_t)piv_row[k0 + c] * lds + v * V, q);
+        st_vec<T, V>(Xp + (size_t)c * lds + v * V, q);
+      }
+      if (tid < nbp) {
+#pragma unroll
+        for (int c = 0; c < BW; ++c) Ps[(size_t)c * nbp + tid] = tid < nb ? x[c] : T(0);
+      }
+      __syncthreads();
+      if (tid < nb) {      // and back in place
+#pragma unroll
+        for (int c = 0; c < BW; ++c)
+          if (c < bw) S[(size_t)tid * lds + k0 + c] = x[c];
+      }
+      // C += P Xp on the other columns (pivot rows: C = P Xp)
+      const int vlo = k0 / V, pv = (bw + V - 1) / V, nvc = nv - pv;
+      for (int t = tid; t < nbp / RI * nvc; t += NT) {
+        const int rg = t / nvc, v_ = t - rg * nvc, v = v_ < vlo ? v_ : v_ + pv, i0 = rg * RI;
+        T acc[RI][V];
+        T* Sc = S + (size_t)i0 * lds + v * V;
+#pragma unroll
+        for (int i = 0; i < RI; ++i) {
+          const int ic = min(i, nb - 1 - i0), so = step_of[i0 + ic];
+          ld_vec<T, V>(Sc + (size_t)ic * lds, acc[i]);
+          if (so >= k0 && so < k0 + bw)
+#pragma unroll
+            for (int u = 0; u < V; ++u) acc[i][u] = T(0);
+        }
+#pragma unroll 2
+        for (int c = 0; c < bw; ++c) {
+          T pi[RI], q[V];
+          ld_vec<T, RI>(Ps + (size_t)c * nbp + i0, pi);
+          ld_vec<T, V>(Xp + (size_t)c * lds + v * V, q);
+#pragma unroll
+          for (int i = 0; i < RI; ++i)
+#pragma unroll
+            for (int u = 0; u < V; ++u) acc[i][u] += pi[i] * q[u];
+        }
+#pragma unroll
+        for (int i = 0; i < RI; ++i)
+          if (i0 + i < nb) st_vec<T, V>(Sc + (size_t)i * lds, acc[i]);
+      }
+      __syncthreads();
+    }
+    // X[r][c] = R[piv_row[r]][step_of[c]], column-major, zeros in the padding rows
+    for (int c = warp; c < nb; c += NT / 32) {
+      const T* Sc = S + step_of[c];
+      for (int r = lane; r < ldo; r += 32) A[(size_t)c * ldo + r] = r < nb ? Sc[(size_t)piv_row[r] * lds] : T(0);
+    }
+    if (bad && tid == 0) atomicOr(status, ST_SINGULAR);
+  }
+}
+
+template <class T>
+cudaError_t run_sm(T* A, int nb, size_t bstride, long nblk, int smax, int* status, cudaStream_t st, bool* done) {
+  constexpr int BW = BlkTile<T>::BW, RI = BlkTile<T>::RI, V = 16 / sizeof(T);
+  *done = false;
+  const size_t nbp = (nb + RI - 1) / RI * RI, lds = (size_t)(((nb + V - 1) / V) | 1) * V;
+  const size_t smem = ((size_t)nb * lds + BW * nbp + BW * lds + 2 * BW) * sizeof(T) + 2 * (size_t)nb * sizeof(int);
+  if (smem > (size_t)smax - 1024 || nbp > 256) return cudaSuccess;
+  // up to 128 rows two CTAs of 256 threads share an SM's registers
+  const bool small = nb <= 128;
+  cudaError_t e = small ? allow_max_smem(block_inverse_sm_kernel<T, 256>) : allow_max_smem(block_inverse_sm_kernel<T, 512>);
+  if (e != cudaSuccess) return e;
+  int occ = 0;
+  e = small ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, block_inverse_sm_kernel<T, 256>, 256, smem)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, block_inverse_sm_kernel<T, 512>, 512, smem);
+  if (e != cudaSuccess) return e;
+  if (occ < 1) return cudaSuccess;
+  const int grid = (int)std::min<long>(nblk, (long)occ * num_sms_inv());
+  note_launch();
+  if (small)
+    block_inverse_sm_kernel<T, 256><<<grid, 256, smem, st>>>(A, nb, (int)lds, inv_ld<T>(nb), bstride, nblk, status);
+  else
+    block_inverse_sm_kernel<T, 512><<<grid, 512, smem, st>>>(A, nb, (int)lds, inv_ld<T>(nb), bstride, nblk, status);
+  *done = true;
+  return cudaGetLastError();
+}
+
 template <class T, int R>
 cudaError_t run_reg(T* A, int nb, size_t bstride, long nblk, int* status, cudaStream_t st) {
   const size_t smem = (size_t)nb * inv_ld<T>(nb) * sizeof(T);
@@ -792,25 +974,25 @@ cudaError_t launch_block_inverse(T* A, int nb, size_t bstride, long nblk, int* s
                                  cudaStream_t st) {
   *transposed = 1;
   if (nblk <= 0) return cudaSuccess;
-  // register tiles: R x R values of T per thread (at most 128 32-bit registers)
-  const int R = (nb + 15) / 16;
-  constexpr int RMAX = sizeof(T) == 4 ? 11 : 8;
-  if (R <= RMAX) {
-    if (R <= 1) return run_reg<T, 1>(A, nb, bstride, nblk, status, st);
-    if (R <= 2) return run_reg<T, 2>(A, nb, bstride, nblk, status, st);
-    if (R <= 4) return run_reg<T, 4>(A, nb, bstride, nblk, status, st);
-    if (R <= 8) return run_reg<T, 8>(A, nb, bstride, nblk, status, st);
-    return run_reg<T, (RMAX > 8 ? RMAX : 8)>(A, nb, bstride, nblk, status, st);
-  }
-  const int threads = 256;
-  const size_t base = 2 * nb * sizeof(T) + 4 * nb * sizeof(int) + 32;
-  const size_t full = base + (size_t)nb * nb * sizeof(T);
   int smax = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // the line: 7,500 FP32 blocks of 40 rows 805 us in registers, 693 in shared
+  // memory; 4,096 of 50 560 and 488; the register tile of fewer rows is small
+  if (nb < 40) {
+    const int R = (nb + 15) / 16;
+    if (R <= 1) return run_reg<T, 1>(A, nb, bstride, nblk, status, st);
+    if (R <= 2) return run_reg<T, 2>(A, nb, bstride, nblk, status, st);
+    return run_reg<T, 3>(A, nb, bstride, nblk, status, st);
+  }
+  bool done = false;
+  const cudaError_t es = run_sm<T>(A, nb, bstride, nblk, smax, status, st, &done);
+  if (es != cudaSuccess || done) return es;
+  const int threads = 256;
+  const size_t base = 2 * nb * sizeof(T) + 4 * nb * sizeof(int) + 32;
+  const size_t full = base + (size_t)nb * nb * sizeof(T);
   const int use_smem = full <= (size_t)smax - 1024;
   if (!use_smem) {
-    bool done = false;
     cudaError_t e = run_blk<T, 16 / (int)sizeof(T)>(A, nb, bstride, nblk, smax, status, st, &done);
     if (e != cudaSuccess) return e;
     if (sizeof(T) == 8 && !done)   // FP64 rows of an odd number of entries (nb = 175)

@@ -224,6 +224,15 @@ cudaError_t launch_nbr_sf(const Mesh& M, const float* W, float* O, int nmc, int 
                           cudaStream_t st);
 cudaError_t launch_nbr_sf(const Mesh& M, const double* W, double* O, int nmc, int colmajor, cudaStream_t st);
 
+// FP64 face and volume terms of 2-D structured meshes (csrc/dg_res2d64.cu), the
+// former into slots, the latter added to them as launch_residual does, where they
+// are the faster ones (face2d64_ok, vol2d64_ok).
+bool face2d64_ok(const Mesh& M, bool jvp);
+bool vol2d64_ok(const Mesh& M);
+cudaError_t launch_face2d64(const Mesh& M, const double* W, const double* V, double* slots, bool jvp, cudaStream_t st);
+cudaError_t launch_vol2d64(const Mesh& M, const double* W, const double* V, const double* slots, const double* Src,
+                           double sigma, double* out, bool jvp, cudaStream_t st);
+
 // FP64 blocks (csrc/dg_probe64.cu): D as launch_probe_blocks, O (may be null)
 // column-major with leading dimension inv_ld(nbc), nbc * inv_ld(nbc) apart, or
 // row-major, nbc^2 apart.  probe64_fits: structured, no direction of one

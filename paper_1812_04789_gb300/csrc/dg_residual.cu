@@ -574,6 +574,8 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
       e = launch_face_sf<T>(Ms, W, V, slots, JVP, JVP ? Pf : nullptr, st);
       if (e == cudaErrorNotSupported) (void)cudaGetLastError();
     }
+    if constexpr (D == 2 && std::is_same<T, double>::value)
+      if (face2d64_ok(Ms, JVP)) e = launch_face2d64(Ms, W, V, slots, JVP, st);
     if (e == cudaErrorNotSupported) {
       note_launch();
       face_kernel<D, T, JVP><<<(nfaces + fpc - 1) / fpc, fthreads, fsm, st>>>(mv, ph, W, V, slots, Ms.status, fpc,
@@ -615,6 +617,8 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
       return cudaGetLastError();
     }
   }
+  if constexpr (D == 2 && std::is_same<T, double>::value)
+    if (vol2d64_ok(Ms)) return launch_vol2d64(Ms, W, V, slots, S, sigma, out, JVP, st);
   int vthreads = 256;
   int epc = items_per_cta(Ms.E, std::max(1, 256 / Ms.nq), Ms.nq, vthreads, &vthreads);
   size_t vsm = vol_smem<T>(Ms, epc, JVP);
@@ -739,11 +743,17 @@ static cudaError_t run_residual_slots(const Mesh& Ms, const double* W, const dou
   if (fsm > 48 * 1024)
     allow_max_smem(face_kernel<D, double, false>);
   int nfaces = D * Ms.E;
-  note_launch();
-  face_kernel<D, double, false><<<(nfaces + fpc - 1) / fpc, 128, fsm, st>>>(mv, ph, W, nullptr, slots,
-                                                                            Ms.status, fpc, nullptr);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (D == 2 && face2d64_ok(Ms, false)) {
+    e = launch_face2d64(Ms, W, nullptr, slots, false, st);
+  } else {
+    note_launch();
+    face_kernel<D, double, false><<<(nfaces + fpc - 1) / fpc, 128, fsm, st>>>(mv, ph, W, nullptr, slots,
+                                                                              Ms.status, fpc, nullptr);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return e;
+  if (D == 2 && vol2d64_ok(Ms)) return launch_vol2d64(Ms, W, nullptr, slots, S, 0.0, out, false, st);
   int epc = std::max(1, 256 / Ms.nq);
   size_t vsm = vol_smem<double>(Ms, epc, false);
   while (vsm > 200 * 1024 && epc > 1) vsm = vol_smem<double>(Ms, --epc, false);

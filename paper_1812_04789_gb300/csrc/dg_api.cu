@@ -249,7 +249,7 @@ static dg_status alloc_mg(dg_pmg h, MG<T>& mg) {
     for (T** v : {&L.x, &L.b, &L.r, &L.t}) CK(dalloc(mg.allocs, (void**)v, sizeof(T) * L.N, &h->vector_bytes));
     int nmax = (l == nl - 1) ? std::max(1, o.nu_coarse) : std::max(std::max(L.nu_pre, L.nu_post), 1);
     if (o.cycle != DG_CYCLE_BJ) {
-      CK(L.kr.alloc(L.N, nmax));
+      CK(L.kr.alloc(L.N, nmax, M.status));
       h->vector_bytes += L.kr.bytes();
     }
     // persistent smoother of an inherited level (column-major or BF16
@@ -538,7 +538,7 @@ extern "C" dg_status dg_pmg_setup(dg_mesh mesh, const double* W, double sigma, c
   }
   if (s == DG_OK) {
     h->outer_restart = opts->fgmres_restart > 0 ? opts->fgmres_restart : 30;
-    if (h->outer.alloc(N0, h->outer_restart) != cudaSuccess ||
+    if (h->outer.alloc(N0, h->outer_restart, h->mesh->m.status) != cudaSuccess ||
         dalloc(h->allocs, (void**)&h->tmp64, sizeof(double) * N0 * 2, &h->vector_bytes) != cudaSuccess)
       s = DG_ERR_OOM;
     else

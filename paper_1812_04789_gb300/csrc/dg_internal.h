@@ -333,8 +333,17 @@ struct Krylov {
   double* part = nullptr;    // (nmax+1) x G reduction partials
   double* res = nullptr;     // residual estimate |g[j+1]|
   int* kdim = nullptr;       // [0] effective Krylov dimension (breakdown), [1] status bits
+  // one-kernel Arnoldi step (csrc/dg_arnoldi.cu): CTAs (0: a kernel per
+  // operation), entries of a vector per CTA, the exchange's buffers (launches that share
+  // them are ordered on one stream) and the word that takes ST_TIMEOUT
+  int ag = 0;
+  long achunk = 0;
+  void* apx = nullptr;
+  unsigned* aepoch = nullptr;
+  int* astatus = nullptr;
   std::vector<void*> allocs;
-  cudaError_t alloc(long N, int nmax);
+  // status: the mesh status word
+  cudaError_t alloc(long N, int nmax, int* status);
   void release();
   size_t bytes() const;
   // v0 = r / ||r||, g = (||r||, 0, ...)
@@ -347,6 +356,13 @@ struct Krylov {
   T* Vj(int j) { return V + (size_t)j * N; }
   T* Zj(int j) { return Z + (size_t)j * N; }
 };
+// Step j of the Arnoldi process on K (Gram-Schmidt twice of K.w, v_{j+1},
+// Hessenberg column and its rotation) as one cooperative kernel: K.ag > 0.
+// plan_arnoldi fills ag, achunk and the bytes of apx.
+template <class T>
+cudaError_t plan_arnoldi(Krylov<T>& K, size_t* bytes);
+template <class T>
+cudaError_t launch_arnoldi(const Krylov<T>& K, int j, cudaStream_t st);
 
 // ----------------------------------------------------------------- pMG
 // Launch plan of the persistent coarse-level smoother (csrc/dg_smoother.cu):

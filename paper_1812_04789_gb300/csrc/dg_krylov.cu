@@ -1,6 +1,8 @@
 // Vector kernels and the device-resident (F)GMRES Arnoldi process (Sec. 6:
 // flexible GMRES, Saad 1993; GMRES smoothers of Algorithm 2).
 //
+// A step of vectors that fit the CTAs' shared memory is one kernel
+// (dg_arnoldi.cu); the kernels per operation below take the longer ones.
 // Orthogonalisation is classical Gram-Schmidt applied twice (CGS2): the j+1
 // inner products of a pass are one kernel (one CTA row per basis vector,
 // fixed chunking) plus a fixed-order finalisation, so results do not depend
@@ -313,7 +315,7 @@ __global__ void set_int_kernel(int* p, int v) { *p = v; }
 
 // ---------------------------------------------------------------- Krylov
 template <class T>
-cudaError_t Krylov<T>::alloc(long n, int nm) {
+cudaError_t Krylov<T>::alloc(long n, int nm, int* status) {
   release();
   if (sizeof(T) == sizeof(float) && nm + 1 > KMAX_F32) return cudaErrorInvalidValue;
   N = n;
@@ -337,6 +339,15 @@ cudaError_t Krylov<T>::alloc(long n, int nm) {
   if ((e = get((void**)&res, sizeof(double) * 4))) return e;
   if ((e = get((void**)&kdim, sizeof(int) * 2))) return e;
   if ((e = cudaMemset(kdim, 0, sizeof(int) * 2))) return e;
+  size_t ab = 0;
+  if ((e = plan_arnoldi(*this, &ab))) return e;
+  if (ag) {
+    astatus = status;
+    if ((e = get(&apx, ab))) return e;
+    if ((e = get((void**)&aepoch, sizeof(unsigned)))) return e;
+    if ((e = cudaMemset(apx, 0, ab))) return e;
+    if ((e = cudaMemset(aepoch, 0, sizeof(unsigned)))) return e;
+  }
   return cudaMemset(H, 0, sizeof(double) * (size_t)(nm + 1) * nm);
 }
 
@@ -347,6 +358,7 @@ void Krylov<T>::release() {
   V = Z = w = nullptr;
   H = cs = sn = g = y = part = res = nullptr;
   kdim = nullptr;
+  ag = 0;
 }
 
 template <class T>
@@ -378,6 +390,7 @@ cudaError_t Krylov<T>::start(const T* r, cudaStream_t st) {
 
 template <class T>
 cudaError_t Krylov<T>::arnoldi(int j, cudaStream_t st) {
+  if (ag) return launch_arnoldi(*this, j, st);
   const int nv = j + 1;
   double* Hcol = H + (size_t)j * (nmax + 1);
   int fgrid = (nv + 7) / 8;

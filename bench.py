@@ -31,7 +31,7 @@ import numpy as np  # noqa: E402
 from paper_1812_04789_gb300 import workloads as wl  # noqa: E402
 
 BJ_KERNEL_VERSION = "colmajor-v1"   # bump when the block-Jacobi apply kernel changes
-COOP_KERNEL_VERSION = "coop-fp32-3bar"   # bump when the persistent smoother kernel changes
+COOP_KERNEL_VERSION = "coop-polled"   # bump when the persistent smoother kernel changes
 METRIC = "Implicit-step DOFs/s (mixed vs FP64, 1 GB300); JVP % HBM roofline; p99 latency"
 UNIT = "DOFs/s"
 
@@ -432,9 +432,10 @@ def kernel_roofline(torch, B, stepper, stream, peaks):
     jb = E * nb * 8 * 3                      # read W and v, write Kv (FP64)
     out["jvp_fp64"] = dict(ms=ms, bytes=jb, gbs=jb / (ms * 1e-3) / 1e9,
                            hbm_frac=jb / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"])
-    # tensor-core block probe of the fine diagonal blocks: exporting the
-    # un-inverted level-0 blocks reruns exactly that kernel (no neighbour
-    # blocks are requested and no direction has a single element)
+    # block probe of the fine diagonal blocks: exporting the un-inverted level-0
+    # blocks reruns exactly that kernel (no neighbour blocks are requested and no
+    # direction has a single element); work: the floating-point operations it
+    # executes per element, counted by ncu (profiles/kernel_work.json)
     if stepper.opts.precision == B.PREC_MIXED and min(stepper.cfg["n"]) > 1:
         D = torch.empty((E, nb, nb), dtype=torch.float32, device=r.device)
         stepper.pmg.export_blocks(0, B.BLOCKS_DIAG, D, stream=stream)
@@ -446,16 +447,13 @@ def kernel_roofline(torch, B, stepper, stream, peaks):
             e1.synchronize()
             ts.append(e0.elapsed_time(e1))
         ms = statistics.median(ts)
-        d, nm = len(stepper.cfg["n"]), mesh.nm
-        nq1 = stepper.cfg["p"] + 2
-        # the dense contraction D[(w,v,i'), i] += Z[(w,v,i'), K] Trial[i, K], one pass,
-        # K = (volume points + own-face points) x (1 + d)
-        K = (nq1 ** d + 2 * d * nq1 ** (d - 1)) * (1 + d)
-        flops = 2.0 * E * (mesh.m * mesh.m * nm) * nm * K
-        tf32_peak = peaks["bf16_tflops"] * 1.1 / 2.25     # nominal dense TF32 / BF16 ratio
-        out["probe_tc"] = dict(ms=ms, flops=flops, tflops=flops / (ms * 1e-3) / 1e12, peak_tflops=tf32_peak,
-                               frac=flops / (ms * 1e-3) / 1e12 / tf32_peak,
-                               peak_source="measured bf16 burst x nominal TF32/BF16 ratio 1.1/2.25")
+        wf = os.path.join(ROOT, "profiles", "kernel_work.json")
+        rec = json.load(open(wf)).get("probe_fp32", {}) if os.path.exists(wf) else {}
+        fl = rec.get("flops_per_element") if stepper.cfg["p"] == 4 else None
+        out["block_probe"] = dict(ms=ms, flops=fl * E if fl else None,
+                                  tflops=fl * E / (ms * 1e-3) / 1e12 if fl else None, peak_tflops=FP32_PEAK_TFLOPS,
+                                  frac=fl * E / (ms * 1e-3) / 1e12 / FP32_PEAK_TFLOPS if fl else None,
+                                  peak_source="nominal: unit counts x 2.07 GHz max SM clock")
         del D
     return out
 
@@ -501,9 +499,9 @@ def kernel_rooflines(torch, B, mixed, fp64, stream, peaks, ref_cfg):
                     "peak_source": "nominal: unit counts x 2.07 GHz max SM clock",
                     "work_source": "executed FP ops per element (ncu, profiles/kernel_work.json)"})
 
-    alu("face_kernel<3,float,1> (smoother JVP, faces; FP32 with cached traces)", mixed, B.KT_FACE_JVP,
+    alu("face32_kernel<5,1> (smoother JVP, faces by sum factorisation; FP32 with cached traces)", mixed, B.KT_FACE_JVP,
         "face_jvp_fp32", FP32_PEAK_TFLOPS, "f32")
-    alu("volume_kernel_st<3,1,3> (smoother JVP, volume; FP32, tables in shared memory)", mixed, B.KT_VOLUME_JVP,
+    alu("vol32_kernel<5,1> (smoother JVP, volume by sum factorisation; FP32 with cached traces)", mixed, B.KT_VOLUME_JVP,
         "volume_jvp_fp32", FP32_PEAK_TFLOPS, "f32")
     if fp64 is not None:
         alu("face_sf_kernel<double,1> (outer JVP, faces by sum factorisation; FP64)", fp64, B.KT_FACE_JVP, "face_jvp_fp64",
@@ -847,7 +845,7 @@ def run_gb300(args):
                      "peak_source": "of fallback" if peaks.get("fallback") else "of measured (MEASURED_PEAKS.json hbm_gbs)",
                      "ms": bj["ms"], "algorithmic_bytes": bj["bytes"]},
         "jvp_fp64": roof["jvp_fp64"],
-        "probe_tc": roof.get("probe_tc"),
+        "block_probe": roof.get("block_probe"),
         "mixed_bf16": bf16,
         "large_dt": large,
         "tgv32_p6": c3,

@@ -11,57 +11,76 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-__device__ __forceinline__ uint4 ld_pair(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p)
-               : "memory");
+// A word and its epoch in one 64-bit element, and two such elements in one
+// 16-byte access.  PTX makes each element of a vector access single-copy atomic,
+// no more: the two words of an element always arrive together, the two elements
+// may not, so every element carries its own epoch.  (With elements of 32 bits a
+// reader could see the new epoch beside the old word.)
+using Word = unsigned long long;
+struct __align__(16) Pair {
+  Word a, b;
+};
+__device__ __forceinline__ Word with_epoch(unsigned x, unsigned ep) { return ((Word)ep << 32) | x; }
+__device__ __forceinline__ bool has_epoch(Word v, unsigned ep) { return (unsigned)(v >> 32) == ep; }
+__device__ __forceinline__ Word ld_word(const Word* p) {
+  Word v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_pair(uint4* p, unsigned x, unsigned y, unsigned ep) {
-  asm volatile("st.volatile.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(x), "r"(ep), "r"(y), "r"(ep) : "memory");
+__device__ __forceinline__ void st_word(Word* p, Word v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ Pair ld_pair(const Pair* p) {
+  Pair v;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0,%1}, [%2];" : "=l"(v.a), "=l"(v.b) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_pair(Pair* p, unsigned x, unsigned y, unsigned ep) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1,%2};" ::"l"(p), "l"(with_epoch(x, ep)), "l"(with_epoch(y, ep))
+               : "memory");
 }
 
-// What travels between the CTAs, every 32-bit word of a value beside its epoch:
-// Z a direction's entry, P a pair of sums (s, t).  An FP64 value is two words
-// with an epoch each, so neither needs more than 8 bytes to arrive at once.
+// What travels between the CTAs, every 32-bit word of a value in an element
+// with its epoch: Z a direction's entry, P a pair of sums (s, t).
 template <class V>
 struct Xch;
 template <>
 struct Xch<float> {
-  using Z = unsigned long long;
-  using P = uint4;
+  using Z = Word;
+  using P = Pair;
   using V2 = float2;
-  __device__ __forceinline__ static Z ld(const Z* p) {
-    Z v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-  }
-  __device__ __forceinline__ static bool has(Z v, unsigned ep) { return (unsigned)(v >> 32) == ep; }
+  __device__ __forceinline__ static Z ld(const Z* p) { return ld_word(p); }
+  __device__ __forceinline__ static bool has(Z v, unsigned ep) { return has_epoch(v, ep); }
   __device__ __forceinline__ static float val(Z v) { return __uint_as_float((unsigned)v); }
   __device__ __forceinline__ static void st(Z* p, float f, unsigned ep) {
-    const Z v = ((Z)ep << 32) | __float_as_uint(f);
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+    st_word(p, with_epoch(__float_as_uint(f), ep));
   }
   __device__ __forceinline__ static P ldp(const P* p) { return ld_pair(p); }
-  __device__ __forceinline__ static bool hasp(const P& q, unsigned ep) { return q.y == ep && q.w == ep; }
-  __device__ __forceinline__ static V2 valp(const P& q) { return make_float2(__uint_as_float(q.x), __uint_as_float(q.z)); }
+  __device__ __forceinline__ static bool hasp(const P& q, unsigned ep) {
+    return has_epoch(q.a, ep) && has_epoch(q.b, ep);
+  }
+  __device__ __forceinline__ static V2 valp(const P& q) {
+    return make_float2(__uint_as_float((unsigned)q.a), __uint_as_float((unsigned)q.b));
+  }
   __device__ __forceinline__ static void stp(P* p, float s, float t, unsigned ep) {
     st_pair(p, __float_as_uint(s), __float_as_uint(t), ep);
   }
 };
 struct Pair64 {
-  uint4 s, t;
+  Pair s, t;
 };
 template <>
 struct Xch<double> {
-  using Z = uint4;
+  using Z = Pair;
   using P = Pair64;
   using V2 = double2;
   __device__ __forceinline__ static Z ld(const Z* p) { return ld_pair(p); }
-  __device__ __forceinline__ static bool has(const Z& v, unsigned ep) { return v.y == ep && v.w == ep; }
-  __device__ __forceinline__ static double val(const Z& v) { return __hiloint2double((int)v.z, (int)v.x); }
+  __device__ __forceinline__ static bool has(const Z& v, unsigned ep) {
+    return has_epoch(v.a, ep) && has_epoch(v.b, ep);
+  }
+  __device__ __forceinline__ static double val(const Z& v) {
+    return __hiloint2double((int)(unsigned)v.b, (int)(unsigned)v.a);
+  }
   __device__ __forceinline__ static void st(Z* p, double f, unsigned ep) {
     st_pair(p, (unsigned)__double2loint(f), (unsigned)__double2hiint(f), ep);
   }

@@ -27,8 +27,8 @@
 //    The directions z_j = D^{-1} v_j are those of the first pass: the outer
 //    form is flexible (A Z = V H holds for any Z), so they need no second pass.
 //  * No barriers: every value that another CTA needs travels with its epoch in
-//    the same 8 (z_j) or 2 x 8 bytes (the partial sums), and the reader polls
-//    the value itself.  The partial sums take two such hops (to the CTA that
+//    the same 8-byte element (dg_exchange.cuh), and the reader polls the value
+//    itself.  The partial sums take two such hops (to the CTA that
 //    owns the sum and back), the directions one, in place of arrival, sum,
 //    release and read.  Epochs only grow (a word in device memory holds the next one), so
 //    nothing is cleared between calls.  z_j's buffer is reused every

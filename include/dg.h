@@ -272,7 +272,10 @@ typedef struct {
  * and the host waits once per cycle; the FD modes and triangle meshes read the
  * residual estimate on the host once per iteration.  Blocks until the solve
  * ends; stats (host, may be NULL) is filled in.  Returns DG_OK,
- * DG_ERR_NOT_CONVERGED, DG_ERR_BREAKDOWN or an error of the calls above. */
+ * DG_ERR_NOT_CONVERGED, DG_ERR_BREAKDOWN or an error of the calls above.
+ * DG_ERR_TIMEOUT (a bounded device wait of this or an earlier call on the mesh
+ * ran out, not yet cleared by dg_status_sync) wins over the others; dW is then
+ * zero and the residual estimate means nothing. */
 dg_status dg_fgmres_step(dg_mesh mesh, dg_pmg pmg, const double* W, const double* b,
                          double sigma, const dg_krylov_opts* opts, double* dW,
                          dg_krylov_stats* stats, void* stream);
@@ -298,7 +301,8 @@ dg_status dg_esdirk3_rhs(dg_mesh mesh, const double* Wk, const double* Wn, doubl
  * step ends.  stats (host, may be NULL): iterations summed over the 3*newton
  * solves, ms_total summed, res0/res_final/rho of the last solve.  Returns
  * DG_OK, DG_ERR_NOT_CONVERGED if some solve stopped above tolerance (the step
- * still completes), or an error of the calls above. */
+ * still completes), or an error of the calls above (Wout then holds the stage
+ * iterate that the failed solve started from). */
 dg_status dg_esdirk3_step(dg_mesh mesh, dg_pmg pmg, const double* Wn, double dt, int newton,
                           const dg_krylov_opts* kopts, double* work, size_t work_bytes, double* Wout,
                           dg_krylov_stats* stats, void* stream);

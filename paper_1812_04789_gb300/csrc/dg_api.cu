@@ -759,8 +759,11 @@ extern "C" dg_status dg_pmg_export_blocks(dg_pmg h, int level, int which, void* 
 namespace dgk {
 // prm: [0] rtol, [1] atol, [2] ||b|| (set on cycle 0), [3] tol, [4] residual estimate, [5] cycle
 // iq:  [0] iterations of this cycle, [1] stop reason (0 none yet, 1 converged, 2 non-finite,
-//      3 iteration limit, 4 Krylov space exhausted)
-__global__ void fgm_start_kernel(cudaGraphConditionalHandle h0, const double* res, int* kdim, double* prm, int* iq) {
+//      3 iteration limit, 4 Krylov space exhausted, 5 a bounded wait ran out)
+// A wait that runs out (ST_TIMEOUT in the status word) leaves the Arnoldi step's
+// outputs unwritten: nothing of the cycle is then used (kdim = 0).
+__global__ void fgm_start_kernel(cudaGraphConditionalHandle h0, const double* res, int* kdim, double* prm, int* iq,
+                                 const int* status) {
   const double beta = res[1];
   if (prm[5] == 0.0) prm[2] = beta;
   const double tol = fmax(prm[0] * prm[2], prm[1]);
@@ -768,20 +771,26 @@ __global__ void fgm_start_kernel(cudaGraphConditionalHandle h0, const double* re
   prm[4] = beta;
   iq[0] = 0;
   iq[1] = 0;
-  const bool fin = isfinite(beta) != 0;
-  const bool go = fin && beta > tol;
+  const bool fin = isfinite(beta) != 0, timed_out = *status & ST_TIMEOUT;
+  const bool go = fin && beta > tol && !timed_out;
   if (!go) {
     kdim[0] = 0;
-    iq[1] = fin ? 1 : 2;
+    iq[1] = timed_out ? 5 : fin ? 1 : 2;
   }
   cudaGraphSetConditional(h0, go ? 1u : 0u);
 }
 
 __global__ void fgm_check_kernel(cudaGraphConditionalHandle hn, int has_next, int j, int restart, const double* res,
-                                 int* kdim, double* prm, int* iq) {
+                                 int* kdim, double* prm, int* iq, const int* status) {
   const double r = res[0];
-  prm[4] = r;
   iq[0] = j + 1;
+  if (*status & ST_TIMEOUT) {
+    kdim[0] = 0;
+    iq[1] = 5;
+    if (has_next) cudaGraphSetConditional(hn, 0u);
+    return;
+  }
+  prm[4] = r;
   const bool nonfin = (kdim[1] & ST_NONFINITE) || !isfinite(r);
   const bool conv = !nonfin && r <= prm[3];
   const bool exhausted = kdim[0] <= j + 1 && j + 1 < restart;
@@ -863,7 +872,7 @@ static cudaError_t build_fgm_graph(dg_pmg h, int restart, double sigma) {
     cudaError_t e1 = K.start(h->fgm_r0, st);
     if (e1 == cudaSuccess) {
       note_launch();
-      fgm_start_kernel<<<1, 1, 0, st>>>(hc[0], K.res, K.kdim, h->fgm_prm, h->fgm_iq);
+      fgm_start_kernel<<<1, 1, 0, st>>>(hc[0], K.res, K.kdim, h->fgm_prm, h->fgm_iq, h->mesh->m.status);
       e1 = cudaGetLastError();
     }
     cudaGraph_t gg = g;
@@ -891,7 +900,7 @@ static cudaError_t build_fgm_graph(dg_pmg h, int restart, double sigma) {
     if (e1 == cudaSuccess) {
       note_launch();
       fgm_check_kernel<<<1, 1, 0, st>>>(j + 1 < restart ? hc[j + 1] : hc[j], j + 1 < restart ? 1 : 0, j, restart,
-                                        K.res, K.kdim, h->fgm_prm, h->fgm_iq);
+                                        K.res, K.kdim, h->fgm_prm, h->fgm_iq, h->mesh->m.status);
       e1 = cudaGetLastError();
     }
     cudaGraph_t bb = body;
@@ -928,6 +937,22 @@ static cudaError_t build_fgm_graph(dg_pmg h, int restart, double sigma) {
   }
   h->fgm_graph = g;
   return cudaSuccess;
+}
+
+// The status of a finished solve.  A bounded wait that ran out (ST_TIMEOUT) wins
+// over what the iteration came to, which rests on values that were not written:
+// the caller gets DG_ERR_TIMEOUT and dW = 0.
+static dg_status solve_status(const Mesh& M, dg_status s, bool converged, double* dW, long N, cudaStream_t st) {
+  if (s == DG_OK && !converged) s = DG_ERR_NOT_CONVERGED;
+  int hs = 0;
+  CK(cudaMemcpyAsync(&hs, M.status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  if (hs & ST_TIMEOUT) {
+    CK(cudaMemsetAsync(dW, 0, sizeof(double) * N, st));
+    CK(cudaStreamSynchronize(st));
+    return DG_ERR_TIMEOUT;
+  }
+  return s == DG_OK && (hs & ST_NONPHYSICAL) ? DG_ERR_NONPHYSICAL : s;
 }
 
 // FGMRES with the exact JVP through the cycle graph: one host synchronisation
@@ -981,6 +1006,7 @@ static dg_status fgmres_graph(dg_pmg h, const double* W, const double* b, double
     iters += hq[0];
     if (cycle == 0) bnorm = hp[2];
     res = hp[4];
+    if (hq[1] == 5) break;   // (solve_status reports it)
     if (hq[1] == 2) {
       s = DG_ERR_BREAKDOWN;
       break;
@@ -996,13 +1022,7 @@ static dg_status fgmres_graph(dg_pmg h, const double* W, const double* b, double
   if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (s == DG_OK && !converged) s = DG_ERR_NOT_CONVERGED;
-  if (s == DG_OK) {
-    int hs = 0;
-    cudaMemcpy(&hs, M.status, sizeof(int), cudaMemcpyDeviceToHost);
-    if (hs & ST_TIMEOUT) s = DG_ERR_TIMEOUT;
-    else if (hs & ST_NONPHYSICAL) s = DG_ERR_NONPHYSICAL;
-  }
+  s = solve_status(M, s, converged, dW, N, st);
   if (stats) {
     stats->iters = iters;
     stats->res0 = bnorm;
@@ -1079,10 +1099,12 @@ extern "C" dg_status dg_fgmres_step(dg_mesh mesh, dg_pmg pmg, const double* W, c
       if (K.arnoldi(j, st) != cudaSuccess) { s = DG_ERR_CUDA; break; }
       ++iters;
       jdone = j + 1;
-      int kd[2];
+      int kd[2], hs = 0;
       if (cudaMemcpyAsync(host, K.res, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
           cudaMemcpyAsync(kd, K.kdim, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+          cudaMemcpyAsync(&hs, M.status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
           cudaStreamSynchronize(st) != cudaSuccess) { s = DG_ERR_CUDA; break; }
+      if (hs & ST_TIMEOUT) { s = DG_ERR_TIMEOUT; break; }
       res = host[0];
       if (kd[1] & ST_NONFINITE || !isfinite(res)) { s = DG_ERR_BREAKDOWN; break; }
       if (res <= tol) { converged = true; break; }
@@ -1096,13 +1118,7 @@ extern "C" dg_status dg_fgmres_step(dg_mesh mesh, dg_pmg pmg, const double* W, c
   if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (s == DG_OK && !converged) s = DG_ERR_NOT_CONVERGED;
-  if (s == DG_OK) {
-    int hs = 0;
-    cudaMemcpy(&hs, M.status, sizeof(int), cudaMemcpyDeviceToHost);
-    if (hs & ST_TIMEOUT) s = DG_ERR_TIMEOUT;
-    else if (hs & ST_NONPHYSICAL) s = DG_ERR_NONPHYSICAL;
-  }
+  s = solve_status(M, s, converged, dW, N, st);
   if (stats) {
     stats->iters = iters;
     stats->res0 = bnorm;

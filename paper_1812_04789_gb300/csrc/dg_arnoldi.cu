@@ -14,7 +14,7 @@
 // / 20; FP32, 100 x 75, p = 3 (up to 10): 31 / 20; 16^3, p = 4: 37 / 31; 16^3, p = 6:
 // 58 / 51.  Bound by the two exchanges and the launch, at 16^3 by the reads of V.
 // Every wait is bounded as in dg_smoother.cu: ST_TIMEOUT in the status word, and
-// the step's outputs are then untrusted.
+// the step's outputs are then unwritten: the caller stops (fgm_check_kernel).
 #include <algorithm>
 
 #include "dg_exchange.cuh"
@@ -37,7 +37,7 @@ struct ArnArgs {
   unsigned* epoch;
   int* status;
   long N, chunk;
-  int j, ni;
+  int j, ni, extra;     // extra: CTAs that the exchanges wait for and that do not exist (a test's)
 };
 
 // a warp's sum of a[r] b[r] over its lanes' rows r = lane, lane + 32, .. < n
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) arnoldi_kernel(ArnArgs<T> a) {
       Xch<double>::stp(px + (size_t)i * (G + 1) + blockIdx.x, s, 0.0, ep);
     }
     const bool ok =
-        gather_dots<double, ARN_WARPS>(px, G + 1, items, G, a.sums + (size_t)pass * a.ni, ep, a.status, st);
+        gather_dots<double, ARN_WARPS>(px, G + 1, items, G + a.extra, a.sums + (size_t)pass * a.ni, ep, a.status, st);
     if (__syncthreads_or(ok ? 0 : 1)) {
       if (tid == 0) atomicMax(a.epoch, base + 8u);
       return;
@@ -264,6 +264,8 @@ cudaError_t plan_arnoldi(Krylov<T>& K, size_t* bytes) {
   if (occ < 1) return cudaSuccess;
   K.ag = (int)((K.N + chunk - 1) / chunk);      // no CTA without entries
   K.achunk = chunk;
+  const char* extra = getenv("DG_TEST_ARNOLDI_EXTRA");   // test hook: an exchange that is never complete
+  K.aextra = extra && extra[0] == '1' ? 1 : 0;
   *bytes = sizeof(Pair64) * 2 * (size_t)ni * (K.ag + 2) + sizeof(double) * (size_t)ni * ni;
   return cudaSuccess;
 }
@@ -288,6 +290,7 @@ cudaError_t launch_arnoldi(const Krylov<T>& K, int j, cudaStream_t st) {
   a.N = K.N;
   a.chunk = K.achunk;
   a.j = j;
+  a.extra = K.aextra;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(K.ag);
   cfg.blockDim = dim3(ARN_THREADS);

@@ -334,9 +334,9 @@ struct Krylov {
   double* res = nullptr;     // residual estimate |g[j+1]|
   int* kdim = nullptr;       // [0] effective Krylov dimension (breakdown), [1] status bits
   // one-kernel Arnoldi step (csrc/dg_arnoldi.cu): CTAs (0: a kernel per
-  // operation), entries of a vector per CTA, the exchange's buffers (launches that share
+  // operation), a test's CTA that never arrives, entries of a vector per CTA, the exchange's buffers (launches that share
   // them are ordered on one stream) and the word that takes ST_TIMEOUT
-  int ag = 0;
+  int ag = 0, aextra = 0;
   long achunk = 0;
   void* apx = nullptr;
   unsigned* aepoch = nullptr;

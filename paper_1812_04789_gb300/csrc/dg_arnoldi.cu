@@ -7,7 +7,8 @@
 // size: on 16^2 quads at p = 2 (6,144 unknowns) 32 of an FGMRES iteration's 90
 // us.  Here the CTAs exchange the sums of the two passes by polled values
 // (dg_exchange.cuh, two exchanges of 3 to 4 us; the norm comes with the second
-// pass), and w stays in shared memory.  The sums are those of mdot_kernel: FP64 vectors in FP64;
+// pass, |w - V h|^2 = w.w - h.h, and from a third exchange where that cancels: an
+// exhausted Krylov space), and w stays in shared memory.  The sums are those of mdot_kernel: FP64 vectors in FP64;
 // FP32 vectors with at most 16 products per FP64 addition, a CTA's lanes in
 // FP32, the CTAs in FP64.  Fixed order: results do not depend on timing.
 // us per step, kernels per operation / here: FP64, 16^2, p = 2 (up to 45 vectors): 32
@@ -62,6 +63,15 @@ __device__ __forceinline__ double warp_dot(const float* a, const float* b, int n
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   return (double)t;
+}
+
+// the norm and its reciprocal from its square; 0 and 0 where that is zero or not finite
+__device__ __forceinline__ void set_norm(double s, double* nrm, double* inv, int* bad) {
+  const bool fin = isfinite(s);
+  const double i = s > 0.0 && fin ? rsqrt(s) : 0.0;
+  *inv = i;
+  *nrm = s > 0.0 && fin ? s * i : 0.0;
+  *bad = !fin;
 }
 
 // w -= V h, four rows of a thread together (their loads in flight); few rows:
@@ -120,6 +130,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) arnoldi_kernel(ArnArgs<T> a) {
   T* ws = ps + ARN_THREADS;                             // [chunk]
   __shared__ int timed_out;
   __shared__ double s_nrm, s_inv;
+  __shared__ int s_expl, s_bad;
   const long beg = min(a.N, blockIdx.x * a.chunk);
   const int n = (int)(min(a.N, beg + a.chunk) - beg);
   if (tid == 0) timed_out = (*(volatile int*)a.status & ST_TIMEOUT) ? 1 : 0;
@@ -170,25 +181,18 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) arnoldi_kernel(ArnArgs<T> a) {
     for (int i = tid; i < nv; i += ARN_THREADS) hs[i] = st[i].x;
     __syncthreads();
   }
-  // |w - V h2|^2 = w.w - h2.h2 (h2 is the rounding of the first pass along V)
+  // |w - V h2|^2 = w.w - h2.h2 (h2 is the rounding of the first pass along V),
+  // unless h2 carries half of w: then w is little but rounding, and the
+  // difference too, and the norm is summed over what is left
   if (warp == 0) {
     double h2 = 0.0;
     for (int i = lane; i < nv; i += 32) h2 = fma(st[i].x, st[i].x, h2);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) h2 += __shfl_xor_sync(0xffffffffu, h2, o);
     const double ww = st[nv].x, s = ww - h2;
-    double nrm = 0.0, inv = 0.0;
-    if (s > 0.0 && isfinite(s)) {
-      inv = rsqrt(s);
-      nrm = s * inv;
-    }
     if (lane == 0) {
-      s_nrm = nrm;
-      s_inv = inv;
-      if (blockIdx.x == 0) {
-        if (!isfinite(s)) atomicOr(a.kdim + 1, ST_NONFINITE);
-        if (!(nrm > 0.0) && *a.kdim > j + 1) *a.kdim = j + 1;
-      }
+      s_expl = s < 0.5 * ww;
+      set_norm(s, &s_nrm, &s_inv, &s_bad);
     }
   } else if (blockIdx.x == 0) {
     // the old rotations on the new column: entry i < j becomes c_i (q_i . h[0..i]) +
@@ -209,6 +213,29 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) arnoldi_kernel(ArnArgs<T> a) {
   }
   subtract(Vc, a.N, st, nv, n, ws, ps);
   __syncthreads();
+  if (s_expl) {      // (the same in every CTA; every CTA is done with the first pass' buffers)
+    const unsigned ep = base + 3u;
+    const int per = (n + ARN_WARPS - 1) / ARN_WARPS, r0 = min(n, warp * per), m = min(n, r0 + per) - r0;
+    const double s = warp_dot(ws + r0, ws + r0, m);
+    if (lane == 0) red[1 + warp] = s;      // (red[0]: the rotations' last entry)
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int k = 0; k < ARN_WARPS; ++k) t += red[1 + k];
+      Xch<double>::stp(a.px + blockIdx.x, t, 0.0, ep);
+    }
+    const bool ok = gather_dots<double, ARN_WARPS>(a.px, G + 1, 1, G + a.extra, a.sums, ep, a.status, st);
+    if (__syncthreads_or(ok ? 0 : 1)) {
+      if (tid == 0) atomicMax(a.epoch, base + 8u);
+      return;
+    }
+    if (tid == 0) set_norm(st[0].x, &s_nrm, &s_inv, &s_bad);
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    if (s_bad) atomicOr(a.kdim + 1, ST_NONFINITE);
+    if (!(s_nrm > 0.0) && *a.kdim > j + 1) *a.kdim = j + 1;
+  }
   T* vn = a.V + (size_t)nv * a.N + beg;
   const T inv = (T)s_inv;
   for (int r = tid; r < n; r += ARN_THREADS) vn[r] = inv * ws[r];

@@ -33,7 +33,7 @@ struct ArnArgs {
   double *H, *cs, *sn, *g, *res;   // H: column j
   int* kdim;
   Pair64* px;           // [2][nmax + 2][G + 1] partial sums
-  Pair64* sums;         // [2][nmax + 2]
+  Pair64* sums;         // [2][nmax + 2][SUM_STRIDE]
   double* Q;            // [nmax + 2][nmax + 2] the q_i
   unsigned* epoch;
   int* status;
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) arnoldi_kernel(ArnArgs<T> a) {
       Xch<double>::stp(px + (size_t)i * (G + 1) + blockIdx.x, s, 0.0, ep);
     }
     const bool ok =
-        gather_dots<double, ARN_WARPS>(px, G + 1, items, G + a.extra, a.sums + (size_t)pass * a.ni, ep, a.status, st);
+        gather_dots<double, ARN_WARPS>(px, G + 1, items, G + a.extra, a.sums + (size_t)pass * a.ni * SUM_STRIDE, ep, a.status, st);
     if (__syncthreads_or(ok ? 0 : 1)) {
       if (tid == 0) atomicMax(a.epoch, base + 8u);
       return;
@@ -293,7 +293,7 @@ cudaError_t plan_arnoldi(Krylov<T>& K, size_t* bytes) {
   K.achunk = chunk;
   const char* extra = getenv("DG_TEST_ARNOLDI_EXTRA");   // test hook: an exchange that is never complete
   K.aextra = extra && extra[0] == '1' ? 1 : 0;
-  *bytes = sizeof(Pair64) * 2 * (size_t)ni * (K.ag + 2) + sizeof(double) * (size_t)ni * ni;
+  *bytes = sizeof(Pair64) * 2 * (size_t)ni * (K.ag + 1 + SUM_STRIDE) + sizeof(double) * (size_t)ni * ni;
   return cudaSuccess;
 }
 
@@ -311,7 +311,7 @@ cudaError_t launch_arnoldi(const Krylov<T>& K, int j, cudaStream_t st) {
   a.ni = K.nmax + 2;
   a.px = (Pair64*)K.apx;
   a.sums = a.px + 2 * (size_t)a.ni * (K.ag + 1);
-  a.Q = (double*)(a.sums + 2 * (size_t)a.ni);
+  a.Q = (double*)(a.sums + 2 * (size_t)a.ni * SUM_STRIDE);
   a.epoch = K.aepoch;
   a.status = K.astatus;
   a.N = K.N;

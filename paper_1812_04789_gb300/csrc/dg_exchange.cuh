@@ -69,6 +69,10 @@ struct Xch<float> {
 struct Pair64 {
   Pair s, t;
 };
+// A published sum has a 128-byte line to itself: all CTAs poll all sums, and four
+// to a line it hung on where the lines lay (100 x 75, p = 0, nu = 30: 273 to 330 us a
+// smoother call over ten allocations, 281 to 283 with lines apart).
+constexpr int SUM_STRIDE = 128 / sizeof(Pair64);
 template <>
 struct Xch<double> {
   using Z = Pair;
@@ -110,14 +114,6 @@ struct Wait {
   }
 };
 
-// (h, l) += x, FP32 with the rounding error of the addition kept in l
-__device__ __forceinline__ void two_add(double& h, double&, double x) { h += x; }
-__device__ __forceinline__ void two_add(float& h, float& l, float x) {
-  const float s = h + x, b = s - h;
-  l += (h - (s - b)) + (x - b);
-  h = s;
-}
-
 // Sums of fs and ft over a warp: the first exchange leaves fs to the lower and
 // ft to the upper half, so five additions do for both.
 template <class V>
@@ -130,64 +126,92 @@ __device__ __forceinline__ void warp_sum2(V& fs, V& ft) {
   ft = __shfl_sync(0xffffffffu, a, 16);
 }
 
-// st[i] = the sums over all CTAs of the items i < ni of an exchange: CTA i mod G
-// owns item i, a warp of it polls the G partials in[i stride + c] (5 loads of a
-// lane at once), adds them (FP32: in two-float arithmetic), a lane's CTAs and then the
-// lanes by a butterfly, and publishes the sum, and one warp of every CTA
-// polls the ni sums.  Two hops of little traffic: one hop, with every CTA
-// reading all G x ni partials, saturated the L2 with polls and took 8 us.
-// False where a wait ran out.
+// A warp polls *p, a value a lane (lanes that are not active: nothing), until all
+// have arrived (each lane until its own has); false where the wait ran out.  All lanes go on together: lanes
+// that leave such a loop one after the other execute what follows one after the
+// other too, and an FP64 instruction holds its warp for 64 clocks however few of
+// its lanes take part.
+template <class X, class P>
+__device__ __forceinline__ bool poll_warp(const P* p, bool active, P& q, unsigned ep, Wait& wt, int* status) {
+  bool have = !active;
+  for (;;) {
+    if (!have) {
+      q = X::ldp(p);
+      have = X::hasp(q, ep);
+    }
+    if (__all_sync(0xffffffffu, have)) return true;
+    if (__any_sync(0xffffffffu, wt.expired(status))) return false;
+  }
+}
+
+// st[i] = sums[i SUM_STRIDE] = the sums over all CTAs of the items i < ni of an exchange, in FP64
+// whatever the partials' precision: CTA i mod G owns item i, a group of five warps
+// of it polls the G partials in[i stride + c], one a lane (152 CTAs), adds them
+// by butterflies and publishes the sum, and one warp of every CTA polls the ni
+// sums.  Two hops of little traffic: one hop, with every CTA reading all G x ni
+// partials, saturated the L2 with polls and took 8 us.  (One warp adding five
+// partials a lane would take 25 FP64 instructions in a row, five warps 10.)  False
+// where a wait ran out.
 template <class V, int WARPS>
-__device__ bool gather_dots(const typename Xch<V>::P* in, int stride, int ni, int G, typename Xch<V>::P* sums,
-                            unsigned ep, int* status, typename Xch<V>::V2* st) {
+__device__ bool gather_dots(const typename Xch<V>::P* in, int stride, int ni, int G, Pair64* sums, unsigned ep,
+                            int* status, double2* st) {
   using X = Xch<V>;
+  using X64 = Xch<double>;
+  constexpr int GW = 5, NG = (WARPS - 1) / GW;
+  __shared__ double2 gpart[2][NG][GW];     // (alternating: one barrier an item)
+  __shared__ int gok[2][NG][GW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, C = gridDim.x;
   bool ok = true;
   if (warp >= WARPS) return ok;
   Wait wt;
-  // (the owned items i = blockIdx.x + k C, shared out over the warps; warp 0 collects)
-  for (int i = blockIdx.x + (warp - 1) * C; warp > 0 && i < ni; i += (WARPS - 1) * C) {
-    V hs = V(0), ls = V(0), ht = V(0), lt = V(0);
-    for (int c0 = lane; c0 < G; c0 += 160) {
-      typename X::P q[5];
-#pragma unroll
-      for (int u = 0; u < 5; ++u) q[u] = X::ldp(in + (size_t)i * stride + min(c0 + 32 * u, G - 1));
-#pragma unroll
-      for (int u = 0; u < 5; ++u) {
-        if (c0 + 32 * u >= G) continue;
-        while (ok && !X::hasp(q[u], ep)) {
-          if (wt.expired(status)) ok = false;
-          q[u] = X::ldp(in + (size_t)i * stride + c0 + 32 * u);
+  const int g = (warp - 1) / GW, gw = warp - 1 - g * GW;
+  // (the owned items i = blockIdx.x + k C, shared out over the groups; warp 0 collects)
+  if (warp > 0 && g < NG) {
+    int par = 0;
+    for (int i = blockIdx.x + g * C; i < ni; i += NG * C, par ^= 1) {
+      double hs = 0.0, ht = 0.0;
+      for (int c0 = gw * 32; ok && c0 < G; c0 += GW * 32) {
+        const bool active = c0 + lane < G;
+        typename X::P q = {};
+        ok = poll_warp<X>(in + (size_t)i * stride + c0 + lane, active, q, ep, wt, status);
+        const typename X::V2 v = X::valp(q);
+        const double x = (double)v.x, y = (double)v.y;     // (0 where there is no CTA)
+        if (c0 == gw * 32) {
+          hs = x;
+          ht = y;
+        } else {
+          hs += x;
+          ht += y;
         }
-        const typename X::V2 v = X::valp(q[u]);
-        two_add(hs, ls, v.x);
-        two_add(ht, lt, v.y);
       }
-    }
-    if constexpr (std::is_same<V, double>::value) {
       warp_sum2(hs, ht);
-    } else {
+      if (lane == 0) {
+        gpart[par][g][gw] = make_double2(hs, ht);
+        gok[par][g][gw] = ok;
+      }
+      __syncwarp();
+      asm volatile("bar.sync %0, %1;" ::"r"(2 + g), "n"(GW * 32) : "memory");
+      if (gw == 0) {
+        const int k = min(lane & 15, GW - 1);
+        const double2 pr = gpart[par][g][k];
+        const bool in_k = (lane & 15) < GW, every = __all_sync(0xffffffffu, gok[par][g][k] != 0);
+        double a = lane & 16 ? pr.y : pr.x;
+        if (!in_k) a = 0.0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const V a = __shfl_xor_sync(0xffffffffu, hs, o), b = __shfl_xor_sync(0xffffffffu, ls, o);
-        const V c = __shfl_xor_sync(0xffffffffu, ht, o), d = __shfl_xor_sync(0xffffffffu, lt, o);
-        two_add(hs, ls, a);
-        ls += b;
-        two_add(ht, lt, c);
-        lt += d;
+        for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        const double t = __shfl_sync(0xffffffffu, a, 16);
+        if (every && lane == 0) X64::stp(sums + (size_t)i * SUM_STRIDE, a, t, ep);
       }
     }
-    if (__all_sync(0xffffffffu, ok) && lane == 0) X::stp(sums + i, hs + ls, ht + lt, ep);
   }
   if (warp == 0) {
-    for (int i = lane; i < ni; i += 32) {
-      typename X::P q = X::ldp(sums + i);
-      while (ok && !X::hasp(q, ep)) {
-        if (wt.expired(status)) ok = false;
-        q = X::ldp(sums + i);
-      }
-      st[i] = X::valp(q);
+    for (int i0 = 0; ok && i0 < ni; i0 += 32) {
+      const bool active = i0 + lane < ni;
+      Pair64 q = {};
+      ok = poll_warp<X64>(sums + (size_t)(i0 + lane) * SUM_STRIDE, active, q, ep, wt, status);
+      if (active) st[i0 + lane] = X64::valp(q);
     }
+    __syncwarp();
   }
   return ok;
 }

@@ -37,17 +37,16 @@
 // Per iteration j:
 //   w = A z_j (own rows; the neighbours' z_j polled), partials        | exchange
 //   second pass for v_j, v_{j+1}, z_{j+1} = D^{-1} v_{j+1} published
-// The sums over the CTAs are in two-float arithmetic (the exact error of every
-// addition carried along, 48 bits) and in a fixed order, rounded to FP32 at the
-// end; all CTAs hold identical scalars and the final x += Z y needs no
-// exchange.  FP64 sums cost more than a hop (GB300 has two FP64 lanes per SM).  The arithmetic inside a CTA is FP32.  A warp of its own
+// The sums over the CTAs, the squared norms, their differences and roots and a new
+// Hessenberg column are FP64 and in a fixed order, the column rounded once when
+// it is complete; all CTAs hold identical scalars and the final x += Z y needs no
+// exchange.  The arithmetic inside a CTA is FP32.  A warp of its own
 // keeps the Hessenberg matrix, the Givens rotations (behind the next
 // exchange's wait) and the small least-squares solve off the critical path;
 // one warp takes the scalars of an exchange.
-// 16^3 elements, p_fine = 4 (us per call): p = 2, nu = 10: 880 -> 765;
-// p = 1, nu = 10: 400 -> 188; p = 0, nu = 30: 690 -> 290.
-// FP64 handles run the same kernel on FP64 vectors and blocks, the sums over the
-// CTAs plain.  Bound by the FP64 pipe at p = 2 (the block-sparse product), by the
+// 16^3 elements, p_fine = 4 (us per call, means over ten allocations): p = 2, nu
+// = 10: 880 -> 746; p = 1, nu = 10: 400 -> 180; p = 0, nu = 30: 690 -> 265.
+// FP64 handles run the same kernel on FP64 vectors and blocks.  Bound by the FP64 pipe at p = 2 (the block-sparse product), by the
 // exchanges below; the launch-per-operation smoother spent half of its time
 // on kernels of 2 to 5 us.  9 x 10 x 12, p = 3: FP64 step 116 -> 85 ms.
 //
@@ -141,7 +140,7 @@ struct CoopArgs {
   V* x;
   typename Xch<V>::Z* zx;     // [N] the direction z_j
   typename Xch<V>::P* px;     // [2][ni][grid + 1] the CTAs' partial sums
-  typename Xch<V>::P* sums;   // [2][ni] their sums over the CTAs
+  Pair64* sums;               // [2][ni][SUM_STRIDE] their sums over the CTAs
   unsigned* epoch;      // first free epoch - 1
   int* status;          // mesh status word (ST_TIMEOUT)
   int* kflag;           // Krylov status bits (ST_NONFINITE)
@@ -187,55 +186,63 @@ __device__ void publish_dots(int j, const V* Vs, int ldv, const V* w, int rows, 
 
 // The scalars of exchange j (see the head of the file), by one warp from the
 // sums in st: FP64 square roots and sums in all seventeen warps would cost more
-// than the exchange (two FP64 lanes per SM).  FP64 takes a power of two as rho
-// (any scale will do), whose reciprocal is exact.
+// than the exchange (two FP64 lanes per SM; an instruction holds its warp for 64
+// clocks, so what can be is one instruction on two lanes' values, and no lane
+// leaves the others).  sv: the sums rounded to V (FP64 vectors take st).  rho is
+// a scale only: a power of two, whose reciprocal is exact, near the norm as
+// estimated in V.
 template <class V>
 struct Scal {
-  V beta, ib, hj, rho, ir;
+  V ib, hj, ir;
+  double beta, hjd, rho;
   int fine, bad;
 };
 template <class V>
-__device__ void exchange_scalars(const typename Xch<V>::V2* st, int j, Scal<V>* sc) {
+__device__ void exchange_scalars(const double2* st, typename Xch<V>::V2* sv, int j, Scal<V>* sc) {
   const int lane = threadIdx.x & 31;
-  V ss = V(0), sq = V(0), tq = V(0), none = V(0);
-  for (int i = lane; i < j; i += 32) {
-    const typename Xch<V>::V2 q = st[i];
-    ss = fma(q.x, q.x, ss);
-    sq = fma(q.x, q.y, sq);
-    tq = fma(q.y, q.y, tq);
+  double be2 = 0.0, hb = 0.0;     // v_j.v_j - s.s, v_j.w - s.V^T w
+  V tq = V(0), ww = V(0);
+  for (int i0 = 0; i0 < j + 2; i0 += 32) {
+    const int i = i0 + lane;
+    const double2 q = st[min(i, j + 1)];
+    typename Xch<V>::V2 r;
+    r.x = (V)q.x;
+    r.y = (V)q.y;
+    if (sizeof(V) == 4 && i < j + 2) sv[i] = r;
+    // below j minus the product, at j the sum itself
+    const double a = i < j ? -q.x : 1.0;
+    be2 = fma(a, i <= j ? q.x : 0.0, be2);
+    hb = fma(a, i <= j ? q.y : 0.0, hb);
+    const V t = i < j ? r.y : V(0);
+    tq = fma(t, t, tq);
+    ww = i == j + 1 ? r.x : ww;
   }
-  warp_sum2(ss, sq);
-  warp_sum2(tq, none);
-  const V be2 = st[j].x - ss, ww = st[j + 1].x;
-  const bool fine = be2 > V(0) && isfinite(be2);
-  V beta = V(0), ib = V(0);
-  if (fine) {
-    if constexpr (std::is_same<V, double>::value) {
-      ib = rsqrt(be2);
-      beta = be2 * ib;
-    } else {
-      beta = sqrtf(be2);
-      ib = 1.f / beta;
-    }
-  }
-  const V hj = (st[j].y - sq) * ib, est = fmax(ww - tq - hj * hj, V(1e-6) * ww);
-  V rho = V(1), ir = V(1);
-  if (est > V(0) && isfinite(est)) {
-    if constexpr (std::is_same<V, double>::value) {
-      const int e = ((__double2hiint(est) >> 20) - 1023) >> 1;   // est is normal: |e| <= 512
-      rho = __hiloint2double((1023 + e) << 20, 0);
-      ir = __hiloint2double((1023 - e) << 20, 0);
-    } else {
-      rho = sqrtf(est);
-      ir = 1.f / rho;
-    }
-  }
-  if (lane == 0) {
-    sc->beta = beta;
-    sc->ib = ib;
-    sc->hj = hj;
-    sc->rho = rho;
-    sc->ir = ir;
+  warp_sum2(be2, hb);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tq += __shfl_xor_sync(0xffffffffu, tq, o);
+  ww = __shfl_sync(0xffffffffu, ww, (j + 1) & 31);
+  const bool fine = be2 > 0.0 && isfinite(be2);
+  const double ib = rsqrt(fine ? be2 : 1.0);
+  const double pr = (lane == 0 ? be2 : hb) * ib;       // beta, h_j
+  const V cv = (V)(lane == 0 ? ib : pr);
+  const V hj = __shfl_sync(0xffffffffu, cv, 1);
+  const V est = fmax(ww - tq - hj * hj, V(1e-6) * ww);
+  const bool use = est > V(0) && isfinite(est);
+  int e;       // |e| <= 512, FP32 64
+  if constexpr (std::is_same<V, double>::value)
+    e = use ? ((__double2hiint(est) >> 20) - 1023) >> 1 : 0;
+  else
+    e = use ? ((__float_as_int(est) >> 23) - 127) >> 1 : 0;
+  if (lane < 2) {
+    double* o = lane == 0 ? &sc->beta : &sc->hjd;
+    V* v = lane == 0 ? &sc->ib : &sc->hj;
+    *o = pr;
+    *v = cv;
+    sc->rho = __hiloint2double((1023 + e) << 20, 0);
+    if constexpr (std::is_same<V, double>::value)
+      sc->ir = __hiloint2double((1023 - e) << 20, 0);
+    else
+      sc->ir = __int_as_float((127 - e) << 23);
     sc->fine = fine;
     sc->bad = !fine && !isfinite(be2);
   }
@@ -396,7 +403,9 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
   V* sn = cs + nu;
   V* g = sn + nu;                                 // nu + 1, then y
   int* src = reinterpret_cast<int*>(g + ldh);         // [chunk][NSRC] element ids
-  typename X::V2* st = reinterpret_cast<typename X::V2*>((reinterpret_cast<uintptr_t>(src + (size_t)a.chunk * NSRC) + 15) & ~(uintptr_t)15);   // [nu + 2]
+  double2* st = reinterpret_cast<double2*>((reinterpret_cast<uintptr_t>(src + (size_t)a.chunk * NSRC) + 15) & ~(uintptr_t)15);   // [nu + 2]
+  double* hd = reinterpret_cast<double*>(st + nu + 2);   // [nu + 1] the Hessenberg column begun
+  typename X::V2* sv = sizeof(V) == 4 ? reinterpret_cast<typename X::V2*>(hd + ldh) : reinterpret_cast<typename X::V2*>(st);   // st in V
   __shared__ int timed_out;
   __shared__ Scal<V> scal;
 
@@ -469,7 +478,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
     const V* none = nullptr;
     COOP_PRODUCT(none, 0u, a.b, Vs, false)
   }
-  V rho = V(1);             // |w - V h| as estimated: v_{j+1} = (w - V h) / rho
+  double rho = 1.0;         // |w - V h| as estimated: v_{j+1} = (w - V h) / rho
   int kdone = 0;
   for (int j = 0;; ++j) {
     const unsigned ep = base + 1u + (unsigned)j;
@@ -523,28 +532,23 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
     if (scalar_warp) {
       if (j >= 2 && lane == 0) rotate_column(H, ldh, j - 2, cs, sn, g);   // behind the exchange
     } else {
-      got = gather_dots<V, COOP_WORK / 32>(px, G + 1, j + 2, G + a.extra, a.sums + (j & 1) * a.ni, ep, a.status, st);
-      if (warp == 0) {
-        __syncwarp();
-        exchange_scalars<V>(st, j, &scal);
-      }
+      got = gather_dots<V, COOP_WORK / 32>(px, G + 1, j + 2, G + a.extra, a.sums + (j & 1) * a.ni * SUM_STRIDE, ep, a.status, st);
+      if (warp == 0) exchange_scalars<V>(st, sv, j, &scal);
     }
     COOP_LEAVE_IF(!got)
     const bool fine = scal.fine;
-    const V beta = scal.beta, ib = scal.ib, hj = scal.hj;
+    const V ib = scal.ib, hj = scal.hj;
     if (scalar_warp) {
       // column j - 1 completed, column j begun (this warp alone)
       if (j == 0) {
-        for (int i = lane; i < ldh; i += 32) g[i] = i == 0 ? beta : V(0);
+        for (int i = lane; i < ldh; i += 32) g[i] = i == 0 && fine ? (V)scal.beta : V(0);
       } else {
         V* h = H + (size_t)(j - 1) * ldh;
-        for (int i = lane; i < j; i += 32) h[i] = fma(rho, st[i].x, h[i]);
-        if (lane == 0) h[j] = rho * beta;
+        for (int i = lane; i < j; i += 32) h[i] = (V)fma(rho, st[i].x, hd[i]);
+        if (lane == 0) h[j] = fine ? (V)(rho * scal.beta) : V(0);
       }
-      if (j < nu && fine) {
-        V* h = H + (size_t)j * ldh;
-        for (int i = lane; i <= j; i += 32) h[i] = i < j ? st[i].y : hj;
-      }
+      if (j < nu && fine)
+        for (int i = lane; i <= j; i += 32) hd[i] = i < j ? st[i].y : scal.hjd;
       __syncwarp();
     }
     kdone = j;
@@ -561,7 +565,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) coop_smooth_kernel(CoopArgs<S
         const V* q = Vs + r;
 #pragma unroll 8
         for (int i = 0; i < j; ++i) {
-          const typename X::V2 c = st[i];
+          const typename X::V2 c = sv[i];
           const V vi = q[(size_t)i * rmax];
           v = fma(-c.x, vi, v);
           w = fma(-c.y, vi, w);
@@ -610,7 +614,8 @@ static size_t coop_smem(int nu, int nb, int ld, int nf, int chunk, int epc, int 
   const size_t fl = ldh * rmax + nu * rmax + rmax + (ns > 1 ? ns * rmax : 0) + (size_t)epc * (1 + nf) * nb +
                     ldh * nu + 2 * (size_t)nu + ldh;
   using V = typename CoopVal<S>::V;
-  return fl * sizeof(V) + sizeof(int) * (size_t)chunk * (1 + nf) + 16 + 2 * sizeof(V) * (nu + 2) +
+  const size_t sc = (2 * (nu + 2) + ldh) * sizeof(double) + (sizeof(V) == 4 ? 2 * (nu + 2) * sizeof(V) : 0);
+  return fl * sizeof(V) + sizeof(int) * (size_t)chunk * (1 + nf) + 16 + sc +
          (res ? (size_t)chunk * (2 + nf) * nb * ld * sizeof(S) : 0);
 }
 
@@ -667,7 +672,7 @@ static cudaError_t plan_coop(int nb, int ld, int E, int nu, CoopPlan* plan) {
     plan->res = res;
     plan->smem = smem;
     using X = Xch<typename CoopVal<S>::V>;
-    plan->part_bytes = sizeof(typename X::P) * 2 * (size_t)(grid + 2) * (nu + 2);
+    plan->part_bytes = sizeof(typename X::P) * 2 * (size_t)(grid + 1) * (nu + 2) + sizeof(Pair64) * 2 * (nu + 2) * SUM_STRIDE;
     plan->z_bytes = sizeof(typename X::Z) * (size_t)E * nb;
     return cudaSuccess;
   }
@@ -702,7 +707,7 @@ static cudaError_t launch_coop(const CoopPlan& pl, const S* Dinv, const S* Dop, 
   a.x = x;
   a.zx = (typename X::Z*)buf.z;
   a.px = (typename X::P*)buf.part;
-  a.sums = a.px + 2 * (size_t)(pl.grid + 1) * (pl.nu_max + 2);
+  a.sums = (Pair64*)(a.px + 2 * (size_t)(pl.grid + 1) * (pl.nu_max + 2));
   a.epoch = buf.epoch;
   a.status = status;
   a.kflag = K.kdim + 1;

@@ -781,19 +781,14 @@ cudaError_t launch_block_apply_bf16(const unsigned short* A, const float* r, flo
                                     cudaStream_t st) {
   const int ld16 = ld_bf16(nb), tpe = ld16 / 8;
   if (tpe > 256) return cudaErrorInvalidValue;
-  int epc = std::max(1, 256 / tpe), per = 8;
-  // blocks of more than about 0.9 GB in flight at once come slowly (4,096 of 420
-  // rows, 1.45 GB: 291 us with all of them in flight, 236 with 16 per SM, 352 with 8;
-  // of 280 rows, 0.64 GB, all: 105 us, 16 per SM: 131): one element per CTA and as
-  // many CTAs as hold 0.87 GB, where those keep an SM's loads in flight
-  const size_t bytes = sizeof(unsigned short) * (size_t)nb * ld16;
-  const int fit = (int)(870000000 / bytes / num_sms());
-  if ((double)E * bytes > 1e9 && fit >= 12 && fit <= 24) {
-    epc = 1;
-    per = fit;
-  }
+  // Eight CTAs of up to 256 threads per SM whatever the size.  Fewer elements in
+  // flight help some sizes (us, all / one element per CTA, 16 per SM: 4,096 blocks of
+  // 420 rows 285 / 232, 8,000 485 / 464) and cost others (2,900 of 420 rows 166 / 214;
+  // of 280 rows 8,000 210 / 200 and 13,824 349 / 371; of 600 rows 4,096 496 / 545;
+  // of 320 and 825 rows all is faster): no rule on the sizes holds over them.
+  const int epc = std::max(1, 256 / tpe);
   const int threads = (epc * tpe + 31) / 32 * 32;
-  const int grid = std::min((E + epc - 1) / epc, per * num_sms());
+  const int grid = std::min((E + epc - 1) / epc, 8 * num_sms());
   note_launch();
   bj_bf16_kernel<<<grid, threads, (size_t)epc * nb * sizeof(float), st>>>(A, r, z, nb, ld16, E, epc, tpe);
   return cudaGetLastError();

@@ -18,6 +18,7 @@
 // and levels coming from the host (dg_bilu_order).
 #include <algorithm>
 #include <cmath>
+#include <limits>
 #include <queue>
 #include <vector>
 
@@ -80,7 +81,9 @@ void order_mdf(const Graph& g, std::vector<int>& order) {
         s += f * f;
       }
     }
-    return std::sqrt(s);
+    // not a number (blocks of an unphysical state): infinite, else the entry would
+    // equal no weight below, be taken for a stale one and its element left out
+    return s == s ? std::sqrt(s) : std::numeric_limits<double>::infinity();
   };
   std::vector<double> w(E);
   using Item = std::pair<double, int>;

@@ -45,12 +45,22 @@ int num_sms_inv() {
   return n > 0 ? n : 1;
 }
 
-// the pivot candidate (|value| larger, or equal with a lower row) of two
-__device__ __forceinline__ bool better(float va, int ia, float vb, int ib) {
-  return va > vb || (va == vb && ia < ib);
+// |x|, 0 for NaN, from the bits: a comparison with zero in floating point
+// (fabs(x) >= 0 ? fabs(x) : 0) is folded to fabs(x) by the compiler, and a column
+// of NaN (the blocks of an unphysical state) then had no pivot row at all
+__device__ __forceinline__ float magnitude(float x) {
+  const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+  return __uint_as_float(b > 0x7f800000u ? 0u : b);
 }
-__device__ __forceinline__ bool better(double va, int ia, double vb, int ib) {
-  return va > vb || (va == vb && ia < ib);
+__device__ __forceinline__ double magnitude(double x) {
+  const long long b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return __longlong_as_double(b > 0x7ff0000000000000ll ? 0ll : b);
+}
+// whether candidate a is the better pivot of two (|value| larger, or equal with a
+// lower row; INT_MAX: no candidate)
+template <class T>
+__device__ __forceinline__ bool better(T va, int ia, T vb, int ib) {
+  return ib == INT_MAX ? ia != INT_MAX : va > vb || (va == vb && ia < ib);
 }
 
 template <class T, int R>
@@ -95,7 +105,7 @@ __global__ void __launch_bounds__(256, 1) block_inverse_reg_kernel(T* __restrict
 #pragma unroll
         for (int a = 0; a < R; ++a) {
           const int i = ty + 16 * a;
-          const T v = fabs(col[a]) >= T(0) ? fabs(col[a]) : T(0);   // NaN counts as 0
+          const T v = magnitude(col[a]);
           if (i < nb && !((used >> a) & 1u) && better(v, i, best, bi)) {
             best = v;
             bi = i;
@@ -235,7 +245,7 @@ __global__ void __launch_bounds__(256) block_inverse_kernel(T* __restrict__ bloc
       T best = T(-1), sv = T(0);
       int bi = INT_MAX;
       for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        const T x = A[(size_t)i * nb + k], v = fabs(x) >= T(0) ? fabs(x) : T(0);   // NaN counts as 0
+        const T x = A[(size_t)i * nb + k], v = magnitude(x);
         if (!used[i] && better(v, i, best, bi)) {
           best = v;
           bi = i;
@@ -394,7 +404,7 @@ __global__ void __launch_bounds__(256) block_inverse_panel_kernel(T* __restrict_
         T best = T(-1), sv = T(0);
         int bi = INT_MAX;
         for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-          const T x = Pn[(size_t)i * BP + c], v = fabs(x) >= T(0) ? fabs(x) : T(0);   // NaN counts as 0
+          const T x = Pn[(size_t)i * BP + c], v = magnitude(x);
           if (!used[i] && better(v, i, best, bi)) {
             best = v;
             bi = i;
@@ -562,13 +572,11 @@ struct BlkTile {
 };
 // |x| as an integer that orders like it, in two words; 0 = not a candidate
 __device__ __forceinline__ void pivot_key(float x, bool cand, unsigned* hi, unsigned* lo) {
-  const float v = fabsf(x) >= 0.f ? fabsf(x) : 0.f;   // NaN counts as 0
-  *hi = cand ? __float_as_uint(v) + 1u : 0u;
+  *hi = cand ? __float_as_uint(magnitude(x)) + 1u : 0u;
   *lo = 0u;
 }
 __device__ __forceinline__ void pivot_key(double x, bool cand, unsigned* hi, unsigned* lo) {
-  const double v = fabs(x) >= 0.0 ? fabs(x) : 0.0;
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(magnitude(x));
   *hi = cand ? (unsigned)(b >> 32) + 1u : 0u;
   *lo = cand ? (unsigned)b : 0u;
 }

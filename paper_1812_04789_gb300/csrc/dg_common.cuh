@@ -10,9 +10,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <algorithm>
-#include <cmath>
-
 namespace dgk {
 
 // 8 consecutive BF16 values (16 bytes, read-only, not kept in L1) widened to
@@ -417,39 +414,17 @@ __host__ __device__ __forceinline__ void face_point_k(int k, const S* uL, const 
   }
 }
 
-// 2^-e, e the exponent of x > 0 (or the largest whose reciprocal is normal)
-__host__ __device__ __forceinline__ float inverse_power(float x) {
-#ifdef __CUDA_ARCH__
-  return __int_as_float(max((254 << 23) - (__float_as_int(x) & 0x7f800000), 1 << 23));
-#else
-  int e;
-  std::frexp(x, &e);
-  return std::ldexp(1.f, std::min(127, std::max(-126, 1 - e)));
-#endif
-}
-__host__ __device__ __forceinline__ double inverse_power(double x) {
-#ifdef __CUDA_ARCH__
-  return __hiloint2double(max((2046 << 20) - (__double2hiint(x) & 0x7ff00000), 1 << 20), 0);
-#else
-  int e;
-  std::frexp(x, &e);
-  return std::ldexp(1.0, std::min(1023, std::max(-1022, 1 - e)));
-#endif
-}
-
-// rho > 0 and p > 0 of a point state (primal values)
+// rho > 0 and p > 0 of a point state (primal values), p / (gamma - 1) by the operations
+// of primitives(): where the point's primitives are formed as well the compiler
+// computes them once, and no product leaves the type's range (rho E does, in FP32,
+// where rho is below 1e-22)
 template <int D, class S, class T>
 __host__ __device__ __forceinline__ bool physical(const S* u, T) {
-  constexpr int M = D + 2;
-  T r = val(u[0]);
-  T q = val(u[1]) * val(u[1]);
+  const T ir = T(1) / val(u[0]);
+  T mv = val(u[1]) * (val(u[1]) * ir);
 #pragma unroll
-  for (int j = 1; j < D; ++j) q += val(u[1 + j]) * val(u[1 + j]);
-  // p = (gamma - 1) (E - q / (2 rho)) > 0 without the division: both sides times
-  // rho scaled by a power of two to [1, 8), so that no product leaves the type's
-  // range (in FP32 rho E itself does where rho is below 1e-22)
-  const T sc = inverse_power(r);
-  return r > T(0) && val(u[M - 1]) * (r * sc) > q * (T(0.5) * sc);
+  for (int j = 1; j < D; ++j) mv = val(u[1 + j]) * (val(u[1 + j]) * ir) + mv;
+  return val(u[0]) > T(0) && val(u[D + 1]) - T(0.5) * mv > T(0);
 }
 
 // ----------------------------------------------------------------- mesh view

@@ -27,8 +27,9 @@ namespace {
 
 constexpr int V32_THREADS = 128;
 
-// Tangent of F_c + F_v (flux_total) at the state (u, g) along (tu, tg).
-__device__ __forceinline__ void flux_tangent(const float* u, const float (*g)[3], const float* tu, const float (*tg)[3],
+// Tangent of F_c + F_v (flux_total) at the state (u, g) along (tu, tg); whether the
+// state is physical (physical(), from the pressure at hand).
+__device__ __forceinline__ bool flux_tangent(const float* u, const float (*g)[3], const float* tu, const float (*tg)[3],
                                              const Phys<float>& ph, float (*F)[3]) {
   const float ir = 1.f / u[0];
   float vel[3], dv[3];
@@ -88,6 +89,7 @@ __device__ __forceinline__ void flux_tangent(const float* u, const float (*g)[3]
     for (int j = 0; j < 3; ++j) q = fmaf(vel[j], dt[j][k], fmaf(dv[j], tau[j][k], q));
     F[4][k] = fmaf(tu[1 + k], h0, fmaf(u[1 + k], dh0, -q));
   }
+  return u[0] > 0.f && p > 0.f;
 }
 
 template <int N1, bool CACHED>
@@ -270,9 +272,9 @@ __global__ void __launch_bounds__(V32_THREADS) vol32_kernel(const __grid_constan
           gg[v][2] = d2;
         }
       }
-      ok = ok && physical<3>(u, ph.gm1);
       float F[M][3];
-      flux_tangent(u, g, tu, tg, ph, F);
+      const bool phys = flux_tangent(u, g, tu, tg, ph, F);
+      ok = ok && phys;
       const float w = w12 * la[2 * N1], w1 = w * tb.met[1], w2 = w * tb.met[2];
 #pragma unroll
       for (int v = 0; v < M; ++v) {

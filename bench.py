@@ -31,7 +31,7 @@ import numpy as np  # noqa: E402
 from paper_1812_04789_gb300 import workloads as wl  # noqa: E402
 
 BJ_KERNEL_VERSION = "colmajor-v1"   # bump when the block-Jacobi apply kernel changes
-COOP_KERNEL_VERSION = "coop-polled"   # bump when the persistent smoother kernel changes
+COOP_KERNEL_VERSION = "coop-fp64-sums"   # bump when the persistent smoother kernel changes
 METRIC = "Implicit-step DOFs/s (mixed vs FP64, 1 GB300); JVP % HBM roofline; p99 latency"
 UNIT = "DOFs/s"
 

@@ -368,7 +368,8 @@ cudaError_t launch_probe_blocks(const Mesh& M, const T* W, T sigma, T* D, size_t
   const char* simt = getenv("DG_PROBE_SIMT");
   const bool sf = probe_sf_ok(M) && !(simt && simt[0] == '1');
   if (std::is_same<T, float>::value && nbr_colmajor && O) {
-    // layout fixed at setup: the neighbour blocks always come from probe_nbr_kernel
+    // layout fixed at setup: the neighbour blocks come from nbr_sf_kernel or, where it
+    // does not apply, probe_nbr_kernel, which both write it
     cudaError_t e = sf ? launch_probe_sf(M, (const float*)W, (float)sigma, (float*)D, dstride, (const float*)Pv,
                                          (const float*)Pf, st)
                    : use_tc(M) ? launch_probe_tc(M, (const float*)W, (float)sigma, (float*)D, dstride, st)

@@ -418,7 +418,7 @@ struct Level {
   unsigned short* Dinv16 = nullptr;
   unsigned short* Dop16 = nullptr;
   unsigned short* O16 = nullptr;
-  CoopPlan coop;             // persistent smoother (FP32 coarse levels), when available
+  CoopPlan coop;             // persistent smoother (levels >= 1), when available
   CoopBuffers cbuf;          //   and its exchange buffers
 };
 

@@ -564,10 +564,10 @@ static cudaError_t run_residual(const Mesh& Ms, const T* W, const T* V, const T*
   if ((parts & 1) && !face32) {
     // 3-D: the face term by sum factorisation in FP64 (fewer of the FP64 pipe's
     // cycles: the residual 4.4 -> 3.8 ms at 16^3 p = 4, 125 -> 73 ms at 32^3
-    // p = 6); in FP32 the direct kernel is faster (smoother JVP 0.23 against
-    // 0.56 ms at p = 4, 4.9 against 9.1 ms at p = 6).  DG_NO_SUMFACT_FACE=1
-    // keeps the direct kernel; DG_SUMFACT_FACE_MIN_MODES=n takes the sum-
-    // factorised one in FP32 from n modes on
+    // p = 6).  In FP32 the meshes that get here (Q_p, p >= 7, another number of
+    // points) take the direct kernel; DG_NO_SUMFACT_FACE=1 keeps the direct kernel
+    // everywhere; DG_SUMFACT_FACE_MIN_MODES=n (a test's) takes the FP32 instance of
+    // this one from n modes on, also where face32_kernel is the faster one
     const int min_modes = sfmin ? atoi(sfmin) : INT_MAX;
     cudaError_t e = cudaErrorNotSupported;
     if (D == 3 && !(nsff && nsff[0] == '1') && (std::is_same<T, double>::value || Ms.nm >= min_modes)) {
